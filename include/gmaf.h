@@ -127,8 +127,11 @@ typedef struct {
                                   static schedule; 3000000 + 10000 RPW + 1000 NS + TB for
                                   the block-marched phase B with TMA tiles.  Chosen per
                                   problem shape by the autotuner on the first solve of
-                                  that shape */
-    int32_t tasks;             /* strip x row-block x condition tasks per PCG phase       */
+                                  that shape.  50000000 + 1000 VEC + 10 RR: the resident
+                                  solve (one launch, RR rows a thread), taken wherever
+                                  the system fits on the SMs */
+    int32_t tasks;             /* strip x row-block x condition tasks per PCG phase
+                                  (resident solve: blocks)                              */
     int32_t iterations_sum;    /* PCG iterations summed over the conditions: n_cond x
                                   iterations under the synchronized criterion, the sum of
                                   the per-condition counts under the asynchronized one
@@ -228,7 +231,8 @@ int gmaf_picard_step_simplified(gmaf_ctx *ctx, const gmaf_grid *grid, const gmaf
 
 /* Per-phase kernel timing (tracing).  When enabled (on != 0), the PCG loop of
  * later solves is driven in host chunks instead of the graph WHILE node, with a
- * CUDA event pair around every phase launch on the context's stream; results
+ * CUDA event pair around every phase launch on the context's stream (a resident
+ * solve, which is one launch, times its phases by the GPU's clock); results
  * are bitwise the same.  gmaf_phase_timing returns, per kernel kind
  * [0] phase A (u update + stencil), [1] phase B (residual update + ASSOR-II),
  * [2] initial preconditioner pass, [3] FP64 residual, the summed event time in

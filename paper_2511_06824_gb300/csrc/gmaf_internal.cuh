@@ -112,6 +112,8 @@ enum BufId {
     B_CHUNK, B_CHUNKCTR,
     // boundary rows' Dirichlet term of the FP32 diagonal (phase A with the rebuilt diagonal)
     B_DBND32,
+    // resident PCG: exchanged rows, words of the exchanged sums, phase times
+    B_RES, B_RESWORDS, B_RESTIME,
     B_COUNT
 };
 
@@ -162,6 +164,8 @@ struct gmaf_ctx {
     double inner_floor;            // smallest relative residual asked of an inner FP32 solve
     int mixed_restart;             // restart the inner FP32 PCG at each refinement (else continue it)
     double reliable_delta;         // continued recurrence: residual reduction between two refinements
+    unsigned res_epoch;            // resident PCG: last exchange number used in B_RES,
+    size_t res_ring;               //   words of B_RESWORDS used since they were cleared
     int loop_guard;                // GMAF_LOOP_GUARD: fixed loop-guard limit (0: max_iter + 4)
 };
 

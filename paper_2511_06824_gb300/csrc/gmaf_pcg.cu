@@ -35,6 +35,7 @@
 #include "gmaf_mphase_kernels.cuh"
 #include "gmaf_tma.h"
 #include "gmaf_drec.h"
+#include "gmaf_resident.h"
 
 namespace gmaf {
 
@@ -863,6 +864,222 @@ static int solve_async64(gmaf_ctx *ctx, int nth, int nz, int K, const int *cslot
     return status;
 }
 
+// ---------------------------------------------------------------- resident solve
+//
+// Systems whose rows fit on the SMs are solved in one cooperative launch
+// (gmaf_resident.cuh).  GMAF_VARIANT with the id of a phase kernel turns it off.
+
+constexpr size_t kResRing = 64 * 1024;
+
+template <typename T>
+struct ResRun {
+    bool on = false;
+    ResPlan pl{};
+    ResParams<T> q{};
+};
+
+// The plan and its buffers; off (phase kernels) when the system does not fit, when a
+// phase kernel is asked for, or when the budget has no room for the exchanged words.
+template <typename T>
+static void res_setup(gmaf_ctx *ctx, ResRun<T> &rr, int nth, int nz, int K, bool vec)
+{
+    rr.on = false;
+    if (ctx->force_variant >= 0 && ctx->force_variant / 10000000 != kResVariant / 10000000) return;
+    if (!res_plan<T>(nth, nz, K, vec, ctx->num_sms, &rr.pl)) return;
+    int coop = 0;
+    if (cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, ctx->device) != cudaSuccess || !coop) {
+        cudaGetLastError();
+        return;
+    }
+    if (ensure(ctx, B_RESWORDS, kResRing) != GMAF_OK) return;
+    if (ensure(ctx, B_RES, rr.pl.halo_bytes) != GMAF_OK) return;
+    if (ctx->phase_timing && ensure(ctx, B_RESTIME, 64) != GMAF_OK) return;
+    ResParams<T> &q = rr.q;
+    q.nth = nth;
+    q.nz = nz;
+    q.n = (long long)nth * nz;
+    q.groups = 1;
+    q.mask = ~0ull;
+    q.halo = (unsigned long long *)ctx->buf[B_RES];
+    res_fill<T>(rr.pl, &q);
+    rr.on = true;
+}
+
+// One launch; max_iter - start iterations at most.  *off: the blocks cannot all be
+// resident here, nothing was launched.
+template <typename T>
+static int res_run(gmaf_ctx *ctx, ResRun<T> &rr, long long most_iterations, bool *off)
+{
+    cudaStream_t s = ctx->stream;
+    ResParams<T> &q = rr.q;
+    // two exchanges an iteration and two at the start; the words are cleared before the
+    // numbers run out
+    const unsigned long long need = 2ull * (unsigned long long)std::max(0LL, most_iterations) + 4ull;
+    if ((unsigned long long)ctx->res_epoch + need > 0xffffffffull) {
+        GMAF_CUDA(cudaMemsetAsync(ctx->buf[B_RES], 0, ctx->bytes[B_RES], s));
+        ctx->res_epoch = 0;
+    }
+    q.epoch = ctx->res_epoch;
+    // the words of the sums start from zero: fresh ones for each run, from a ring that is
+    // cleared when it is used up (buffers are cleared when they are allocated)
+    const size_t room = (size_t)q.groups * kResGroupWords * 8;
+    if (ctx->res_ring + room > kResRing) {
+        GMAF_CUDA(cudaMemsetAsync(ctx->buf[B_RESWORDS], 0, kResRing, s));
+        ctx->res_ring = 0;
+    }
+    q.words = (unsigned long long *)((char *)ctx->buf[B_RESWORDS] + ctx->res_ring);
+    ctx->res_ring += room;
+    ctx->res_epoch = (unsigned)std::min<unsigned long long>(0xffffffffull, ctx->res_epoch + need);
+    q.times = nullptr;
+    if (ctx->phase_timing) {
+        q.times = (unsigned long long *)ctx->buf[B_RESTIME];
+        GMAF_CUDA(cudaMemsetAsync(q.times, 0, 64, s));
+    }
+    *off = false;
+    const cudaError_t e = res_launch<T>(rr.pl, q, s);
+    if (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorNotSupported) {
+        cudaGetLastError();
+        *off = true;
+        return GMAF_OK;
+    }
+    GMAF_CUDA(e);
+    if (q.times) {
+        unsigned long long t[5];
+        GMAF_CUDA(cudaMemcpyAsync(t, q.times, sizeof t, cudaMemcpyDeviceToHost, s));
+        GMAF_CUDA(cudaStreamSynchronize(s));
+        for (int k = 0; k < 3; ++k) ctx->phase_ms[k] += 1e-6 * (double)t[k];
+        ctx->phase_count[0] += (long long)t[3];
+        ctx->phase_count[1] += (long long)t[4];
+        ctx->phase_count[2] += 1;
+    }
+    return GMAF_OK;
+}
+
+// FP64, either criterion: the joint system is one group of blocks, under the
+// asynchronized criterion each condition is one (its own scalars, its own end).
+// After a run each group gets the FP64 true-residual check, and once, if that
+// fails, a restart from the true residual.
+static int solve_resident64(gmaf_ctx *ctx, ResRun<double> &rr, int K, const int *cslot_host,
+                            const double *S, double *p, const gmaf_solver_opts *opts,
+                            gmaf_solve_info *info, bool *off)
+{
+    cudaStream_t s = ctx->stream;
+    ResParams<double> &q = rr.q;
+    const bool async = opts->criterion == 1;
+    const int G = async ? K : 1;
+    const long long n = q.n;
+    Scalars *scal = (Scalars *)ctx->buf[B_SCAL];
+    Scalars *gsc = async ? scal + 3 : scal;                   // [G] the runs
+    Scalars *rsc = gsc + G;                                   // [G] their true residuals
+    q.groups = G;
+    q.sc = gsc;
+    q.mode = kResFresh;
+    q.keep_iter = 0;
+    // descriptors of the residuals: condition k, or the joint system
+    const size_t o_slot = align256((size_t)kMaxCond * sizeof(ResidDesc));
+    GMAF_TRY(ensure(ctx, B_ASYNC, o_slot + 256));
+    ResidDesc *d_rd = (ResidDesc *)ctx->buf[B_ASYNC];
+    const int gs = stream_grid(async ? n : n * K, ctx->num_sms);
+    GMAF_TRY(ensure(ctx, B_PART, (size_t)2 * gs * G * sizeof(double)));
+    std::vector<ResidDesc> rd(G);
+    for (int k = 0; k < G; ++k) {
+        const long long o = (long long)k * n, c = async ? (long long)cslot_host[k] * n : 0;
+        rd[k] = ResidDesc{};
+        rd[k].nth = q.nth;
+        rd[k].nz = q.nz;
+        rd[k].K = async ? 1 : K;
+        rd[k].n = n;
+        rd[k].D = q.D + c;
+        rd[k].aE = q.aE + c;
+        rd[k].aN = q.aN + c;
+        rd[k].cslot = async ? (const int *)((char *)ctx->buf[B_ASYNC] + o_slot) : q.cslot;
+        rd[k].S = S + o;
+        rd[k].p = p + o;
+        rd[k].sc = rsc + k;
+        rd[k].partials = (double *)ctx->buf[B_PART] + (size_t)2 * gs * k;
+    }
+    GMAF_CUDA(cudaMemsetAsync(gsc, 0, (size_t)2 * G * sizeof(Scalars), s));
+    if (async) GMAF_CUDA(cudaMemsetAsync((char *)ctx->buf[B_ASYNC] + o_slot, 0, sizeof(int), s));
+    std::vector<Scalars> h(2 * G);
+    std::vector<int> restarted(G, 0), ok(G, 0);
+    std::vector<double> true_rel(G, 0.0);
+    unsigned long long ran = G == 64 ? ~0ull : (1ull << G) - 1;
+    for (int pass = 0; ran; ++pass) {
+        q.mask = ran;
+        GMAF_TRY(res_run<double>(ctx, rr, opts->max_iter, off));
+        if (*off) return GMAF_OK;
+        auto residuals = [&]() -> int {
+            // (pageable source: consumed when the call returns)
+            GMAF_CUDA(cudaMemcpyAsync(d_rd, rd.data(), (size_t)G * sizeof(ResidDesc),
+                                      cudaMemcpyHostToDevice, s));
+            PhaseClock clk{ctx};
+            clk.begin(s);
+            k_resid64<<<dim3(gs, G), kThreads, 0, s>>>(d_rd);
+            clk.end(s, 3);
+            GMAF_CUDA(cudaGetLastError());
+            GMAF_CUDA(cudaMemcpyAsync(h.data(), gsc, (size_t)2 * G * sizeof(Scalars),
+                                      cudaMemcpyDeviceToHost, s));
+            GMAF_CUDA(cudaStreamSynchronize(s));
+            clk.collect(0);
+            return GMAF_OK;
+        };
+        GMAF_TRY(residuals());
+        unsigned long long again = 0;
+        for (int k = 0; k < G; ++k) {
+            if (!((ran >> k) & 1ull)) continue;
+            true_rel[k] = h[G + k].true_rel;
+            if (h[k].zero_rhs) {
+                GMAF_CUDA(cudaMemsetAsync(p + (long long)k * n, 0,
+                                          (size_t)(async ? n : n * K) * sizeof(double), s));
+                true_rel[k] = 0.0;
+            }
+            if (h[k].status != 0 || h[G + k].status != 0) continue;
+            if ((h[k].converged || h[k].zero_rhs) && true_rel[k] <= 10.0 * opts->eps) {
+                ok[k] = 1;
+                continue;
+            }
+            if (restarted[k] || h[k].iter >= opts->max_iter) continue;
+            restarted[k] = 1;
+            again |= 1ull << k;
+        }
+        ran = again;
+        if (ran) {
+            // restart those from S - A p
+            GMAF_TRY(ensure(ctx, B_R0, (size_t)n * K * sizeof(double)));
+            for (int k = 0; k < G; ++k) rd[k].r = (double *)ctx->buf[B_R0] + (long long)k * n;
+            GMAF_TRY(residuals());
+            q.r_in = (const double *)ctx->buf[B_R0];
+            q.mode = kResRestart;
+            q.keep_iter = 1;
+        }
+    }
+    GMAF_CUDA(cudaStreamSynchronize(s));
+    gmaf_solve_info inf{};
+    int status = GMAF_OK;
+    for (int k = 0; k < G; ++k) {
+        inf.iterations = std::max(inf.iterations, h[k].iter);
+        inf.iterations_sum += h[k].iter;
+        inf.rel_residual = std::max(inf.rel_residual, h[k].rel);
+        inf.true_rel_residual = std::max(inf.true_rel_residual, true_rel[k]);
+        inf.restarts += restarted[k];
+        const int st = h[k].status != 0 ? h[k].status : h[G + k].status;
+        if (st != 0 && status == GMAF_OK) status = st;
+        if (!ok[k] && st == 0 && status == GMAF_OK) status = GMAF_NOT_CONVERGED;
+    }
+    if (!async) {
+        inf.iterations_sum = inf.iterations * K;
+        inf.rel_residual = h[0].rel;
+        inf.true_rel_residual = true_rel[0];
+    }
+    inf.status = status;
+    inf.outer_iterations = 1;
+    inf.kernel_variant = kResVariant + 1000 * rr.pl.vec + 10 * rr.pl.rr;
+    inf.tasks = rr.pl.grid;
+    inf.p_update_period = 1;
+    *info = inf;
+    return status;
+}
+
 int solve_joint_device(gmaf_ctx *ctx, int nth, int nz, int K, int nslots, const int *cslot_host,
                        const double *D, const double *aE, const double *aN, const double *S,
                        double *p, const gmaf_solver_opts *opts, gmaf_solve_info *info)
@@ -910,10 +1127,36 @@ int solve_joint_device(gmaf_ctx *ctx, int nth, int nz, int K, int nslots, const 
 
     if (opts->precision == 0) {
         GMAF_TRY(ensure(ctx, B_INVD, (size_t)m * sizeof(double)));
-        const int bufs[] = {B_R0, B_R1, B_U0, B_U1, B_Z, B_V};
-        for (int b : bufs) GMAF_TRY(ensure(ctx, b, (size_t)N * sizeof(double)));
         diag_inverse64(opts, D, aE, aN, nth, nz, m, (double *)ctx->buf[B_INVD], ctx->num_sms, s);
         GMAF_CUDA(cudaGetLastError());
+        ResRun<double> rr;
+        const void *ptrs[] = {D, aE, aN, S, p};
+        bool vec = nth % 2 == 0;
+        for (const void *x : ptrs) vec = vec && aligned16(x);
+        res_setup<double>(ctx, rr, nth, nz, K, vec);
+        if (rr.on) {
+            ResParams<double> &q = rr.q;
+            q.precond = kernel_precond(opts);
+            q.zero_init = opts->zero_init;
+            q.max_iter = opts->max_iter;
+            q.guard_limit = ctx->loop_guard;
+            q.eps = opts->eps;
+            q.cscale = 0.0;
+            q.D = D;
+            q.invD = (const double *)ctx->buf[B_INVD];
+            q.aE = aE;
+            q.aN = aN;
+            q.cslot = cslot;
+            q.b = S;
+            q.r_in = nullptr;
+            q.p = p;
+            q.u = nullptr;
+            bool off = false;
+            const int st = solve_resident64(ctx, rr, K, cslot_host, S, p, opts, info, &off);
+            if (!off) return st;
+        }
+        const int bufs[] = {B_R0, B_R1, B_U0, B_U1, B_Z, B_V};
+        for (int b : bufs) GMAF_TRY(ensure(ctx, b, (size_t)N * sizeof(double)));
         if (opts->criterion == 1) {
             const bool vec = (nth % 2) == 0;     // 16-byte rows of doubles in every condition
             const double *iv = (const double *)ctx->buf[B_INVD];
@@ -1007,8 +1250,16 @@ int solve_joint_device(gmaf_ctx *ctx, int nth, int nz, int K, int nslots, const 
     GMAF_TRY(ensure(ctx, B_INVD32, (size_t)m * sizeof(float)));
     GMAF_TRY(ensure(ctx, B_AE32, (size_t)m * sizeof(float)));
     GMAF_TRY(ensure(ctx, B_AN32, (size_t)m * sizeof(float)));
-    const int fbufs[] = {B_B32, B_X32, B_R032, B_R132, B_U032, B_U132, B_Z32, B_V32};
-    for (int b : fbufs) GMAF_TRY(ensure(ctx, b, (size_t)N * sizeof(float)));
+    for (int b : {B_B32, B_X32, B_U032}) GMAF_TRY(ensure(ctx, b, (size_t)N * sizeof(float)));
+    ResRun<float> rr;
+    res_setup<float>(ctx, rr, nth, nz, K, nth % 4 == 0);
+    // the fields of the phase kernels
+    auto phase_buffers = [&]() -> int {
+        for (int b : {B_R032, B_R132, B_U132, B_Z32, B_V32})
+            GMAF_TRY(ensure(ctx, b, (size_t)N * sizeof(float)));
+        return GMAF_OK;
+    };
+    if (!rr.on) GMAF_TRY(phase_buffers());
     GMAF_TRY(ensure(ctx, B_R64, (size_t)N * sizeof(double)));
     k_to_f32<<<stream_grid(m, ctx->num_sms), kThreads, 0, s>>>(
         D, aE, aN, (float *)ctx->buf[B_D32], (float *)ctx->buf[B_INVD32], (float *)ctx->buf[B_AE32],
@@ -1034,22 +1285,40 @@ int solve_joint_device(gmaf_ctx *ctx, int nth, int nz, int K, int nslots, const 
     h.cslot = cslot;
     h.b = (const float *)ctx->buf[B_B32];
     h.p = (float *)ctx->buf[B_X32];
-    h.z = (float *)ctx->buf[B_Z32];
-    h.v = (float *)ctx->buf[B_V32];
-    h.u[0] = (float *)ctx->buf[B_U032];
-    h.u[1] = (float *)ctx->buf[B_U132];
-    h.r[0] = (float *)ctx->buf[B_R032];
-    h.r[1] = (float *)ctx->buf[B_R132];
     h.omega = (float)opts->omega;
     h.sc = dsc;
     h.nslots = nslots;
-    if (nth % 4 == 0) {
+    if (!rr.on && nth % 4 == 0) {
         // the boundary term of the diagonal for the phase A variant that rebuilds it
         GMAF_TRY(ensure(ctx, B_DBND32, (size_t)nslots * 2 * nth * sizeof(float)));
         GMAF_TRY(launch_dbnd32(h.D, h.aE, h.aN, (float *)ctx->buf[B_DBND32], nth, nz, nslots,
                                ctx->num_sms, s));
         h.dbnd = (const float *)ctx->buf[B_DBND32];
         run.drec_ready = true;
+    }
+    auto phase_fields = [&]() {
+        h.z = (float *)ctx->buf[B_Z32];
+        h.v = (float *)ctx->buf[B_V32];
+        h.u[0] = (float *)ctx->buf[B_U032];
+        h.u[1] = (float *)ctx->buf[B_U132];
+        h.r[0] = (float *)ctx->buf[B_R032];
+        h.r[1] = (float *)ctx->buf[B_R132];
+    };
+    if (!rr.on) phase_fields();
+    if (rr.on) {
+        ResParams<float> &q = rr.q;
+        q.precond = kernel_precond(opts);
+        q.zero_init = 1;
+        q.D = h.D;
+        q.invD = h.invD;
+        q.aE = h.aE;
+        q.aN = h.aN;
+        q.cslot = cslot;
+        q.b = h.b;
+        q.r_in = nullptr;
+        q.p = h.p;
+        q.u = (float *)ctx->buf[B_U032];
+        q.sc = dsc;
     }
     // The first outer residual and the inner right-hand side are formed before the
     // kernel set is chosen, so that the autotuner times iterations on real data.
@@ -1100,7 +1369,7 @@ int solve_joint_device(gmaf_ctx *ctx, int nth, int nz, int K, int nslots, const 
         k_make_b32<<<gs, kThreads, 0, s>>>((const double *)ctx->buf[B_R64], (float *)ctx->buf[B_B32],
                                            N, dsc_outer);
         GMAF_CUDA(cudaGetLastError());
-        if (!tuned) {
+        if (!tuned && !rr.on) {
             GMAF_TRY(setup_run<float>(ctx, run, (PcgDesc<float> *)(dbase + 1024)));
             rd.partials = h.partials;
             GMAF_CUDA(cudaMemcpyAsync(d_rdesc, &rd, sizeof(ResidDesc), cudaMemcpyHostToDevice, s));
@@ -1119,8 +1388,28 @@ int solve_joint_device(gmaf_ctx *ctx, int nth, int nz, int K, int nslots, const 
         const int cap = std::max(1000, 4 * longest);
         h.max_iter = cont ? last_iter + std::min(left, cap) : left;
         h.guard_limit = ctx->loop_guard;
-        GMAF_TRY(prepare<float>(ctx, run, ctx->graph32));
-        GMAF_TRY(pcg_once<float>(ctx, run, ctx->graph32, cont, true, cont ? rnorm_prev / ho->rnorm : 0.0));
+        const double cscale = cont ? rnorm_prev / ho->rnorm : 0.0;
+        if (rr.on) {
+            ResParams<float> &q = rr.q;
+            q.mode = cont ? kResContinue : kResFresh;
+            q.keep_iter = cont ? 1 : 0;
+            q.max_iter = h.max_iter;
+            q.guard_limit = h.guard_limit;
+            q.eps = h.eps;
+            q.cscale = cscale;
+            bool off = false;
+            GMAF_TRY(res_run<float>(ctx, rr, cont ? h.max_iter - last_iter : h.max_iter, &off));
+            if (off) {
+                // the blocks cannot all be resident: the phase kernels from here on
+                rr.on = false;
+                GMAF_TRY(phase_buffers());
+                phase_fields();
+                continue;
+            }
+        } else {
+            GMAF_TRY(prepare<float>(ctx, run, ctx->graph32));
+            GMAF_TRY(pcg_once<float>(ctx, run, ctx->graph32, cont, true, cscale));
+        }
         rnorm_prev = ho->rnorm;
         k_update_p64<<<gs, kThreads, 0, s>>>(p, (const float *)ctx->buf[B_X32], N, dsc_outer);
         GMAF_CUDA(cudaGetLastError());
@@ -1140,8 +1429,8 @@ int solve_joint_device(gmaf_ctx *ctx, int nth, int nz, int K, int nslots, const 
     inf.iterations = total_inner;
     inf.iterations_sum = total_inner * K;
     inf.outer_iterations = outer;
-    inf.kernel_variant = run.ks.id;
-    inf.tasks = (int)run.h.ntiles;
+    inf.kernel_variant = rr.on ? kResVariant + 1000 * rr.pl.vec + 10 * rr.pl.rr : run.ks.id;
+    inf.tasks = rr.on ? rr.pl.grid : (int)run.h.ntiles;
     inf.p_update_period = std::max(1, run.ks.p_period);
     *info = inf;
     return inf.status;

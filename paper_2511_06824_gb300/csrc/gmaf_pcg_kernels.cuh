@@ -1105,9 +1105,10 @@ static __global__ void k_reset(Scalars *sc, int keep_iter)
 // ------------------------------------------------------------------ FP64 residual, conversions
 
 // r = S - A p (FP64), partial ||r||^2 and ||S||^2; last block sets true_rel and rnorm.
+// blockIdx.y: one of several systems, each with its own descriptor.
 static __global__ void __launch_bounds__(kThreads) k_resid64(const ResidDesc *__restrict__ dp)
 {
-    const ResidDesc &d = *dp;
+    const ResidDesc &d = dp[blockIdx.y];
     const int nth = d.nth, nz = d.nz;
     const long long n = d.n, N = n * d.K;
     double arr = 0.0, ass = 0.0;

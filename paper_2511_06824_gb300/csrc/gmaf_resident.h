@@ -1,0 +1,77 @@
+// Host-visible part of the resident PCG (gmaf_resident.cuh): the shape of a launch
+// and the launch itself, used by the joint solver (gmaf_pcg.cu) and the
+// allocation-free solve (gmaf_noalloc.cu).  Internal; not part of the ABI.
+#pragma once
+
+#include <cstddef>
+
+#include "gmaf_internal.cuh"
+
+namespace gmaf {
+
+constexpr int kResThreads = 512;        // most threads that own rows (one more warp exchanges)
+constexpr int kResMaxBlocks = 160;      // most blocks of a launch (they are counted in a byte)
+constexpr int kResGroupWords = 16;      // 8-byte words of a group of blocks for its sums
+constexpr int kResSegs = kResThreads / 32;   // segments of 32 threads in a row, at most
+constexpr int kResVariant = 50000000;   // gmaf_solve_info.kernel_variant: + 1000 VEC + 10 RR
+
+// Whether a run's r lives in shared memory: with over 64 bytes a thread the registers do
+// not hold r beside the product.
+__host__ __device__ constexpr bool res_r_shared(int rr, int vec, int size) { return rr * vec * size > 64; }
+
+enum ResMode {
+    kResFresh = 0,      // r = b - A p (p = 0 with zero_init)
+    kResRestart = 1,    // r handed in, p continued, the norm of b kept from the last run
+    kResContinue = 2    // r = b, p = 0, the recurrence continued with the direction in u
+};
+
+// Kernel parameters.  o_*: byte offsets in shared memory (-1: the array stays in
+// global memory).
+template <typename T>
+struct ResParams {
+    int nth, nz, bpc, groups;           // bpc blocks a condition; groups: 1 joint system or K
+    int threads, P, ncg, nrr, rows;
+    int precond, mode, zero_init, keep_iter, max_iter, guard_limit;
+    int o_rows, o_edge, o_x;
+    unsigned epoch;                     // exchanges of this run are epoch + 1, epoch + 2, ...
+    unsigned long long mask;            // groups that run
+    long long n;
+    const T *D, *invD, *aE, *aN;
+    const int *cslot;
+    const T *b, *r_in;
+    T *p, *u;                           // u: written at the end (null: not wanted)
+    Scalars *sc;                        // [groups]
+    double eps, cscale;
+    unsigned long long *words;          // [groups][kResGroupWords], zero at the start of the run
+    unsigned long long *halo;           // flagged rows, [blocks][4]
+    int halo_row;                       // 8-byte words of one flagged row
+    unsigned long long *times;          // ns in A, B and set-up, counts of A and B (added to; or null)
+};
+
+struct ResPlan {
+    const void *fn;
+    int grid, smem, vec, rr;
+    int bpc, threads, P, ncg, nrr, rows;
+    int o_rows, o_edge, o_x;
+    size_t halo_bytes;                  // flagged rows, zero before the first launch
+};
+
+// Whether (and how) a solve of K conditions on nth x nz fits on the SMs: vec_ok says
+// that rows can be read 16 bytes at a time.
+template <typename T>
+bool res_plan(int nth, int nz, int K, bool vec_ok, int num_sms, ResPlan *out);
+
+// Fills the plan's part of the parameters.
+template <typename T>
+void res_fill(const ResPlan &pl, ResParams<T> *q);
+
+// Kernel of a plan (compiled for T in a translation unit of its own).
+const void *res_kernel_f32(int vec, int rr, bool cs);
+const void *res_kernel_f64(int vec, int rr, bool cs);
+
+// Cooperative launch; cudaErrorCooperativeLaunchTooLarge when the blocks cannot all
+// be resident (a partitioned GPU): the caller then takes the phase kernels.
+template <typename T>
+cudaError_t res_launch(const ResPlan &pl, ResParams<T> &q, cudaStream_t s);
+
+}  // namespace gmaf

@@ -1,0 +1,153 @@
+"""The resident PCG (one cooperative launch a solve, vectors on the SMs) against the
+FP64 oracle and against the phase kernels, at the edges of its decomposition: one row
+a block and runs of 1, 2, 4 and 8 rows, a last run that is not full, rows of less
+than, exactly and more than a warp of threads, one and two columns a thread in FP64
+and one and four in FP32, arrays that are not 16-byte aligned, as many conditions as
+the library takes, and grids just beyond what it holds.
+
+Both run the same recurrence, so FP64 iteration counts agree to 2 and solutions to
+far less than the tolerance (1e-10; eps 1e-12 leaves 1e-11).  In mixed precision both
+end at a true FP64 residual below 1e-12, which leaves about 1e-11 as well."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2511_06824_gb300 import inputs
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+PHYS = inputs.phys_vector()
+RESIDENT = 50000000
+
+
+@pytest.fixture(scope="module")
+def g():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2511_06824_gb300 import build, gmaf
+    build.build()
+    gmaf.load()
+    return gmaf
+
+
+def system(nth, nz, K, seed, shift=0):
+    """Coefficients and sources on the device; shift: doubles by which every array misses
+    a 16-byte boundary."""
+    rng = np.random.default_rng(seed)
+    tex = inputs.dimple_texture(rng)
+    conds = [inputs.random_state(rng) for _ in range(K)]
+    st, *arrs = oracle.assemble_joint(nth, nz, PHYS, tex, conds)
+    assert st == 0
+    out = []
+    for a in arrs:
+        t = torch.zeros(a.size + shift, dtype=torch.float64, device="cuda")
+        t[shift:] = torch.from_numpy(np.ascontiguousarray(a).ravel()).cuda()
+        out.append(t[shift:])
+    return arrs, out
+
+
+def solve(g, monkeypatch, nth, nz, K, arrs, variant=None, start=None, budget=0, allow=False, **opts):
+    if variant is None:
+        monkeypatch.delenv("GMAF_VARIANT", raising=False)
+    else:
+        monkeypatch.setenv("GMAF_VARIANT", str(variant))
+    with g.Context(hbm_budget_bytes=budget) as c:
+        p = torch.full((K * nth * nz,), 5.0, dtype=torch.float64, device="cuda")
+        if start is not None:
+            p.copy_(start)
+            opts["zero_init"] = 0
+        st, it, rel = g.gmaf_solve_joint(c.handle, nth, nz, K, *arrs, p,
+                                         g.solver_opts(**{"eps": 1e-12, **opts}),
+                                         allow_not_converged=allow)
+        info = g.gmaf_last_solve_info(c.handle)
+    return p, it, rel, info
+
+
+def rel_l2(a, b):
+    return float(torch.linalg.norm(a - b) / torch.linalg.norm(b))
+
+
+# (n_theta, n_z, K, shift, precision): columns and rows a thread as the plan picks them
+@pytest.mark.parametrize("nth,nz,K,shift,precision", [
+    (3, 2, 1, 0, 0), (3, 2, 1, 0, 1), (4, 3, 2, 0, 0), (4, 3, 2, 0, 1),   # fewer columns than a warp
+    (64, 32, 1, 0, 0), (128, 17, 9, 0, 1),      # one row a block; rows of exactly a warp (FP32)
+    (132, 33, 9, 0, 1), (66, 40, 5, 0, 0),      # a second, nearly empty segment of a row
+    (130, 45, 9, 1, 0),                         # unaligned arrays: one column a thread
+    (255, 97, 3, 0, 0), (255, 97, 3, 0, 1),     # odd rows
+    (256, 131, 9, 0, 0), (512, 100, 9, 0, 1),   # runs of 2 rows, the last one not full
+    (512, 250, 9, 0, 0), (512, 250, 9, 0, 1),   # runs of 8 and 4 rows
+    (640, 200, 9, 0, 1),                        # runs of 8 rows in FP32
+    (40, 9, 64, 0, 0), (40, 9, 64, 0, 1),       # two blocks a condition
+    (511, 5, 64, 0, 0),                         # one column a thread, almost every thread
+])
+def test_resident_solve_matches_phase_kernels(g, monkeypatch, nth, nz, K, shift, precision):
+    _, arrs = system(nth, nz, K, nth + nz, shift)
+    p, it, rel, info = solve(g, monkeypatch, nth, nz, K, arrs, precision=precision)
+    assert info["kernel_variant"] // RESIDENT == 1
+    ref, itr, relr, infr = solve(g, monkeypatch, nth, nz, K, arrs, precision=precision,
+                                 variant=1001003 if precision == 0 else 1001004)
+    assert infr["kernel_variant"] // RESIDENT == 0
+    assert rel <= (1e-11 if precision == 0 else 1e-12)
+    assert abs(it - itr) <= (2 if precision == 0 else 2 + itr // 50)
+    assert rel_l2(p, ref) <= 1e-10
+    # bitwise the same again, and from the solution itself no iteration is left to do
+    p2, it2, _, _ = solve(g, monkeypatch, nth, nz, K, arrs, precision=precision)
+    assert it2 == it and torch.equal(p, p2)
+    p3, it3, _, _ = solve(g, monkeypatch, nth, nz, K, arrs, precision=precision, start=p, eps=1e-10)
+    assert it3 == 0 and torch.equal(p3, p)
+
+
+@pytest.mark.parametrize("nth,nz,K,precond,criterion", [
+    (130, 45, 9, 0, 0), (130, 45, 9, 2, 0), (131, 7, 3, 1, 1), (130, 45, 9, 0, 1), (66, 30, 20, 2, 1),
+])
+def test_resident_options_match_phase_kernels(g, monkeypatch, nth, nz, K, precond, criterion):
+    _, arrs = system(nth, nz, K, nth + K)
+    kw = dict(precond=precond, criterion=criterion)
+    p, it, rel, info = solve(g, monkeypatch, nth, nz, K, arrs, **kw)
+    ref, itr, _, infr = solve(g, monkeypatch, nth, nz, K, arrs, variant=1001003, **kw)
+    assert info["kernel_variant"] // RESIDENT == 1 and infr["kernel_variant"] // RESIDENT == 0
+    assert abs(it - itr) <= 2 and abs(info["iterations_sum"] - infr["iterations_sum"]) <= 2 * K
+    assert rel <= 1e-11 and rel_l2(p, ref) <= 1e-10
+    # a warm start from elsewhere, and a run stopped by its budget
+    start = ref * (1.0 + 1e-3)
+    a, ita, _, _ = solve(g, monkeypatch, nth, nz, K, arrs, start=start, **kw)
+    b, itb, _, _ = solve(g, monkeypatch, nth, nz, K, arrs, start=start, variant=1001003, **kw)
+    assert abs(ita - itb) <= 2 and rel_l2(a, b) <= 1e-10
+    a, ita, _, ia = solve(g, monkeypatch, nth, nz, K, arrs, max_iter=7, allow=True, **kw)
+    b, itb, _, ib = solve(g, monkeypatch, nth, nz, K, arrs, max_iter=7, allow=True, variant=1001003, **kw)
+    assert ia["status"] == ib["status"] == g.GMAF_NOT_CONVERGED and ita == itb == 7
+    assert rel_l2(a, b) <= 1e-10
+
+
+def test_resident_solve_matches_the_oracle(g, monkeypatch):
+    nth, nz, K = 132, 45, 9
+    host, arrs = system(nth, nz, K, 3)
+    st, po, ito, _, _ = oracle.solve_joint(nth, nz, *host, precond=1, omega=1.2, eps=1e-12)
+    assert st == 0
+    for precision in (0, 1):
+        p, it, rel, info = solve(g, monkeypatch, nth, nz, K, arrs, precision=precision)
+        assert info["kernel_variant"] // RESIDENT == 1
+        assert np.linalg.norm(p.cpu().numpy() - po.ravel()) <= 1e-10 * np.linalg.norm(po)
+
+
+@pytest.mark.parametrize("nth,nz,K,precision", [(513, 5, 1, 0), (2052, 3, 1, 1), (512, 257, 16, 0)])
+def test_grids_beyond_the_resident_solve_take_the_phase_kernels(g, monkeypatch, nth, nz, K, precision):
+    _, arrs = system(nth, nz, K, 5)
+    p, it, rel, info = solve(g, monkeypatch, nth, nz, K, arrs, precision=precision, allow=True)
+    ref, itr, relr, infr = solve(g, monkeypatch, nth, nz, K, arrs, precision=precision, allow=True,
+                                 variant=1001003 if precision == 0 else 1001004)
+    assert info["kernel_variant"] // RESIDENT == 0 and info["status"] == infr["status"]
+    assert rel_l2(p, ref) <= 1e-10
+
+
+def test_sources_of_any_scale(g, monkeypatch):
+    """The sums over blocks are fixed-point numbers on a scale that follows them: sources
+    scaled by powers of two give the scaled solution, bit for bit."""
+    nth, nz, K = 66, 20, 3
+    _, arrs = system(nth, nz, K, 9)
+    p, it, _, _ = solve(g, monkeypatch, nth, nz, K, arrs)
+    for k in (-300, -40, 60, 300):
+        scaled = arrs[:3] + [arrs[3] * 2.0 ** k]
+        q, itq, _, _ = solve(g, monkeypatch, nth, nz, K, scaled)
+        assert itq == it and torch.equal(q, p * 2.0 ** k)
