@@ -267,7 +267,7 @@ int gmaf_assemble(gmaf_ctx *c, const gmaf_grid *grid, const gmaf_physics *phys,
     if (e != cudaSuccess) return cuda_status(e);
     if ((st = launch_trig(g, (double *)c->buf[B_TRIG], s))) return st;
     if ((st = launch_assemble(g, n_cond, (const double *)c->buf[B_CONDS], slots, D, aE, aN, S,
-                              (const double *)c->buf[B_TRIG], (int *)c->buf[B_FLAGS], n_cond, s)))
+                              (const double *)c->buf[B_TRIG], (int *)c->buf[B_FLAGS], conds, false, s)))
         return st;
     int *flag_h = (int *)((char *)c->pinned + 12288);
     e = cudaMemcpyAsync(flag_h, c->buf[B_FLAGS], sizeof(int), cudaMemcpyDeviceToHost, s);
@@ -317,7 +317,7 @@ int gmaf_integrate_loads(gmaf_ctx *c, const gmaf_grid *grid, const gmaf_physics 
     unsigned *tickets = (unsigned *)c->buf[B_LOADPART];
     double *part = (double *)((char *)c->buf[B_LOADPART] + kMaxCond * sizeof(unsigned));
     return launch_loads(g, n_cond, (const double *)c->buf[B_CONDS], p, (const double *)c->buf[B_TRIG],
-                        part, tickets, loads, (int *)c->buf[B_FLAGS], c->num_sms, s);
+                        part, tickets, loads, (int *)c->buf[B_FLAGS], c->num_sms, conds, false, s);
 }
 
 }  // extern "C"
@@ -369,7 +369,7 @@ static int picard_impl(gmaf_ctx *c, const gmaf_grid *grid, const gmaf_physics *p
     if ((st = launch_fanout(base, d_e, d_edot, conds, cslot_write, s, simplified ? 1 : 0))) return st;
     if ((st = launch_trig(g, (double *)c->buf[B_TRIG], s))) return st;
     if ((st = launch_assemble(g, K, conds, cslot_write, D, aE, aN, S, (const double *)c->buf[B_TRIG],
-                              (int *)c->buf[B_FLAGS], NSLOT, s)))
+                              (int *)c->buf[B_FLAGS], nullptr, simplified, s)))
         return st;
     // (a3) joint solve; the edot-perturbed conditions use the coefficients of condition 0.
     // zero_init = 0 warm-starts from the fields the previous step of this shape and
@@ -393,7 +393,8 @@ static int picard_impl(gmaf_ctx *c, const gmaf_grid *grid, const gmaf_physics *p
     unsigned *tickets = (unsigned *)c->buf[B_LOADPART];
     double *part = (double *)((char *)c->buf[B_LOADPART] + kMaxCond * sizeof(unsigned));
     if ((st = launch_loads(g, K, conds, p, (const double *)c->buf[B_TRIG], part, tickets,
-                           (double *)c->buf[B_LOADS], (int *)c->buf[B_FLAGS], c->num_sms, s)))
+                           (double *)c->buf[B_LOADS], (int *)c->buf[B_FLAGS], c->num_sms, nullptr,
+                           simplified, s)))
         return st;
     PicardIn in{};
     std::memcpy(in.base, base, sizeof base);

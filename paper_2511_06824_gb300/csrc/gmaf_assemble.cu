@@ -1,12 +1,12 @@
 // Geometry, FVM assembly, load integration and the Picard update on the GPU.
 //
 //  - film thickness: Eq. 2.3 with h_Text from a hexagonal dimple lattice;
-//  - assembly: Sec. 2.1 (Eq. 2.1, 2.4-2.7) and Sec. 2.4-I, one thread per cell
-//    looping over the conditions, so the texture and the trigonometry of a cell
-//    are evaluated once for the whole joint batch;
-//  - loads: Sec. 2.4-III, pressure and viscous shear;
+//  - assembly: Sec. 2.1 (Eq. 2.1, 2.4-2.7) and Sec. 2.4-I, one thread per column
+//    marching down the rows, for all conditions of the same eccentricities at once;
+//  - loads: Sec. 2.4-III, pressure and viscous shear, the same way;
 //  - Picard: Eq. 2.12-2.19 with the backward-difference closure of Eq. 2.22.
 #include <cmath>
+#include <cstring>
 
 #include "gmaf_internal.cuh"
 
@@ -56,30 +56,62 @@ Geom make_geom(const gmaf_grid *g, const gmaf_physics *ph, const gmaf_texture *t
 
 // ------------------------------------------------------------------ device: film thickness
 
-// Texture depth at unwrapped (x, z).  The lattice decision is an integer one,
-// so it is written with explicitly rounded operations (no contraction into
-// fused multiply-adds) to take the same decision as a plain IEEE evaluation.
-__device__ __forceinline__ double texture_depth(const Lattice &lt, double x, double z)
+// A point at unwrapped (x, z) is inside a dimple if its distance to the nearest centre
+// of one of four lattice rows is below r.  The lattice decision is an integer one, so
+// it is written with explicitly rounded operations (no contraction into fused
+// multiply-adds) to take the same decision as a plain IEEE evaluation, (dx dx) + (dz dz)
+// < r r for the centres left and right of the point.  It separates: dz depends on the
+// level z and the lattice row only, dx on the column and on the row's parity (odd rows
+// are shifted) only.  A block therefore tables the rows that reach each of its levels
+// (those with dz dz < r r: the sum cannot be smaller), a thread the smaller dx dx of its
+// column for either parity, and a cell is left with one addition and one comparison
+// per row in reach instead of two divisions and eight squares (rounding is monotonic,
+// so the smaller square decides).
+struct Reach {
+    double dz2[4];      // squared distances to the lattice rows in reach
+    int n, odd;         // how many; bit q: row q is odd
+};
+
+__device__ __forceinline__ void lattice_reach(const Lattice &lt, double z, Reach &out)
 {
-    if (!lt.on) return 0.0;
+    out.n = out.odd = 0;
+    if (!lt.on) return;
     const double k0 = floor(__ddiv_rn(__dsub_rn(z, lt.oz), lt.az));
     const double r2 = __dmul_rn(lt.r, lt.r);
-#pragma unroll
     for (int dk = -1; dk <= 2; ++dk) {
         const double k = __dadd_rn(k0, (double)dk);
         const double zc = __dadd_rn(lt.oz, __dmul_rn(k, lt.az));
         const double dz = __dsub_rn(z, zc);
-        const long long ki = (long long)k;
-        const double shift = (ki & 1LL) ? __dmul_rn(0.5, lt.ath) : 0.0;
+        const double dz2 = __dmul_rn(dz, dz);
+        if (!(dz2 < r2)) continue;
+        if ((long long)k & 1LL) out.odd |= 1 << out.n;
+        out.dz2[out.n++] = dz2;
+    }
+}
+
+// The smaller squared distance of column x to the centres of an even (q[0]) or odd (q[1]) row.
+__device__ __forceinline__ void lattice_column(const Lattice &lt, double x, double (&q)[2])
+{
+    q[0] = q[1] = 0.0;
+    if (!lt.on) return;
+#pragma unroll
+    for (int odd = 0; odd < 2; ++odd) {
+        const double shift = odd ? __dmul_rn(0.5, lt.ath) : 0.0;
         const double u = __dsub_rn(__dsub_rn(x, lt.oth), shift);
         const double m = floor(__ddiv_rn(u, lt.ath));
         const double dxa = __dsub_rn(u, __dmul_rn(m, lt.ath));
         const double dxb = __dsub_rn(u, __dmul_rn(__dadd_rn(m, 1.0), lt.ath));
-        const double dz2 = __dmul_rn(dz, dz);
-        if (__dadd_rn(__dmul_rn(dxa, dxa), dz2) < r2) return lt.depth;
-        if (__dadd_rn(__dmul_rn(dxb, dxb), dz2) < r2) return lt.depth;
+        const double a = __dmul_rn(dxa, dxa), b = __dmul_rn(dxb, dxb);
+        q[odd] = a < b ? a : b;
     }
-    return 0.0;
+}
+
+__device__ __forceinline__ double texture_depth(const Lattice &lt, const Reach &z, const double (&q)[2])
+{
+    const double r2 = __dmul_rn(lt.r, lt.r);
+    bool in = false;
+    for (int c = 0; c < z.n; ++c) in = in || __dadd_rn((z.odd >> c) & 1 ? q[1] : q[0], z.dz2[c]) < r2;
+    return in ? lt.depth : 0.0;
 }
 
 // Smooth part of Eq. 2.3 for a condition: sqrt((Rc cos - ex)^2 + (Rc sin - ey)^2) - Rk.
@@ -161,57 +193,141 @@ int launch_fanout(const double *b, double d_e, double d_edot, double *conds, int
     return cuda_status(cudaGetLastError());
 }
 
-// ------------------------------------------------------------------ assembly
+// ------------------------------------------------------------------ conditions of one film
+//
+// The film thickness depends on the eccentricities only, so conditions that differ in
+// their rates share it (a Picard step's base and its four rate perturbations).  A batch
+// is up to kBatch of them; the kernels below evaluate the film once for a batch.
 
-// Pass 1, one thread per cell, all conditions: a_E, a_N, the Dirichlet
-// conductance (parked in D) and the source S.  coef_slot[k] >= 0 selects where
-// condition k's coefficients go; -1 writes only S.
-__global__ void __launch_bounds__(256) k_assemble(Geom g, int ncond,
-                                                  const double *__restrict__ conds,
-                                                  const int *__restrict__ coef_slot,
-                                                  double *__restrict__ D, double *__restrict__ aE,
-                                                  double *__restrict__ aN, double *__restrict__ S,
-                                                  const double *__restrict__ trig,
-                                                  int *__restrict__ flags)
+constexpr int kBatch = 5;
+
+struct Batches {
+    int n;
+    unsigned char cnt[kMaxCond], idx[kMaxCond][kBatch];
+};
+
+// Conditions 0 .. ncond - 1 with the same e (e == nullptr: of a Picard step's fan-out).
+static Batches make_batches(int ncond, const gmaf_state *conds, bool simplified)
 {
+    Batches b{};
+    auto same = [&](int k, int l) {
+        if (conds) return std::memcmp(conds[k].e, conds[l].e, sizeof conds[k].e) == 0;
+        return simplified || ((k == 0 || k >= 5) && (l == 0 || l >= 5));
+    };
+    for (int k = 0; k < ncond; ++k) {
+        int at = -1;
+        for (int q = 0; q < b.n && at < 0; ++q)
+            if (b.cnt[q] < kBatch && same(b.idx[q][0], k)) at = q;
+        if (at < 0) at = b.n++;
+        b.idx[at][b.cnt[at]++] = (unsigned char)k;
+    }
+    return b;
+}
+
+// ------------------------------------------------------------------ assembly
+//
+// Bound by the FP64 pipe (one warp instruction in 16 cycles an SM): every film point
+// costs a square root, every cell two quotients more.  A thread marches down its column
+// for one batch of conditions, so the film at the south face is the one at the north
+// face of the row before, and per row there are three film points for the whole batch.
+// Lane 0 of a warp works on the column west of the warp's 31 others: its a_E is the
+// neighbour's a_W, so that the diagonal is complete without a second pass.  The
+// results are bitwise those of evaluating every cell and condition by itself.
+// 1024 x 512 x 9 cells of a Picard step's conditions: 1486 us that way, 738 us now.
+
+// a / b, correctly rounded, from y = 1 / b (correctly rounded): the product and two
+// corrections by the residual (Markstein), for a divisor that is the same for all cells.
+__device__ __forceinline__ double quotient(double a, double b, double y)
+{
+    double t = a * y;
+    t = fma(y, fma(-b, t, a), t);
+    return fma(y, fma(-b, t, a), t);
+}
+
+constexpr int kAsmWarps = 4, kAsmRows = 32;
+
+// Per row of a block: the axial coordinate of its centre and north face, and what of the
+// texture is in reach of them.
+struct AsmRow {
+    double tc, tn;
+    Reach c, n;
+};
+
+__global__ void __launch_bounds__(kAsmWarps * 32) k_assemble(Geom g, Batches bt,
+                                                             const double *__restrict__ conds,
+                                                             const int *__restrict__ coef_slot,
+                                                             double *__restrict__ D,
+                                                             double *__restrict__ aE,
+                                                             double *__restrict__ aN,
+                                                             double *__restrict__ S,
+                                                             const double *__restrict__ trig,
+                                                             int rows, double inv_dx, double inv_dz,
+                                                             int *__restrict__ flags)
+{
+    __shared__ AsmRow row[kAsmRows];
+    __shared__ Reach south;
+    __shared__ double st[kBatch][8];
+    __shared__ int slot[kBatch];
     const long long n = (long long)g.nth * g.nz;
+    const int nb = bt.cnt[blockIdx.z];
+    const int tid = threadIdx.x, lane = tid & 31;
+    if (tid < 8 * nb) st[tid >> 3][tid & 7] = conds[8 * bt.idx[blockIdx.z][tid >> 3] + (tid & 7)];
+    if (tid < nb) slot[tid] = coef_slot[bt.idx[blockIdx.z][tid]];
+    const int i0 = (blockIdx.x * kAsmWarps + (tid >> 5)) * 31;      // the warp's first own column
+    int i = i0 + lane - 1;
+    const bool own = lane > 0 && i < g.nth;
+    if (i < 0) i = g.nth - 1;
+    if (i >= g.nth) i = g.nth - 1;
+
     const double Ub = -g.v;
     const double inv12mu = 1.0 / (12.0 * g.mu);
     int contact = 0;
-    for (long long P = (long long)blockIdx.x * blockDim.x + threadIdx.x; P < n;
-         P += (long long)gridDim.x * blockDim.x) {
-        const int j = (int)(P / g.nth);
-        const int i = (int)(P - (long long)j * g.nth);
-        const double cc = trig[i], sc = trig[g.nth + i];
-        const double ce = trig[2 * g.nth + i], se = trig[3 * g.nth + i];
-        const double thc = ((double)i + 0.5) * g.dth;
-        const double the = ((double)i + 1.0) * g.dth;
-        const double zc = ((double)j + 0.5) * g.dz;
-        const double zn = ((double)j + 1.0) * g.dz;
-        const double zs = (double)j * g.dz;
-        // texture once per face for the whole joint batch
-        const double hTe = texture_depth(g.lt, __dmul_rn(g.Rk, the), zc);
-        const double hTn = texture_depth(g.lt, __dmul_rn(g.Rk, thc), zn);
-        const double hTs = texture_depth(g.lt, __dmul_rn(g.Rk, thc), zs);
-        const double tc = zc * g.invL, tn = zn * g.invL, ts = zs * g.invL;
-        for (int k = 0; k < ncond; ++k) {
-            const double *st = conds + 8 * k;
-            const FilmPt fe = film_pt(g, st, ce, se, tc);
-            const FilmPt fn = film_pt(g, st, cc, sc, tn);
-            const FilmPt fs = film_pt(g, st, cc, sc, ts);
-            const FilmPt fc = film_pt(g, st, cc, sc, tc);
-            const double he = (fe.rho - g.Rk) + hTe;
-            const double hn = (fn.rho - g.Rk) + hTn;
-            const double hs = (fs.rho - g.Rk) + hTs;
-            contact |= (he <= 0.0) | (hn <= 0.0) | (hs <= 0.0);
-            // dh/dt = -(X/rho) dex/dt - (Y/rho) dey/dt at the cell centre
-            const double exd = st[4] * (1.0 - tc) + st[6] * tc;
-            const double eyd = st[5] * (1.0 - tc) + st[7] * tc;
-            const double hdot = -(fc.X * exd + fc.Y * eyd) / fc.rho;
+    const double cc = trig[i], sc = trig[g.nth + i];
+    const double ce = trig[2 * g.nth + i], se = trig[3 * g.nth + i];
+    double qc[2], qe[2];
+    lattice_column(g.lt, __dmul_rn(g.Rk, ((double)i + 0.5) * g.dth), qc);
+    lattice_column(g.lt, __dmul_rn(g.Rk, ((double)i + 1.0) * g.dth), qe);
+    const int segs = (g.nz + rows - 1) / rows;
+    for (int seg = blockIdx.y; seg < segs; seg += gridDim.y) {
+        const int j0 = seg * rows, j1 = min(j0 + rows, g.nz);
+        __syncthreads();
+        for (int q = tid; q < 2 * (j1 - j0) + 1; q += blockDim.x) {
+            if (q == 2 * (j1 - j0)) {
+                lattice_reach(g.lt, (double)j0 * g.dz, south);
+            } else {
+                const int j = j0 + q / 2;
+                const double z = q & 1 ? ((double)j + 1.0) * g.dz : ((double)j + 0.5) * g.dz;
+                AsmRow &r = row[q / 2];
+                (q & 1 ? r.tn : r.tc) = z * g.invL;
+                lattice_reach(g.lt, z, q & 1 ? r.n : r.c);
+            }
+        }
+        __syncthreads();
+        if (i0 >= g.nth) continue;                                  // (a whole warp)
+        // the south face of the first row
+        double hs, south_n = 0.0;
+        {
+            const FilmPt fs = film_pt(g, st[0], cc, sc, ((double)j0 * g.dz) * g.invL);
+            hs = (fs.rho - g.Rk) + texture_depth(g.lt, south, qc);
+            contact |= hs <= 0.0;
+            if (j0 > 0) south_n = quotient(hs * hs * hs * inv12mu * g.dx, g.dz, inv_dz);
+        }
+        for (int j = j0; j < j1; ++j) {
+            const AsmRow &rw = row[j - j0];
+            const FilmPt fe = film_pt(g, st[0], ce, se, rw.tc);
+            const FilmPt fn = film_pt(g, st[0], cc, sc, rw.tn);
+            const FilmPt fc = film_pt(g, st[0], cc, sc, rw.tc);
+            const double he = (fe.rho - g.Rk) + texture_depth(g.lt, rw.c, qe);
+            const double hn = (fn.rho - g.Rk) + texture_depth(g.lt, rw.n, qc);
+            contact |= (he <= 0.0) | (hn <= 0.0);
             const double gn = hn * hn * hn * inv12mu;
-            const double gs = hs * hs * hs * inv12mu;
+            const double ge = he * he * he * inv12mu;
+            const double east = quotient(ge * g.dz, g.dx, inv_dx);
+            const double north = j < g.nz - 1 ? quotient(gn * g.dx, g.dz, inv_dz) : 0.0;
+            const double west = __shfl_up_sync(0xffffffffu, east, 1);
             double aB = 0.0, sB = 0.0;
             if (j == 0) {
+                const double gs = hs * hs * hs * inv12mu;
                 const double a = gs * g.dx / (0.5 * g.dz);
                 aB += a;
                 sB += a * g.pch;
@@ -221,203 +337,286 @@ __global__ void __launch_bounds__(256) k_assemble(Geom g, int ncond,
                 aB += a;
                 sB += a * g.pcase;
             }
-            const size_t q = (size_t)k * (size_t)n + (size_t)P;
-            S[q] = -(Ub / 2.0) * (hn - hs) * g.dx - hdot * g.dx * g.dz + sB;
-            const int slot = coef_slot[k];
-            if (slot >= 0) {
-                const double ge = he * he * he * inv12mu;
-                const size_t qc = (size_t)slot * (size_t)n + (size_t)P;
-                aE[qc] = ge * g.dz / g.dx;
-                aN[qc] = (j < g.nz - 1) ? gn * g.dx / g.dz : 0.0;
-                D[qc] = aB;
+            // D = a_E + a_W + a_N + a_S + a_B, with a_W(i) = a_E(i - 1) (periodic) and
+            // a_S(j) = a_N(j - 1), so that the stored diagonals describe a symmetric matrix
+            const double diag = east + west + north + south_n + aB;
+            if (own) {
+                const size_t P = (size_t)j * g.nth + i;
+                for (int k = 0; k < nb; ++k) {
+                    // dh/dt = -(X/rho) dex/dt - (Y/rho) dey/dt at the cell centre; the
+                    // multiply-adds are written out, so that S does not depend on how
+                    // the compiler pairs these terms
+                    const double rest = 1.0 - rw.tc;
+                    const double exd = __fma_rn(st[k][4], rest, __dmul_rn(st[k][6], rw.tc));
+                    const double eyd = __fma_rn(st[k][5], rest, __dmul_rn(st[k][7], rw.tc));
+                    const double hdot = -__fma_rn(fc.X, exd, __dmul_rn(fc.Y, eyd)) / fc.rho;
+                    const double wedge = __dmul_rn(-(Ub / 2.0), __dsub_rn(hn, hs));
+                    const double squeeze = __dmul_rn(__dmul_rn(hdot, g.dx), g.dz);
+                    S[(size_t)bt.idx[blockIdx.z][k] * (size_t)n + P] =
+                        __dadd_rn(__fma_rn(wedge, g.dx, -squeeze), sB);
+                    if (slot[k] >= 0) {
+                        const size_t at = (size_t)slot[k] * (size_t)n + P;
+                        aE[at] = east;
+                        aN[at] = north;
+                        D[at] = diag;
+                    }
+                }
             }
+            hs = hn;
+            south_n = north;
         }
     }
     if (contact) atomicOr(flags, 1);
 }
 
-// Pass 2: D = a_E + a_W + a_N + a_S + a_B, with a_W(i) = a_E(i-1) (periodic) and
-// a_S(j) = a_N(j-1), so that the stored diagonals describe a symmetric matrix.
-__global__ void __launch_bounds__(256) k_diag(int nth, int nz, int nslots, double *__restrict__ D,
-                                              const double *__restrict__ aE,
-                                              const double *__restrict__ aN)
-{
-    const long long n = (long long)nth * nz;
-    const long long total = n * nslots;
-    for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; q < total;
-         q += (long long)gridDim.x * blockDim.x) {
-        const long long s = q / n;
-        const long long P = q - s * n;
-        const int j = (int)(P / nth);
-        const int i = (int)(P - (long long)j * nth);
-        const long long base = s * n + (long long)j * nth;
-        const double aW = aE[base + (i == 0 ? nth - 1 : i - 1)];
-        const double aS = (j > 0) ? aN[q - nth] : 0.0;
-        D[q] = aE[q] + aW + aN[q] + aS + D[q];
-    }
-}
-
+// conds_host: the conditions' states (null: a Picard step's fan-out, general or simplified).
 int launch_assemble(const Geom &g, int ncond, const double *conds, const int *coef_slot,
                     double *D, double *aE, double *aN, double *S, const double *trig, int *flags,
-                    int nslots, cudaStream_t s)
+                    const gmaf_state *conds_host, bool simplified, cudaStream_t s)
 {
-    const long long n = (long long)g.nth * g.nz;
-    int blocks = (int)((n + 255) / 256);
-    if (blocks > 152 * 16) blocks = 152 * 16;
-    k_assemble<<<blocks, 256, 0, s>>>(g, ncond, conds, coef_slot, D, aE, aN, S, trig, flags);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return cuda_status(e);
-    long long tot = n * nslots;
-    int b2 = (int)((tot + 255) / 256);
-    if (b2 > 152 * 16) b2 = 152 * 16;
-    k_diag<<<b2, 256, 0, s>>>(g.nth, g.nz, nslots, D, aE, aN);
+    const Batches bt = make_batches(ncond, conds_host, simplified);
+    const int strips = (g.nth + 31 * kAsmWarps - 1) / (31 * kAsmWarps);
+    // rows a block marches: 32, fewer while there are fewer than about 8 blocks an SM
+    int rows = kAsmRows;
+    while (rows > 2 && (long long)strips * ((g.nz + rows - 1) / rows) * bt.n < 152 * 8) rows /= 2;
+    const int segs = (g.nz + rows - 1) / rows;
+    const dim3 grid(strips, segs < 65535 ? segs : 65535, bt.n);
+    k_assemble<<<grid, kAsmWarps * 32, 0, s>>>(g, bt, conds, coef_slot, D, aE, aN, S, trig, rows,
+                                              1.0 / g.dx, 1.0 / g.dz, flags);
     return cuda_status(cudaGetLastError());
 }
 
 // ------------------------------------------------------------------ loads
-
-__device__ __forceinline__ double warp_sum(double x)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-    return x;
-}
-
+//
 // Pressure: the element-wise 2-D trapezoid (mean of the 4 corners times the
 // element area) summed over elements equals a sum over pressure nodes with
 // weight R_k dth (dz_below + dz_above)/2, dz_e = dz/2 for the two boundary
 // element rows.  Shear: per element at its centre, dp/dz and dp/dtheta from
 // differences of edge means.  Node rows r = 0 .. nz+1 (0: z = 0 with p_ch,
 // nz+1: z = L with p_case, else cell centres); element rows er = 0 .. nz.
-// Grid: blockIdx.y = condition.  Each block writes 12 partial sums; the last
-// block of a condition (by ticket) adds them in block order.
-__global__ void __launch_bounds__(256) k_loads(Geom g, const double *__restrict__ conds,
-                                               const double *__restrict__ p,
-                                               const double *__restrict__ trig,
-                                               double *__restrict__ partials,
-                                               unsigned int *__restrict__ tickets,
-                                               double *__restrict__ loads, int *flags)
+//
+// Bound by the FP64 pipe.  The directions (cos, sin) depend on the column only, so a
+// thread marches down its column and keeps five sums for each condition, of p w,
+// z p w, tau_theta A, z tau_theta A and tau_z A; the twelve forces and moments are
+// formed from them once, at the end of the column.  The film of an element is formed
+// once for a batch of conditions of the same eccentricities.  1024 x 512 x 9 cells: 347 us,
+// 2107 us when every thread added up the twelve sums of one condition cell by cell.
+//
+// Grid: blocks (each takes units of a strip of columns x a segment of rows) x batches.
+// Each block writes 12 partial sums a condition; the last block of a batch (by ticket) adds them in block order.
+
+constexpr int kLoadThreads = 128, kLoadRows = 64;
+constexpr int kSums = 12, kShare = 8;           // sums; threads that add up one sum of a block
+
+struct LoadRow {
+    double w, zw;           // weight of node row r = er, and z times it
+    double t, zc;           // z / L and z of the element's centre
+    double cs, ct, cv;      // factors: h dp/dz A, h dp/dtheta / R_k A, 1 / h (Couette) A
+    Reach reach;
+};
+
+// Adds part[b * kSums + c], b = 0 .. nblk - 1, for c = tid / kShare: its kShare threads take
+// every kShare-th block and are added in order.  Threads from kSums * kShare on idle.
+template <typename F>
+__device__ __forceinline__ void add_up(int tid, int nblk, F &&get, double *out)
 {
-    const int k = blockIdx.y;
+    const int c = tid / kShare, l = tid % kShare;
+    double s = 0.0;
+    if (tid < kSums * kShare) {
+#pragma unroll 4
+        for (int b = l; b < nblk; b += kShare) s += get(b, c);
+    }
+    // (whole warps: kSums * kShare is a multiple of 32)
+    if (tid < kSums * kShare) {
+#pragma unroll
+        for (int o = 1; o < kShare; o *= 2) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (l == 0) out[c] = s;
+    }
+}
+
+__global__ void __launch_bounds__(kLoadThreads) k_loads(Geom g, Batches bt,
+                                                        const double *__restrict__ conds,
+                                                        const double *__restrict__ p,
+                                                        const double *__restrict__ trig,
+                                                        double *__restrict__ partials,
+                                                        unsigned int *__restrict__ tickets,
+                                                        double *__restrict__ loads, int rows,
+                                                        int *flags)
+{
+    __shared__ LoadRow row[kLoadRows];
+    __shared__ double red[kSums][kLoadThreads + 1], total[kBatch][kSums], one[kSums];
+    __shared__ int s_last;
     const int nth = g.nth, nz = g.nz;
     const long long n = (long long)nth * nz;
-    const double *pk = p + (size_t)k * (size_t)n;
-    const double *st = conds + 8 * k;
+    const int nb = bt.cnt[blockIdx.y];
+    const unsigned char *idx = bt.idx[blockIdx.y];
+    const int nblk = gridDim.x, blk = blockIdx.x;
+    const int tid = threadIdx.x;
     const double Ub = -g.v;
-    double acc[12];
+    const int strips = (nth + kLoadThreads - 1) / kLoadThreads, segs = (nz + 1 + rows - 1) / rows;
+    double e4[4];
 #pragma unroll
-    for (int q = 0; q < 12; ++q) acc[q] = 0.0;
+    for (int q = 0; q < 4; ++q) e4[q] = conds[8 * idx[0] + q];
+    if (tid < kBatch * kSums) total[tid / kSums][tid % kSums] = 0.0;
     int contact = 0;
-    const long long total = (long long)nth * (nz + 2);
-    for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; q < total;
-         q += (long long)gridDim.x * blockDim.x) {
-        const int r = (int)(q / nth);
-        const int i = (int)(q - (long long)r * nth);
-        // node (i, r): pressure
-        const double zr = (r == 0) ? 0.0 : ((r == nz + 1) ? g.L : ((double)r - 0.5) * g.dz);
-        const double pr = (r == 0) ? g.pch : ((r == nz + 1) ? g.pcase : pk[(size_t)(r - 1) * nth + i]);
-        const double dzb = (r == 0) ? 0.0 : ((r == 1 || r == nz + 1) ? 0.5 * g.dz : g.dz);
-        const double dza = (r == nz + 1) ? 0.0 : ((r == 0 || r == nz) ? 0.5 * g.dz : g.dz);
-        const double w = g.Rk * g.dth * (0.5 * (dzb + dza));
-        {
-            const double ct = trig[i], sn = trig[nth + i];
-            const double fx = -pr * ct * w, fy = -pr * sn * w;
-            const double rx = g.Rk * ct, ry = g.Rk * sn;
-            acc[0] += fx;
-            acc[1] += fy;
-            acc[3] += -zr * fy;
-            acc[4] += zr * fx;
-            acc[5] += rx * fy - ry * fx;
-        }
-        if (r <= nz) {
-            // element (i, er = r): corners (i, r), (i+1, r), (i, r+1), (i+1, r+1)
-            const int i2 = (i + 1 == nth) ? 0 : i + 1;
-            const int er = r;
-            const double pla = pr;
-            const double plb = (er == 0) ? g.pch : pk[(size_t)(er - 1) * nth + i2];
-            const double pha = (er == nz) ? g.pcase : pk[(size_t)er * nth + i];
-            const double phb = (er == nz) ? g.pcase : pk[(size_t)er * nth + i2];
+    for (long long unit = blk; unit < (long long)strips * segs; unit += nblk) {
+        const int seg = (int)(unit / strips), strip = (int)(unit - (long long)seg * strips);
+        const int e0 = seg * rows, e1 = min(e0 + rows, nz + 1);             // element rows
+        __syncthreads();
+        for (int q = tid; q < e1 - e0; q += blockDim.x) {
+            const int er = e0 + q;
+            LoadRow &w = row[q];
+            const double zr = (er == 0) ? 0.0 : ((double)er - 0.5) * g.dz;
+            const double dzb = (er == 0) ? 0.0 : (er == 1 ? 0.5 * g.dz : g.dz);
+            const double dza = (er == 0 || er == nz) ? 0.5 * g.dz : g.dz;
+            w.w = g.Rk * g.dth * (0.5 * (dzb + dza));
+            w.zw = zr * w.w;
             const double dze = (er == 0 || er == nz) ? 0.5 * g.dz : g.dz;
-            const double zlo = zr;
             const double zhi = (er == nz) ? g.L : ((double)er + 0.5) * g.dz;
-            const double zc = 0.5 * (zlo + zhi);
-            const double thc = ((double)i + 1.0) * g.dth;
-            const double ce = trig[2 * nth + i], se = trig[3 * nth + i];
-            const double hT = texture_depth(g.lt, __dmul_rn(g.Rk, thc), zc);
-            const FilmPt f = film_pt(g, st, ce, se, zc * g.invL);
-            const double hc = (f.rho - g.Rk) + hT;
-            contact |= (hc <= 0.0);
-            const double A = g.Rk * g.dth * dze;
-            const double dpdz = ((pha + phb) - (pla + plb)) / (2.0 * dze);
-            const double dpdt = ((plb + phb) - (pla + pha)) / (2.0 * g.dth);
-            const double tz = -(hc / 2.0) * dpdz + g.mu * Ub / hc;
-            const double tt = -(hc / 2.0) * dpdt / g.Rk;
-            const double fx = -tt * se * A, fy = tt * ce * A, fz = tz * A;
-            const double rx = g.Rk * ce, ry = g.Rk * se;
-            acc[6] += fx;
-            acc[7] += fy;
-            acc[8] += fz;
-            acc[9] += ry * fz - zc * fy;
-            acc[10] += zc * fx - rx * fz;
-            acc[11] += rx * fy - ry * fx;
+            w.zc = 0.5 * (zr + zhi);
+            w.t = w.zc * g.invL;
+            // with A = R_k dth dze: -(h/2) dp/dz A = h cs (north - south edge sums),
+            // -(h/2) dp/dtheta / R_k A = h ct (east - west edge sums), mu U_b / h A = cv / h
+            w.cs = -0.25 * g.Rk * g.dth;
+            w.ct = -0.25 * dze;
+            w.cv = g.mu * Ub * (g.Rk * g.dth * dze);
+            lattice_reach(g.lt, w.zc, w.reach);
+        }
+        __syncthreads();
+        const int i = strip * kLoadThreads + tid;
+        double sum[kBatch][5];
+#pragma unroll
+        for (int k = 0; k < kBatch; ++k)
+#pragma unroll
+            for (int q = 0; q < 5; ++q) sum[k][q] = 0.0;
+        double ct = 0.0, sn = 0.0, ce = 0.0, se = 0.0;
+        if (i < nth) {
+            const int i2 = (i + 1 == nth) ? 0 : i + 1;
+            ct = trig[i];
+            sn = trig[nth + i];
+            ce = trig[2 * nth + i];
+            se = trig[3 * nth + i];
+            double qe[2];
+            lattice_column(g.lt, __dmul_rn(g.Rk, ((double)i + 1.0) * g.dth), qe);
+            // pressure of node row r at columns i and i + 1
+            auto node = [&](int k, int r, double &a, double &b) {
+                if (r == 0) {
+                    a = b = g.pch;
+                } else if (r == nz + 1) {
+                    a = b = g.pcase;
+                } else {
+                    const double *pk = p + (size_t)idx[k] * (size_t)n + (size_t)(r - 1) * nth;
+                    a = pk[i];
+                    b = pk[i2];
+                }
+            };
+            double pa[kBatch], pb[kBatch];
+#pragma unroll
+            for (int k = 0; k < kBatch; ++k)
+                if (k < nb) node(k, e0, pa[k], pb[k]);
+            for (int er = e0; er < e1; ++er) {
+                const LoadRow &w = row[er - e0];
+                double na[kBatch], nc[kBatch];
+#pragma unroll
+                for (int k = 0; k < kBatch; ++k)
+                    if (k < nb) node(k, er + 1, na[k], nc[k]);
+                const FilmPt f = film_pt(g, e4, ce, se, w.t);
+                const double h = (f.rho - g.Rk) + texture_depth(g.lt, w.reach, qe);
+                contact |= (h <= 0.0);
+                const double couette = w.cv / h, hcs = h * w.cs, hct = h * w.ct;
+#pragma unroll
+                for (int k = 0; k < kBatch; ++k) {
+                    if (k >= nb) continue;
+                    const double tz = fma(hcs, (na[k] + nc[k]) - (pa[k] + pb[k]), couette);
+                    const double tt = hct * ((pb[k] + nc[k]) - (pa[k] + na[k]));
+                    sum[k][0] = fma(pa[k], w.w, sum[k][0]);
+                    sum[k][1] = fma(pa[k], w.zw, sum[k][1]);
+                    sum[k][2] += tt;
+                    sum[k][3] = fma(w.zc, tt, sum[k][3]);
+                    sum[k][4] += tz;
+                    pa[k] = na[k];
+                    pb[k] = nc[k];
+                }
+            }
+            if (e1 == nz + 1) {
+                // the last node row, z = L
+                const double wl = g.Rk * g.dth * (0.5 * (0.5 * g.dz));
+#pragma unroll
+                for (int k = 0; k < kBatch; ++k)
+                    if (k < nb) {
+                        sum[k][0] = fma(pa[k], wl, sum[k][0]);
+                        sum[k][1] = fma(pa[k], g.L * wl, sum[k][1]);
+                    }
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < kBatch; ++k) {
+            if (k >= nb) continue;
+            const double P = sum[k][0], Pz = sum[k][1], T = sum[k][2], Tz = sum[k][3], Z = sum[k][4];
+            const double fx = -P * ct, fy = -P * sn;
+            red[0][tid] = fx;
+            red[1][tid] = fy;
+            red[2][tid] = 0.0;
+            red[3][tid] = Pz * sn;
+            red[4][tid] = -Pz * ct;
+            red[5][tid] = g.Rk * ct * fy - g.Rk * sn * fx;
+            red[6][tid] = -T * se;
+            red[7][tid] = T * ce;
+            red[8][tid] = Z;
+            red[9][tid] = g.Rk * se * Z - Tz * ce;
+            red[10][tid] = -Tz * se - g.Rk * ce * Z;
+            red[11][tid] = g.Rk * ce * (T * ce) + g.Rk * se * (T * se);
+            __syncthreads();
+            add_up(tid, kLoadThreads, [&](int b, int c) { return red[c][b]; }, one);
+            __syncthreads();
+            if (tid < kSums) total[k][tid] += one[tid];
         }
     }
     if (contact) atomicOr(flags, 1);
-
-    __shared__ double red[12][8];
-    __shared__ int s_last;
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-#pragma unroll
-    for (int q = 0; q < 12; ++q) {
-        const double s = warp_sum(acc[q]);
-        if (lane == 0) red[q][wid] = s;
-    }
     __syncthreads();
-    double *part = partials + (size_t)k * gridDim.x * 12;
-    if (threadIdx.x < 12) {
-        double s = 0.0;
-        for (int w2 = 0; w2 < nw; ++w2) s += red[threadIdx.x][w2];
-        part[(size_t)blockIdx.x * 12 + threadIdx.x] = s;
-    }
+    for (int q = tid; q < nb * kSums; q += blockDim.x)
+        partials[((size_t)idx[q / kSums] * nblk + blk) * kSums + q % kSums] = total[q / kSums][q % kSums];
     __threadfence();
     __syncthreads();
-    if (threadIdx.x == 0) {
-        const unsigned t = atomicAdd(&tickets[k], 1u);
-        s_last = (t == gridDim.x - 1);
+    if (tid == 0) {
+        const unsigned t = atomicAdd(&tickets[idx[0]], 1u);
+        s_last = (t == (unsigned)nblk - 1u);
     }
     __syncthreads();
     if (!s_last) return;
     __threadfence();
-    if (threadIdx.x < 12) {
-        double s = 0.0;
-        for (unsigned b = 0; b < gridDim.x; ++b) s += __ldcg(&part[(size_t)b * 12 + threadIdx.x]);
-        loads[(size_t)k * 12 + threadIdx.x] = s;
+    for (int k = 0; k < nb; ++k) {
+        const double *part = partials + (size_t)idx[k] * nblk * kSums;
+        add_up(tid, nblk, [&](int b, int c) { return __ldcg(part + (size_t)b * kSums + c); },
+               loads + (size_t)idx[k] * kSums);
     }
-    if (threadIdx.x == 0) tickets[k] = 0u;
+    if (tid == 0) tickets[idx[0]] = 0u;
 }
 
-static int loads_blocks(const Geom &g, int num_sms)
-{
-    const long long total = (long long)g.nth * (g.nz + 2);
-    long long b = (total + 255) / 256;
-    long long cap = (long long)num_sms * 2;
-    if (b > cap) b = cap;
-    if (b < 1) b = 1;
-    return (int)b;
-}
-
+// Blocks a condition may have (its partial sums): two an SM.
 size_t loads_partials_bytes(int ncond, int num_sms)
 {
-    return (size_t)ncond * (size_t)num_sms * 2 * 12 * sizeof(double) + kMaxCond * sizeof(unsigned);
+    return (size_t)ncond * (size_t)num_sms * 2 * kSums * sizeof(double) + kMaxCond * sizeof(unsigned);
 }
 
+// conds_host: as in launch_assemble.
 int launch_loads(const Geom &g, int ncond, const double *conds, const double *p,
                  const double *trig, double *partials, unsigned int *tickets, double *loads,
-                 int *flags, int num_sms, cudaStream_t s)
+                 int *flags, int num_sms, const gmaf_state *conds_host, bool simplified,
+                 cudaStream_t s)
 {
-    const int bx = loads_blocks(g, num_sms);
-    dim3 grid(bx, ncond);
-    k_loads<<<grid, 256, 0, s>>>(g, conds, p, trig, partials, tickets, loads, flags);
+    const Batches bt = make_batches(ncond, conds_host, simplified);
+    const int er = g.nz + 1, strips = (g.nth + kLoadThreads - 1) / kLoadThreads;
+    // segments of rows: short ones on small grids, so that every SM has work, but no more
+    // blocks a condition than there are partial sums
+    const long long most = 2LL * num_sms;
+    int rows = kLoadRows;
+    while (rows > 2 && (long long)strips * ((er + rows - 1) / rows) * bt.n < 8LL * num_sms &&
+           (long long)strips * ((er + rows / 2 - 1) / (rows / 2)) <= most)
+        rows /= 2;
+    const long long units = (long long)strips * ((er + rows - 1) / rows);
+    k_loads<<<dim3((unsigned)(units < most ? units : most), bt.n), kLoadThreads, 0, s>>>(
+        g, bt, conds, p, trig, partials, tickets, loads, rows, flags);
     return cuda_status(cudaGetLastError());
 }
 

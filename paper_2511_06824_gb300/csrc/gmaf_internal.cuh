@@ -211,12 +211,14 @@ int launch_trig(const Geom &g, double *trig, cudaStream_t s);
 // in 5 coefficient slots; 1: the 5 of the simplified scheme (base, edot_j + d_edot) in 1 slot.
 int launch_fanout(const double *base, double d_e, double d_edot, double *conds, int *cslot_write,
                   cudaStream_t s, int simplified = 0);
+// conds_host: the states behind conds (null: a Picard step's fan-out, general or simplified).
 int launch_assemble(const Geom &g, int ncond, const double *conds, const int *coef_slot,
                     double *D, double *aE, double *aN, double *S, const double *trig, int *flags,
-                    int nslots, cudaStream_t s);
+                    const gmaf_state *conds_host, bool simplified, cudaStream_t s);
 int launch_loads(const Geom &g, int ncond, const double *conds, const double *p,
                  const double *trig, double *partials, unsigned int *tickets, double *loads,
-                 int *flags, int num_sms, cudaStream_t s);
+                 int *flags, int num_sms, const gmaf_state *conds_host, bool simplified,
+                 cudaStream_t s);
 struct PicardIn {
     double base[8], e_prev[4], F_ext[4];
     int simplified;                // Eq. 2.20-2.22 on the 5-condition batch

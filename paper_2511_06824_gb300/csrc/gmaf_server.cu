@@ -364,7 +364,7 @@ static int admit(gmaf_server *sv, Request *r)
     if ((st = launch_fanout(base, r->in.d_e, r->in.d_edot, r->conds, r->cslot_w, s))) return st;
     if ((st = launch_trig(r->g, r->trig, s))) return st;
     if ((st = launch_assemble(r->g, 9, r->conds, r->cslot_w, r->D, r->aE, r->aN, r->S, r->trig,
-                              r->flags, 5, s)))
+                              r->flags, nullptr, false, s)))
         return st;
     const long long m = 5 * r->n;
     k_to_f32<<<stream_grid_s(m, sv->num_sms), kThreads, 0, s>>>(r->D, r->aE, r->aN, r->D32, r->invD32,
@@ -440,7 +440,7 @@ static int retire(gmaf_server *sv, Request *r, int status, double true_rel)
     cudaStream_t s = sv->stream;
     int st;
     if ((st = launch_loads(r->g, 9, r->conds, r->p, r->trig, r->part, r->tickets, r->loads, r->flags,
-                           sv->num_sms, s)))
+                           sv->num_sms, nullptr, false, s)))
         return st;
     PicardIn in{};
     std::memcpy(in.base, r->in.state.e, 4 * sizeof(double));
