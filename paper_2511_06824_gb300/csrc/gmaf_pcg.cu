@@ -944,13 +944,15 @@ static int res_run(gmaf_ctx *ctx, ResRun<T> &rr, long long most_iterations, bool
     }
     GMAF_CUDA(e);
     if (q.times) {
-        unsigned long long t[5];
+        unsigned long long t[7];
         GMAF_CUDA(cudaMemcpyAsync(t, q.times, sizeof t, cudaMemcpyDeviceToHost, s));
         GMAF_CUDA(cudaStreamSynchronize(s));
         for (int k = 0; k < 3; ++k) ctx->phase_ms[k] += 1e-6 * (double)t[k];
         ctx->phase_count[0] += (long long)t[3];
         ctx->phase_count[1] += (long long)t[4];
         ctx->phase_count[2] += 1;
+        ctx->phase_ms[3] += 1e-6 * (double)t[5];
+        ctx->phase_count[3] += (long long)t[6];
     }
     return GMAF_OK;
 }
@@ -974,7 +976,6 @@ static int solve_resident64(gmaf_ctx *ctx, ResRun<double> &rr, int K, const int 
     q.groups = G;
     q.sc = gsc;
     q.mode = kResFresh;
-    q.keep_iter = 0;
     // descriptors of the residuals: condition k, or the joint system
     const size_t o_slot = align256((size_t)kMaxCond * sizeof(ResidDesc));
     GMAF_TRY(ensure(ctx, B_ASYNC, o_slot + 256));
@@ -1050,7 +1051,6 @@ static int solve_resident64(gmaf_ctx *ctx, ResRun<double> &rr, int K, const int 
             GMAF_TRY(residuals());
             q.r_in = (const double *)ctx->buf[B_R0];
             q.mode = kResRestart;
-            q.keep_iter = 1;
         }
     }
     GMAF_CUDA(cudaStreamSynchronize(s));
@@ -1079,6 +1079,9 @@ static int solve_resident64(gmaf_ctx *ctx, ResRun<double> &rr, int K, const int 
     *info = inf;
     return status;
 }
+
+// FP64 refinements of a mixed-precision solve, continued or restarted each time.
+constexpr int kMaxOuterContinued = 200, kMaxOuterRestart = 12;
 
 int solve_joint_device(gmaf_ctx *ctx, int nth, int nz, int K, int nslots, const int *cslot_host,
                        const double *D, const double *aE, const double *aN, const double *S,
@@ -1141,7 +1144,6 @@ int solve_joint_device(gmaf_ctx *ctx, int nth, int nz, int K, int nslots, const 
             q.max_iter = opts->max_iter;
             q.guard_limit = ctx->loop_guard;
             q.eps = opts->eps;
-            q.cscale = 0.0;
             q.D = D;
             q.invD = (const double *)ctx->buf[B_INVD];
             q.aE = aE;
@@ -1150,7 +1152,6 @@ int solve_joint_device(gmaf_ctx *ctx, int nth, int nz, int K, int nslots, const 
             q.b = S;
             q.r_in = nullptr;
             q.p = p;
-            q.u = nullptr;
             bool off = false;
             const int st = solve_resident64(ctx, rr, K, cslot_host, S, p, opts, info, &off);
             if (!off) return st;
@@ -1250,16 +1251,6 @@ int solve_joint_device(gmaf_ctx *ctx, int nth, int nz, int K, int nslots, const 
     GMAF_TRY(ensure(ctx, B_INVD32, (size_t)m * sizeof(float)));
     GMAF_TRY(ensure(ctx, B_AE32, (size_t)m * sizeof(float)));
     GMAF_TRY(ensure(ctx, B_AN32, (size_t)m * sizeof(float)));
-    for (int b : {B_B32, B_X32, B_U032}) GMAF_TRY(ensure(ctx, b, (size_t)N * sizeof(float)));
-    ResRun<float> rr;
-    res_setup<float>(ctx, rr, nth, nz, K, nth % 4 == 0);
-    // the fields of the phase kernels
-    auto phase_buffers = [&]() -> int {
-        for (int b : {B_R032, B_R132, B_U132, B_Z32, B_V32})
-            GMAF_TRY(ensure(ctx, b, (size_t)N * sizeof(float)));
-        return GMAF_OK;
-    };
-    if (!rr.on) GMAF_TRY(phase_buffers());
     GMAF_TRY(ensure(ctx, B_R64, (size_t)N * sizeof(double)));
     k_to_f32<<<stream_grid(m, ctx->num_sms), kThreads, 0, s>>>(
         D, aE, aN, (float *)ctx->buf[B_D32], (float *)ctx->buf[B_INVD32], (float *)ctx->buf[B_AE32],
@@ -1269,6 +1260,52 @@ int solve_joint_device(gmaf_ctx *ctx, int nth, int nz, int K, int nslots, const 
             D, aE, aN, nth, nz, m, opts->omega, dsc_outer, (float *)ctx->buf[B_INVD32]);
     GMAF_CUDA(cudaGetLastError());
     if (opts->zero_init) GMAF_CUDA(cudaMemsetAsync(p, 0, (size_t)N * sizeof(double), s));
+
+    // the whole refinement in one launch where the system fits on the SMs
+    ResRun<float> rr;
+    res_setup<float>(ctx, rr, nth, nz, K, nth % 4 == 0);
+    if (rr.on) {
+        if (rr.pl.o_x < 0) GMAF_TRY(ensure(ctx, B_X32, (size_t)N * sizeof(float)));
+        ResParams<float> &q = rr.q;
+        q.precond = kernel_precond(opts);
+        q.max_iter = opts->max_iter;
+        q.guard_limit = ctx->loop_guard;
+        q.eps = opts->eps;
+        q.D = (const float *)ctx->buf[B_D32];
+        q.invD = (const float *)ctx->buf[B_INVD32];
+        q.aE = (const float *)ctx->buf[B_AE32];
+        q.aN = (const float *)ctx->buf[B_AN32];
+        q.cslot = cslot;
+        q.p = (float *)ctx->buf[B_X32];
+        q.sc = dsc;
+        q.D64 = D;
+        q.aE64 = aE;
+        q.aN64 = aN;
+        q.S64 = S;
+        q.scale = &dsc_outer->scale;
+        q.p64 = p;
+        q.r64 = (double *)ctx->buf[B_R64];
+        q.continued = ctx->mixed_restart ? 0 : 1;
+        q.inner_floor = q.continued ? ctx->reliable_delta : ctx->inner_floor;
+        q.max_outer = q.continued ? kMaxOuterContinued : kMaxOuterRestart;
+        bool off = false;
+        GMAF_TRY(res_run<float>(ctx, rr, (long long)opts->max_iter + 2 * q.max_outer, &off));
+        if (!off) {
+            GMAF_TRY(read_scalars(ctx, dsc, hsc));
+            inf.iterations = hsc->iter;
+            inf.iterations_sum = hsc->iter * K;
+            inf.outer_iterations = hsc->guard;
+            inf.status = hsc->status;
+            inf.true_rel_residual = inf.rel_residual = hsc->true_rel;
+            inf.kernel_variant = kResVariant + 1000 * rr.pl.vec + 10 * rr.pl.rr;
+            inf.tasks = rr.pl.grid;
+            inf.p_update_period = 1;
+            *info = inf;
+            return inf.status;
+        }
+    }
+    for (int b : {B_B32, B_X32, B_R032, B_R132, B_U032, B_U132, B_Z32, B_V32})
+        GMAF_TRY(ensure(ctx, b, (size_t)N * sizeof(float)));
 
     PcgRun<float> run{};
     PcgDesc<float> &h = run.h;
@@ -1288,37 +1325,19 @@ int solve_joint_device(gmaf_ctx *ctx, int nth, int nz, int K, int nslots, const 
     h.omega = (float)opts->omega;
     h.sc = dsc;
     h.nslots = nslots;
-    if (!rr.on && nth % 4 == 0) {
+    h.z = (float *)ctx->buf[B_Z32];
+    h.v = (float *)ctx->buf[B_V32];
+    h.u[0] = (float *)ctx->buf[B_U032];
+    h.u[1] = (float *)ctx->buf[B_U132];
+    h.r[0] = (float *)ctx->buf[B_R032];
+    h.r[1] = (float *)ctx->buf[B_R132];
+    if (nth % 4 == 0) {
         // the boundary term of the diagonal for the phase A variant that rebuilds it
         GMAF_TRY(ensure(ctx, B_DBND32, (size_t)nslots * 2 * nth * sizeof(float)));
         GMAF_TRY(launch_dbnd32(h.D, h.aE, h.aN, (float *)ctx->buf[B_DBND32], nth, nz, nslots,
                                ctx->num_sms, s));
         h.dbnd = (const float *)ctx->buf[B_DBND32];
         run.drec_ready = true;
-    }
-    auto phase_fields = [&]() {
-        h.z = (float *)ctx->buf[B_Z32];
-        h.v = (float *)ctx->buf[B_V32];
-        h.u[0] = (float *)ctx->buf[B_U032];
-        h.u[1] = (float *)ctx->buf[B_U132];
-        h.r[0] = (float *)ctx->buf[B_R032];
-        h.r[1] = (float *)ctx->buf[B_R132];
-    };
-    if (!rr.on) phase_fields();
-    if (rr.on) {
-        ResParams<float> &q = rr.q;
-        q.precond = kernel_precond(opts);
-        q.zero_init = 1;
-        q.D = h.D;
-        q.invD = h.invD;
-        q.aE = h.aE;
-        q.aN = h.aN;
-        q.cslot = cslot;
-        q.b = h.b;
-        q.r_in = nullptr;
-        q.p = h.p;
-        q.u = (float *)ctx->buf[B_U032];
-        q.sc = dsc;
     }
     // The first outer residual and the inner right-hand side are formed before the
     // kernel set is chosen, so that the autotuner times iterations on real data.
@@ -1339,7 +1358,7 @@ int solve_joint_device(gmaf_ctx *ctx, int nth, int nz, int K, int nslots, const 
     // the inner floor (GMAF_INNER_EPS) each time.
     const bool continued = !ctx->mixed_restart;
     const double inner_floor = continued ? ctx->reliable_delta : ctx->inner_floor;
-    const int max_outer = continued ? 200 : 12;
+    const int max_outer = continued ? kMaxOuterContinued : kMaxOuterRestart;
     int total_inner = 0, outer = 0, longest = 0;
     int last_iter = 0;          // the inner iteration counter at the end of the last solve
     bool tuned = false, stalled = false;
@@ -1369,7 +1388,7 @@ int solve_joint_device(gmaf_ctx *ctx, int nth, int nz, int K, int nslots, const 
         k_make_b32<<<gs, kThreads, 0, s>>>((const double *)ctx->buf[B_R64], (float *)ctx->buf[B_B32],
                                            N, dsc_outer);
         GMAF_CUDA(cudaGetLastError());
-        if (!tuned && !rr.on) {
+        if (!tuned) {
             GMAF_TRY(setup_run<float>(ctx, run, (PcgDesc<float> *)(dbase + 1024)));
             rd.partials = h.partials;
             GMAF_CUDA(cudaMemcpyAsync(d_rdesc, &rd, sizeof(ResidDesc), cudaMemcpyHostToDevice, s));
@@ -1388,28 +1407,8 @@ int solve_joint_device(gmaf_ctx *ctx, int nth, int nz, int K, int nslots, const 
         const int cap = std::max(1000, 4 * longest);
         h.max_iter = cont ? last_iter + std::min(left, cap) : left;
         h.guard_limit = ctx->loop_guard;
-        const double cscale = cont ? rnorm_prev / ho->rnorm : 0.0;
-        if (rr.on) {
-            ResParams<float> &q = rr.q;
-            q.mode = cont ? kResContinue : kResFresh;
-            q.keep_iter = cont ? 1 : 0;
-            q.max_iter = h.max_iter;
-            q.guard_limit = h.guard_limit;
-            q.eps = h.eps;
-            q.cscale = cscale;
-            bool off = false;
-            GMAF_TRY(res_run<float>(ctx, rr, cont ? h.max_iter - last_iter : h.max_iter, &off));
-            if (off) {
-                // the blocks cannot all be resident: the phase kernels from here on
-                rr.on = false;
-                GMAF_TRY(phase_buffers());
-                phase_fields();
-                continue;
-            }
-        } else {
-            GMAF_TRY(prepare<float>(ctx, run, ctx->graph32));
-            GMAF_TRY(pcg_once<float>(ctx, run, ctx->graph32, cont, true, cscale));
-        }
+        GMAF_TRY(prepare<float>(ctx, run, ctx->graph32));
+        GMAF_TRY(pcg_once<float>(ctx, run, ctx->graph32, cont, true, cont ? rnorm_prev / ho->rnorm : 0.0));
         rnorm_prev = ho->rnorm;
         k_update_p64<<<gs, kThreads, 0, s>>>(p, (const float *)ctx->buf[B_X32], N, dsc_outer);
         GMAF_CUDA(cudaGetLastError());
@@ -1429,8 +1428,8 @@ int solve_joint_device(gmaf_ctx *ctx, int nth, int nz, int K, int nslots, const 
     inf.iterations = total_inner;
     inf.iterations_sum = total_inner * K;
     inf.outer_iterations = outer;
-    inf.kernel_variant = rr.on ? kResVariant + 1000 * rr.pl.vec + 10 * rr.pl.rr : run.ks.id;
-    inf.tasks = rr.on ? rr.pl.grid : (int)run.h.ntiles;
+    inf.kernel_variant = run.ks.id;
+    inf.tasks = (int)run.h.ntiles;
     inf.p_update_period = std::max(1, run.ks.p_period);
     *info = inf;
     return inf.status;

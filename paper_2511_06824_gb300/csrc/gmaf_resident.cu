@@ -84,7 +84,8 @@ bool res_plan(int nth, int nz, int K, bool vec_ok, int num_sms, ResPlan *out)
     pl.smem = (int)o;
     pl.fn = sz == 4 ? res_kernel_f32(pl.vec, pl.rr, cs) : res_kernel_f64(pl.vec, pl.rr, cs);
     if (!pl.fn) return false;
-    pl.halo_bytes = (size_t)pl.grid * 4 * nth * 2 * sz;
+    // flagged rows: four of T, and for FP32 two of doubles behind them
+    pl.halo_bytes = (size_t)pl.grid * 4 * nth * 2 * sz + (sz == 4 ? (size_t)pl.grid * 2 * nth * 16 : 0);
     *out = pl;
     return true;
 }
@@ -102,6 +103,7 @@ void res_fill(const ResPlan &pl, ResParams<T> *q)
     q->o_edge = pl.o_edge;
     q->o_x = pl.o_x;
     q->halo_row = q->nth * ((int)sizeof(T) / 4);
+    q->halo64 = q->halo + (size_t)pl.grid * 4 * q->halo_row;
 }
 
 template <typename T>

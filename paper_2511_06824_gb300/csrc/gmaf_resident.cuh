@@ -240,24 +240,40 @@ struct ResLimbs {
 // m 2^up in units of the lowest bit (m of `bits` bits), added with its sign.
 __device__ __forceinline__ void res_limbs_add(ResLimbs &x, unsigned long long m, int up, bool neg, int bits)
 {
-    unsigned long long lo, top;
-    if (up >= kResLimb) {
-        lo = 0;
-        top = m << ((up - kResLimb) & 63);
-    } else if (up >= 0) {
-        lo = (m << up) & kResLimbMask;
-        top = m >> (kResLimb - up);
-    } else {
-        m = up > -64 ? m >> -up : 0ull;
-        lo = m & kResLimbMask;
-        top = m >> kResLimb;
+    const bool over = (up + bits > kResTop + 14 || up > 63) && m != 0;
+    const int left = min(max(up, 0), 63);
+    m = over ? 0ull : m >> min(max(-up, 0), 63);
+    const unsigned long long low = m << left, high = left ? m >> (64 - left) : 0ull;
+    const long long lo = (long long)(low & kResLimbMask);
+    const long long top = (long long)((low >> kResLimb) | (high << (64 - kResLimb)));
+    x.over = x.over || over;
+    x.lo += neg ? -lo : lo;
+    x.top += neg ? -top : top;
+}
+// (top 2^44 + lo) 2^(e - 1089), e - 1089 the weight of the lowest bit, rounded to a double.
+__device__ __forceinline__ double res_value(long long top, long long lo, int e)
+{
+    top += lo >> kResLimb;
+    unsigned long long l = (unsigned long long)lo & kResLimbMask;
+    const bool neg = top < 0;
+    unsigned long long h = (unsigned long long)top;
+    if (neg) {
+        h = 0ull - h - (l != 0);
+        l = (0ull - l) & kResLimbMask;
     }
-    if (up + bits > kResTop + 14) {
-        if (m != 0) x.over = true;
-        lo = top = 0;
-    }
-    x.lo += neg ? -(long long)lo : (long long)lo;
-    x.top += neg ? -(long long)top : (long long)top;
+    // the leading 64 bits, the leading one on top
+    const int hz = __clzll(h), lz = __clzll(l);
+    const bool big = h != 0;
+    unsigned long long m = big ? (hz >= kResLimb ? (h << hz) | (l << (hz - kResLimb))
+                                                 : (h << hz) | (l >> (kResLimb - hz)))
+                               : l << (lz & 63);
+    int lead = big ? kResLimb + 63 - hz : 63 - lz;
+    if (!big && l == 0) return 0.0;
+    const unsigned long long r = m + 1024ull;            // to nearest
+    if (r < m) ++lead;
+    const unsigned long long bits = ((unsigned long long)(lead + e - kResTop) << 52) |
+                                    ((r < m ? 0ull : r >> 11) & 0xfffffffffffffull);
+    return __longlong_as_double((long long)(bits | (neg ? 1ull << 63 : 0ull)));
 }
 __device__ __forceinline__ ResLimbs res_limbs(const ResTerm<double> &t, int e)
 {
@@ -295,13 +311,14 @@ __device__ __forceinline__ ResLimbs res_limbs(const ResTerm<float> &t, int e)
 // exchange before.  Words of one kind are added to again only after an exchange of
 // another kind, which no block completes before all have read these.
 
-enum ResWord { kWordUV = 0, kWordRZ = 4, kWordMaxCount = 8, kWordMax = 9 };
-static_assert(kWordMax + 2 <= kResGroupWords, "words of a group");
+enum ResWord { kWordUV = 0, kWordRZ = 4, kWordMaxCount = 8, kWordMax = 9, kWordR64 = 12 };
+static_assert(kWordR64 + 4 <= kResGroupWords, "words of a group");
 
 struct ResSums {
     unsigned long long *w;              // the group's words (zero at the start of the run)
-    unsigned long long prev[6], prev_max;
-    int nb, e[3];                       // blocks; exponent expected of u.v, r.z, r.r (0: not known)
+    unsigned long long prev[10], prev_max;
+    int nb, e[5];                       // blocks; exponent expected of u.v, r.z, r.r, and of
+                                        // r.r and S.S in FP64 (0: not known)
     unsigned turn;
 };
 
@@ -341,9 +358,10 @@ template <int NV, typename T>
 __device__ __forceinline__ bool res_totals(ResSums &x, int kind, const ResTerm<T> (&term)[NV], int lane,
                                            double (&tot)[NV])
 {
-    unsigned long long *const w = x.w + (kind == 0 ? kWordUV : kWordRZ);
-    unsigned long long *prev = x.prev + 2 * kind;
-    int *e = x.e + kind;
+    // kind 0: u.v; 1: r.z and r.r; 2: the FP64 residual's and source's
+    unsigned long long *const w = x.w + (kind == 0 ? kWordUV : kind == 1 ? kWordRZ : kWordR64);
+    unsigned long long *prev = x.prev + (kind == 0 ? 0 : kind == 1 ? 2 : 6);
+    int *e = x.e + (kind == 0 ? 0 : kind == 1 ? 1 : 3);
     bool known = true;
 #pragma unroll
     for (int q = 0; q < NV; ++q) known = known && e[q] != 0;
@@ -388,9 +406,7 @@ __device__ __forceinline__ bool res_totals(ResSums &x, int kind, const ResTerm<T
         for (int q = 0; q < NV; ++q) {
             const long long lo = (long long)(d[2 * q] - prev[2 * q]) >> 8;
             const unsigned long long t = d[2 * q + 1] - prev[2 * q + 1];
-            const double s = fma((double)((long long)t >> 16), (double)(1ull << kResLimb), (double)lo);
-            tot[q] = s == 0.0 ? 0.0 : __hiloint2double(__double2hiint(s) + ((en[q] - 1023 - kResTop) << 20),
-                                                       __double2loint(s));
+            tot[q] = res_value((long long)t >> 16, lo, en[q]);
             good = good && ((t >> 8) & 0xffull) == 0 && res_exp(tot[q]) >= e[q] - 12;
             prev[2 * q] = d[2 * q];
             prev[2 * q + 1] = d[2 * q + 1];
@@ -442,164 +458,293 @@ __device__ __forceinline__ unsigned long long res_time()
 // Shared state of a block.
 template <typename T>
 struct ResShared {
-    ResTerm<T> part[2][kResThreads / 32];   // the warps' sums
+    ResTerm<T> part[2][kResThreads / 32];           // the warps' sums
+    ResTerm<double> part64[2][kResThreads / 32];    // (of the FP64 residual)
     double alpha, beta;
-    int done, halo_failed;
+    double unit, back;                  // mixed precision: 1 / ||r64||; scale ||r64||, which takes x to p
+    int done, stop, halo_failed;
 };
+
+// (one object per block: a function's own shared variable)
+template <typename T>
+__device__ __forceinline__ ResShared<T> &res_shared()
+{
+    __shared__ ResShared<T> sh;
+    return sh;
+}
 
 // The warp that takes no rows: adds the block's sums, exchanges them, updates the
 // scalars (finish_a and finish_b of the phase kernels) and decides when to stop.
 template <typename T>
-__device__ __forceinline__ void res_exchange_warp(const ResParams<T> &q, ResShared<T> &sh, Scalars *sc,
-                                                  int g0, int nb, int lane)
-{
-    const int all = q.threads + 32, warps = q.threads / 32;
-    const int blk = blockIdx.x;
-    int iter = q.keep_iter ? sc->iter : 0;
-    double d = 0.0, normS = q.mode == kResRestart ? sc->normS : 0.0, rr_last = 0.0, alpha = 0.0;
-    int status = 0, converged = 0, zero_rhs = 0, guard = 0, done = 0;
-    const bool timed = q.times != nullptr && lane == 0 && blk == 0;
-    unsigned long long t_mark = timed ? res_time() : 0ull;
-    auto mark = [&](int k) {
+struct ResExchange {
+    const ResParams<T> &q;
+    ResShared<T> &sh;
+    const int all, warps, lane;
+    ResSums sums;
+    int iter, status, converged, zero_rhs, done;
+    double d, normS, rr_last, alpha;
+    bool timed;
+    unsigned long long t_mark;
+
+    __device__ __forceinline__ void mark(int k)
+    {
         if (!timed) return;
         const unsigned long long t = res_time();
         q.times[k] += t - t_mark;
         t_mark = t;
-    };
-    auto gather = [&](int w) {
+    }
+    __device__ __forceinline__ ResTerm<T> gather(int w) const
+    {
         ResTerm<T> t{};
         if (lane < warps) t = sh.part[w][lane];
         return t;
-    };
-    ResSums sums{};
-    sums.w = q.words + (size_t)(q.groups == 1 ? 0 : blk / q.bpc) * kResGroupWords;
-    sums.nb = nb;
-    double d_inv = 0.0;
-    bool d_plain = false;
-    if (lane == 0) sh.done = sh.halo_failed = 0;
-
-    // exchange 0: b.b (and r on the halo rows)
-    bar_sync_n(2, all);
+    }
+    __device__ __forceinline__ ResTerm<double> gather64(int w) const
     {
-        const ResTerm<T> mine[1] = {gather(0)};
-        double tot[1];
-        const bool got = res_totals<1, T>(sums, 0, mine, lane, tot);
-        sums.e[0] = 0;
-        if (!got) {
-            status = GMAF_TIMEOUT;
-            done = 1;
-        } else if (q.mode != kResRestart) {
-            normS = sqrt(tot[0]);
-            zero_rhs = tot[0] == 0.0;
-            if (!finite_d(tot[0])) {
-                status = GMAF_NONFINITE;
-                done = 1;
-            }
-        }
+        ResTerm<double> t{};
+        if (lane < warps) t = sh.part64[w][lane];
+        return t;
     }
-    // a little above (eps ||b||)^2, compared as integers (r.r is not negative)
-    const double thr = q.eps * normS;
-    const long long thr2 = __double_as_longlong(thr * thr * (1.0 + 1e-10));
-    if (lane == 0) {
-        sh.alpha = sh.beta = 0.0;
-        sh.done = done;
-    }
-    bar_sync_n(2, all);
 
-    bool init = true;
-    while (!done) {
-        // after z = M^-1 r
-        bar_sync_n(2, all);
-        {
-            const ResTerm<T> mine[2] = {gather(0), gather(1)};
-            double tot[2], beta = 0.0;
-            if (!res_totals<2, T>(sums, 1, mine, lane, tot) || sh.halo_failed) {
-                status = GMAF_TIMEOUT;
-                done = 1;
-            } else {
-                const double rz = tot[0], rr = tot[1];
-                rr_last = rr;
-                const bool fin = res_exp(rz) != 0x7ff && res_exp(rr) != 0x7ff;
-                if (!init) {
-                    ++iter;
-                    // rz / d: the reciprocal was formed while the product ran
-                    const double t = rz * d_inv;
-                    beta = d_plain ? fma(d_inv, fma(-d, t, rz), t) : rz / d;
-                } else if (q.mode == kResContinue) {
-                    // a continued recurrence: u = z + beta u', the old direction in the new units
-                    const double d_old = sc->d;
-                    if (fin && finite_d(d_old) && d_old > 0.0 && q.cscale > 0.0)
-                        beta = rz / (q.cscale * d_old);
-                }
-                if (zero_rhs) {
-                    converged = 1;
-                    done = 1;
-                } else if (!fin) {
-                    status = GMAF_NONFINITE;
-                    done = 1;
-                } else if (__double_as_longlong(rr) <= thr2 && sqrt(rr) / normS <= q.eps) {
-                    // (Eq. 3.9; the root and the quotient are formed only near the tolerance)
-                    converged = 1;
-                    done = 1;
-                } else if (iter >= q.max_iter) {
-                    done = 1;
-                }
-                if (init || !done) d = rz;
-                // loop guard: never more products than iterations (a host-set limit can lower it)
-                if (!init && guard > (q.guard_limit > 0 ? (long long)q.guard_limit
-                                                        : (long long)q.max_iter + 4)) {
+    // One PCG run from the residual that the row threads hold, to ||r|| <= eps normS or
+    // max_iter (of the running count).  cscale > 0: a continued recurrence (mixed
+    // precision), whose old direction is cscale times smaller in the new units.
+    __device__ __forceinline__ void run(double eps, int max_iter, double cscale)
+    {
+        const double thr = eps * normS;
+        // a little above (eps ||b||)^2, compared as integers (r.r is not negative)
+        const long long thr2 = __double_as_longlong(thr * thr * (1.0 + 1e-10));
+        double d_inv = 0.0;
+        bool d_plain = false, init = true;
+        int guard = 0;
+        while (!done) {
+            // after z = M^-1 r
+            bar_sync_n(2, all);
+            {
+                const ResTerm<T> mine[2] = {gather(0), gather(1)};
+                double tot[2], beta = 0.0;
+                if (!res_totals<2, T>(sums, 1, mine, lane, tot) || sh.halo_failed) {
                     status = GMAF_TIMEOUT;
                     done = 1;
+                } else {
+                    const double rz = tot[0], rr = tot[1];
+                    rr_last = rr;
+                    const bool fin = res_exp(rz) != 0x7ff && res_exp(rr) != 0x7ff;
+                    if (!init) {
+                        ++iter;
+                        // rz / d: the reciprocal was formed while the product ran
+                        const double t = rz * d_inv;
+                        beta = d_plain ? fma(d_inv, fma(-d, t, rz), t) : rz / d;
+                    } else if (cscale > 0.0) {
+                        // u = z + beta u', the old direction in the new units
+                        if (fin && finite_d(d) && d > 0.0) beta = rz / (cscale * d);
+                    }
+                    if (zero_rhs) {
+                        converged = 1;
+                        done = 1;
+                    } else if (!fin) {
+                        status = GMAF_NONFINITE;
+                        done = 1;
+                    } else if (__double_as_longlong(rr) <= thr2 && sqrt(rr) / normS <= eps) {
+                        // (Eq. 3.9; the root and the quotient are formed only near the tolerance)
+                        converged = 1;
+                        done = 1;
+                    } else if (iter >= max_iter) {
+                        done = 1;
+                    }
+                    if (init || !done) d = rz;
+                    // loop guard: never more products than iterations (a host-set limit can lower it)
+                    if (!init && guard > (q.guard_limit > 0 ? (long long)q.guard_limit
+                                                            : (long long)max_iter + 4)) {
+                        status = GMAF_TIMEOUT;
+                        done = 1;
+                    }
+                }
+                if (lane == 0) {
+                    sh.beta = beta;
+                    sh.done = done;
                 }
             }
-            if (lane == 0) {
-                sh.beta = beta;
-                sh.done = done;
-            }
-        }
-        mark(init ? 2 : 1);
-        if (timed && !init) q.times[4] += 1;
-        bar_sync_n(2, all);
-        if (done) break;
-        init = false;
-        d_inv = 1.0 / d;
-        d_plain = res_exp(d) > 100 && res_exp(d) < 1940;
+            mark(init ? 2 : 1);
+            if (timed && !init) q.times[4] += 1;
+            bar_sync_n(2, all);
+            if (done) break;
+            init = false;
+            d_inv = 1.0 / d;
+            d_plain = res_exp(d) > 100 && res_exp(d) < 1940;
 
-        // after v = A u
+            // after v = A u
+            bar_sync_n(2, all);
+            {
+                const ResTerm<T> mine[1] = {gather(0)};
+                double tot[1];
+                ++guard;
+                if (!res_totals<1, T>(sums, 0, mine, lane, tot) || sh.halo_failed) {
+                    status = GMAF_TIMEOUT;
+                    done = 1;
+                } else if (res_exp(tot[0]) == 0x7ff || __double_as_longlong(tot[0]) <= 0 ||
+                           res_exp(d) == 0x7ff) {
+                    status = GMAF_NONFINITE;
+                    done = 1;
+                } else {
+                    alpha = res_quotient(d, tot[0]);
+                }
+                if (lane == 0) {
+                    sh.alpha = alpha;
+                    sh.done = done;
+                }
+            }
+            mark(0);
+            if (timed) q.times[3] += 1;
+            bar_sync_n(2, all);
+        }
+    }
+
+    // FP64: one run (Table 1, or its restart).
+    __device__ __forceinline__ void solve(Scalars *sc)
+    {
+        iter = q.mode == kResRestart ? sc->iter : 0;
+        normS = q.mode == kResRestart ? sc->normS : 0.0;
+        // exchange 0: b.b (and r on the halo rows)
         bar_sync_n(2, all);
         {
             const ResTerm<T> mine[1] = {gather(0)};
             double tot[1];
-            ++guard;
-            if (!res_totals<1, T>(sums, 0, mine, lane, tot) || sh.halo_failed) {
+            const bool got = res_totals<1, T>(sums, 0, mine, lane, tot);
+            sums.e[0] = 0;
+            if (!got) {
                 status = GMAF_TIMEOUT;
                 done = 1;
-            } else if (res_exp(tot[0]) == 0x7ff || __double_as_longlong(tot[0]) <= 0 || res_exp(d) == 0x7ff) {
-                status = GMAF_NONFINITE;
-                done = 1;
-            } else {
-                alpha = res_quotient(d, tot[0]);
-            }
-            if (lane == 0) {
-                sh.alpha = alpha;
-                sh.done = done;
+            } else if (q.mode != kResRestart) {
+                normS = sqrt(tot[0]);
+                zero_rhs = tot[0] == 0.0;
+                if (!finite_d(tot[0])) {
+                    status = GMAF_NONFINITE;
+                    done = 1;
+                }
             }
         }
-        mark(0);
-        if (timed) q.times[3] += 1;
+        if (lane == 0) {
+            sh.alpha = sh.beta = 0.0;
+            sh.done = done;
+        }
         bar_sync_n(2, all);
+        run(q.eps, q.max_iter, 0.0);
     }
-    if (lane == 0 && blk == g0) {
-        sc->iter = iter;
-        sc->d = d;
-        sc->normS = normS;
-        sc->rel = sqrt(rr_last) / normS;
-        sc->alpha = alpha;
-        sc->converged = converged;
-        sc->status = status;
-        sc->zero_rhs = zero_rhs;
-        sc->pending = 0;
-        sc->done = 1;
+
+    // Mixed precision: FP64 refinement around the FP32 run (the loop of solve_joint_device).
+    __device__ __forceinline__ void refine(Scalars *sc)
+    {
+        const double scale = *q.scale;
+        int total = 0, outer = 0, longest = 0, last_iter = 0, verdict = GMAF_NOT_CONVERGED;
+        bool stalled = false, stop = false;
+        double rnorm_prev = 0.0, true_rel = 0.0;
+        for (;;) {
+            // after r64 = S - A p64
+            bar_sync_n(2, all);
+            double cscale = 0.0, eps_in = 0.5, rnorm = 0.0;
+            int max_iter = 0;
+            {
+                const ResTerm<double> mine[2] = {gather64(0), gather64(1)};
+                double tot[2];
+                if (!res_totals<2, double>(sums, 2, mine, lane, tot) || sh.halo_failed) {
+                    verdict = GMAF_TIMEOUT;
+                    stop = true;
+                } else {
+                    rnorm = sqrt(tot[0]);
+                    const double nS = sqrt(tot[1]);
+                    true_rel = nS > 0.0 ? rnorm / nS : 0.0;
+                    if (!finite_d(tot[0]) || !finite_d(tot[1]) || !finite_d(true_rel)) {
+                        verdict = GMAF_NONFINITE;
+                        stop = true;
+                    } else if (nS == 0.0 || true_rel <= q.eps) {
+                        verdict = GMAF_OK;
+                        stop = true;
+                    } else if (stop || outer >= q.max_outer || total >= q.max_iter) {
+                        stop = true;
+                    } else {
+                        // a fixed reduction, but no further than the outer target needs
+                        eps_in = fmin(fmax(0.5 * q.eps / true_rel, q.inner_floor), 0.5);
+                        const bool cont = outer > 0 && q.continued && rnorm_prev > 0.0 && !stalled;
+                        // a continued run that needs more than max(1000, 4 x the longest so
+                        // far) is cut off, and the next one restarts from its residual
+                        const int left = q.max_iter - total, cap = max(1000, 4 * longest);
+                        if (!cont) iter = last_iter = 0;
+                        max_iter = cont ? last_iter + min(left, cap) : left;
+                        cscale = cont ? rnorm_prev / rnorm : 0.0;
+                        rnorm_prev = rnorm;
+                    }
+                }
+            }
+            done = status = converged = 0;
+            normS = 1.0;                // b is r64 / ||r64||
+            if (lane == 0) {
+                sh.alpha = sh.beta = 0.0;
+                sh.unit = 1.0 / rnorm;
+                sh.back = scale * rnorm;
+                sh.done = 0;
+                sh.stop = stop;
+            }
+            mark(5);
+            if (timed) q.times[6] += 1;
+            bar_sync_n(2, all);
+            if (stop) break;
+            // the scales of the sums change with the units
+            if (cscale == 0.0) sums.e[0] = sums.e[1] = sums.e[2] = 0;
+            run(eps_in, max_iter, cscale);
+            const int seg = iter - last_iter;
+            last_iter = iter;
+            total += seg;
+            longest = max(longest, seg);
+            stalled = q.continued && !converged;
+            ++outer;
+            if (status != 0) verdict = status;
+            stop = status != 0 || seg == 0;     // (the row threads still add x to p)
+            if (stop) {
+                bar_sync_n(2, all);             // the residual's sums: not wanted
+                if (lane == 0) sh.stop = 1;
+                bar_sync_n(2, all);
+                break;
+            }
+        }
+        if (lane == 0 && blockIdx.x == 0) {
+            sc->iter = total;
+            sc->guard = outer;
+            sc->status = verdict;
+            sc->true_rel = true_rel;
+        }
+    }
+};
+
+template <typename T>
+__device__ __forceinline__ void res_exchange_warp(const ResParams<T> &q, ResShared<T> &sh, Scalars *sc,
+                                                  int grp, int g0, int nb, int lane)
+{
+    ResExchange<T> x{q, sh, q.threads + 32, q.threads / 32, lane};
+    x.sums = ResSums{};
+    x.sums.w = q.words + (size_t)grp * kResGroupWords;
+    x.sums.nb = nb;
+    x.iter = x.status = x.converged = x.zero_rhs = x.done = 0;
+    x.d = x.normS = x.rr_last = x.alpha = 0.0;
+    x.timed = q.times != nullptr && lane == 0 && blockIdx.x == 0;
+    x.t_mark = x.timed ? res_time() : 0ull;
+    if (lane == 0) sh.done = sh.stop = sh.halo_failed = 0;
+    if constexpr (sizeof(T) == 4) {
+        x.refine(sc);
+    } else {
+        x.solve(sc);
+        if (lane == 0 && (int)blockIdx.x == g0) {
+            sc->iter = x.iter;
+            sc->d = x.d;
+            sc->normS = x.normS;
+            sc->rel = sqrt(x.rr_last) / x.normS;
+            sc->alpha = x.alpha;
+            sc->converged = x.converged;
+            sc->status = x.status;
+            sc->zero_rhs = x.zero_rhs;
+            sc->pending = 0;
+            sc->done = 1;
+        }
     }
 }
 
@@ -635,30 +780,228 @@ struct ResAcc<float> {
 template <typename T>
 using ResSum = decltype(ResAcc<T>{}.value());
 
+// What a thread that owns rows works on.  Built anew for each part of a mixed-precision
+// solve, and set-up and residual are not inlined: the iterations would otherwise pay
+// registers for values that live across them.
 // CS: the coefficients in shared memory (else read from global memory, i.e. L2).
 template <typename T, int VEC, int RR, bool CS>
-__global__ void __launch_bounds__(kResThreads + 32, 1) k_resident(const __grid_constant__ ResParams<T> q)
+struct ResRows {
+    using V = Vec<T, VEC>;
+    static constexpr int S = kResThreads * VEC;     // private fields: [row][thread][VEC]
+    static constexpr int NS = kResSegs;
+    static constexpr bool RS = res_r_shared(RR, VEC, sizeof(T));
+    static constexpr bool kMixed = sizeof(T) == 4;  // FP32 runs inside FP64 refinement
+    static constexpr int FE = RR * S, FN = 2 * RR * S, FI = 3 * RR * S, FD = 4 * RR * S;
+    static constexpr int FR = CS ? 5 * RR * S : RR * S;
+
+    const ResParams<T> &q;
+    ResShared<T> &sh;
+    int nth, nz, TC, all, tid, lane, wid;
+    int j0, run, cg, c, lr0, nr;                    // the block's first row; first local row and rows of the run
+    bool act, top, hasS, hasN;                      // rows at all; the block's last rows; a block below, above
+    bool segw, sege, atw, ate, last;                // edges of a segment, of the row; the run ends at row nz - 1
+    size_t off, coff;                               // first cell in the fields, in the coefficient slots
+    // shared memory: private fields (u, coefficients, r), then rows and edges
+    T *P;                                           // u: P[rr * S]
+    T *HU, *HR, *HI;                                // [2][nth] u, r, omega/D on the halo rows
+    T *HE;                                          // [nth] aE on the north halo row
+    T *YR, *WR;                                     // [nrr][nth] y south of each run, [nrr - 1][nth] w north
+    // edges of a row's segments of 32 threads, [rows + 1][NS]: last y, last aE, first w (own,
+    // of the west and of the east segment); [rows + 1][2] y of column 0 and w of column nth - 1
+    T *EY, *EYl, *EWr, *EC;
+    int er;
+    const T *pS, *pN, *pW, *pE;                     // u beyond the run's rows and the warp's columns
+    T *pX;
+    int stX;
+    // rows of a block's halo area: 0, 1 = first and last row of v; 2, 3 = of z
+    unsigned long long *halo;
+
+    __device__ __forceinline__ ResRows(const ResParams<T> &q_, ResShared<T> &sh_) : q(q_), sh(sh_)
+    {
+        extern __shared__ __align__(16) unsigned char g_res_smem[];
+        nth = q.nth;
+        nz = q.nz;
+        TC = q.threads;
+        all = TC + 32;
+        // (volatile: formed anew where it is used, not kept in registers across refinements)
+        asm volatile("mov.u32 %0, %%tid.x;\n" : "=r"(tid));
+        lane = tid & 31;
+        wid = tid >> 5;
+        const int cond = blockIdx.x / q.bpc, bc = blockIdx.x - cond * q.bpc;
+        j0 = (int)((long long)bc * nz / q.bpc);
+        const int j1 = (int)((long long)(bc + 1) * nz / q.bpc), R = j1 - j0;
+        run = tid / q.P;
+        cg = tid - run * q.P;
+        c = cg * VEC;
+        lr0 = run * RR;
+        nr = R - lr0;
+        nr = cg >= q.ncg || nr < 0 ? 0 : (nr > RR ? RR : nr);
+        act = nr > 0;
+        top = act && lr0 + nr == R;
+        hasS = act && run == 0 && j0 > 0;
+        hasN = top && j1 < nz;
+        segw = (cg & 31) == 0;
+        sege = (cg & 31) == 31 || cg == q.ncg - 1;
+        atw = cg == 0;
+        ate = cg == q.ncg - 1;
+        last = top && j1 == nz;
+        off = (size_t)cond * (size_t)q.n + (size_t)(j0 + lr0) * nth + c;
+        coff = (size_t)q.cslot[cond] * (size_t)q.n + (size_t)(j0 + lr0) * nth + c;
+        T *const sm = reinterpret_cast<T *>(g_res_smem);
+        P = sm + tid * VEC;
+        HU = reinterpret_cast<T *>(g_res_smem + q.o_rows);
+        HR = HU + 2 * nth;
+        HI = HR + 2 * nth;
+        HE = HI + 2 * nth;
+        YR = HE + nth;
+        WR = YR + q.nrr * nth;
+        T *const edge = reinterpret_cast<T *>(g_res_smem + q.o_edge);
+        er = (q.rows + 1) * NS;
+        EY = edge + lr0 * NS + (cg >> 5);
+        EYl = edge + lr0 * NS + (atw ? (q.ncg - 1) >> 5 : (cg >> 5) - 1);
+        EWr = edge + 2 * er + lr0 * NS + (ate ? 0 : (cg >> 5) + 1);
+        EC = edge + 3 * er + 2 * lr0;
+        pS = run == 0 ? HU + c : P - q.P * VEC + (RR - 1) * S;
+        pN = top ? HU + nth + c : P + q.P * VEC;
+        pW = sm + (run * q.P + (atw ? q.ncg - 1 : cg - 1)) * VEC + VEC - 1;
+        pE = sm + (run * q.P + (ate ? 0 : cg + 1)) * VEC;
+        pX = q.o_x >= 0 ? reinterpret_cast<T *>(g_res_smem + q.o_x) + tid * VEC : q.p + off;
+        stX = q.o_x >= 0 ? S : nth;
+        halo = q.halo + (size_t)blockIdx.x * 4 * q.halo_row + c * ((int)sizeof(T) / 4);
+    }
+
+    __device__ __forceinline__ void get_E(int rr, T (&x)[VEC]) const
+    {
+        V::ldrw(CS ? P + FE + rr * S : q.aE + coff + (size_t)rr * nth, x);
+    }
+    __device__ __forceinline__ void get_N(int rr, T (&x)[VEC]) const
+    {
+        V::ldrw(CS ? P + FN + rr * S : q.aN + coff + (size_t)rr * nth, x);
+    }
+    __device__ __forceinline__ void get_I(int rr, T (&x)[VEC]) const
+    {
+        V::ldrw(CS ? P + FI + rr * S : q.invD + coff + (size_t)rr * nth, x);
+    }
+    __device__ __forceinline__ void get_D(int rr, T (&x)[VEC]) const
+    {
+        V::ldrw(CS ? P + FD + rr * S : q.D + coff + (size_t)rr * nth, x);
+    }
+
+    // The coefficients, and zeros for u and where no block lies beyond.
+    __device__ __forceinline__ void setup()
+    {
+        for (int i = tid; i < 2 * nth; i += TC) HU[i] = HR[i] = T(0);
+        for (int i = tid; i < nth; i += TC) YR[i] = T(0);
+        bar_sync_n(1, TC);
+#pragma unroll
+        for (int rr = 0; rr < RR; ++rr) {
+            const size_t go = (size_t)rr * nth;
+            const bool in = rr < nr;
+            T t[VEC], zero[VEC];
+#pragma unroll
+            for (int e = 0; e < VEC; ++e) t[e] = zero[e] = T(0);
+            V::st(P + rr * S, zero);
+            if (in) V::ldrw(q.aE + coff + go, t);
+            if (CS) V::st(P + FE + rr * S, t);
+            if (in && sege) EY[er + rr * NS] = t[VEC - 1];
+            if (CS) {
+                // (a_N of the last row is not read: it couples to nothing)
+                if (in && !(last && rr == nr - 1)) V::ldrw(q.aN + coff + go, t);
+                V::st(P + FN + rr * S, in && !(last && rr == nr - 1) ? t : zero);
+                if (in) V::ldrw(q.invD + coff + go, t);
+                V::st(P + FI + rr * S, in ? t : zero);
+                if (in) V::ldrw(q.D + coff + go, t);
+                V::st(P + FD + rr * S, in ? t : zero);
+            }
+        }
+        if (!act) return;
+        T t[VEC];
+        if (hasS) {
+            V::ldrw(q.invD + coff - nth, t);
+            V::st(HI + c, t);
+        }
+        if (hasN) {
+            V::ldrw(q.invD + coff + (size_t)nr * nth, t);
+            V::st(HI + nth + c, t);
+            V::ldrw(q.aE + coff + (size_t)nr * nth, t);
+            V::st(HE + c, t);
+            if (sege) EY[er + nr * NS] = t[VEC - 1];
+        }
+    }
+
+    // Mixed precision: this thread's rows of r64 = S - A p64, and the warps' sums of r64 r64 and
+    // S S.  The rows of the blocks below and above come as flagged words.
+    __device__ __forceinline__ void residual(unsigned ep)
+    {
+        double *const p64 = q.p64 + off;
+        unsigned long long *const row64 = q.halo64 + ((size_t)blockIdx.x * 2 * nth + c) * 2;
+        double pS64[VEC], pN64[VEC], rr = 0.0, ss = 0.0;
+        if (hasS) {
+#pragma unroll
+            for (int e = 0; e < VEC; ++e) pS64[e] = p64[e];
+            ll_put<VEC>(row64, pS64, ep);
+        }
+        if (hasN) {
+#pragma unroll
+            for (int e = 0; e < VEC; ++e) pN64[e] = p64[(size_t)(nr - 1) * nth + e];
+            ll_put<VEC>(row64 + 2 * nth, pN64, ep);
+        }
+        bar_sync_n(1, TC);                          // p64 of the block's other threads
+#pragma unroll
+        for (int e = 0; e < VEC; ++e) pS64[e] = pN64[e] = 0.0;
+        bool ok = true;
+        if (hasS) ok = ll_get<VEC>(row64 - 2 * nth, pS64, ep);
+        if (hasN) ok = ll_get<VEC>(row64 + 4 * nth, pN64, ep) && ok;
+        if (!ok) sh.halo_failed = 1;
+#pragma unroll 1
+        for (int k = 0; k < nr; ++k) {
+            const int j = j0 + lr0 + k;
+            const size_t go = (size_t)k * nth;
+            const double *p = p64 + go, *aE = q.aE64 + coff + go, *aN = q.aN64 + coff + go;
+#pragma unroll
+            for (int e = 0; e < VEC; ++e) {
+                const int ie = c + e == nth - 1 ? 1 - nth + e : e + 1, iw = c + e == 0 ? nth - 1 : e - 1;
+                double ap = q.D64[coff + go + e] * p[e] - aE[e] * p[ie] - aE[iw] * p[iw];
+                if (j < nz - 1) ap -= aN[e] * (hasN && k == nr - 1 ? pN64[e] : p[nth + e]);
+                if (j > 0) ap -= aN[e - nth] * (hasS && k == 0 ? pS64[e] : p[e - nth]);
+                const double s = q.S64[off + go + e], rv = s - ap;
+                q.r64[off + go + e] = rv;
+                rr = fma(rv, rv, rr);
+                ss = fma(s, s, ss);
+            }
+        }
+        const double x[2] = {rr, ss};
+        ResTerm<double> t[2];
+        res_warp_sums<2>(x, t);
+        if (lane == 0) {
+            sh.part64[0][wid] = t[0];
+            sh.part64[1][wid] = t[1];
+        }
+    }
+};
+
+// One PCG run: the start (ep: the last exchange's number), the iterations, the result.
+// Returns the last exchange's number.
+//
+// Every thread computes all RR rows: rows and threads beyond the block's have zero
+// coefficients and only their stores are left out, so that the rows of a run are
+// independent straight-line code.
+template <typename T, int VEC, int RR, bool CS>
+__device__ __forceinline__ unsigned res_iterate(const ResParams<T> &q, ResShared<T> &sh, unsigned ep)
 {
     using V = Vec<T, VEC>;
     constexpr int S = kResThreads * VEC;            // private fields: [row][thread][VEC]
     constexpr int NS = kResSegs;
     constexpr bool RS = res_r_shared(RR, VEC, sizeof(T));
+    constexpr bool kMixed = sizeof(T) == 4;         // FP32 runs inside FP64 refinement
     constexpr int FE = RR * S, FN = 2 * RR * S, FI = 3 * RR * S, FD = 4 * RR * S;
     constexpr int FR = CS ? 5 * RR * S : RR * S;
     extern __shared__ __align__(16) unsigned char g_res_smem[];
-    __shared__ ResShared<T> sh;
-    const int nth = q.nth, nz = q.nz;
+    const int nth = q.nth, nz = q.nz, TC = q.threads, all = TC + 32;
+    int tid;
+    asm volatile("mov.u32 %0, %%tid.x;\n" : "=r"(tid));
+    const int lane = tid & 31, wid = tid >> 5;
     const int cond = blockIdx.x / q.bpc, bc = blockIdx.x - cond * q.bpc;
-    const int grp = q.groups == 1 ? 0 : cond;
-    if (!((q.mask >> grp) & 1ull)) return;                 // this group does not run
-    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    const int TC = q.threads;                               // threads that own rows
-    if (tid >= TC) {
-        res_exchange_warp<T>(q, sh, q.sc + grp, q.groups == 1 ? 0 : cond * q.bpc,
-                             q.groups == 1 ? (int)gridDim.x : q.bpc, lane);
-        return;
-    }
-    const int all = TC + 32;
     const int j0 = (int)((long long)bc * nz / q.bpc), j1 = (int)((long long)(bc + 1) * nz / q.bpc);
     const int R = j1 - j0;
     const bool assor = q.precond == 1;
@@ -669,13 +1012,14 @@ __global__ void __launch_bounds__(kResThreads + 32, 1) k_resident(const __grid_c
     int nr = R - lr0;
     nr = cg >= q.ncg || nr < 0 ? 0 : (nr > RR ? RR : nr);
     const bool act = nr > 0;
-    const bool bot = act && run == 0, top = act && lr0 + nr == R;
-    const bool hasS = bot && j0 > 0, hasN = top && j1 < nz;    // a block below, above
+    const bool top = act && lr0 + nr == R;
+    const bool hasS = act && run == 0 && j0 > 0, hasN = top && j1 < nz;    // a block below, above
     const bool segw = (cg & 31) == 0, sege = (cg & 31) == 31 || cg == q.ncg - 1;
     const bool atw = cg == 0, ate = cg == q.ncg - 1;
     const bool last = top && j1 == nz;                      // this run ends at row nz - 1
-    const size_t off = (size_t)cond * (size_t)q.n + (size_t)(j0 + lr0) * nth + c;
-    const size_t coff = (size_t)q.cslot[cond] * (size_t)q.n + (size_t)(j0 + lr0) * nth + c;
+    // (whatever fits on the SMs has less than 2^32 cells)
+    const unsigned off = (unsigned)cond * (unsigned)q.n + (unsigned)((j0 + lr0) * nth + c);
+    const unsigned coff = (unsigned)q.cslot[cond] * (unsigned)q.n + (unsigned)((j0 + lr0) * nth + c);
 
     // ---- shared memory: private fields (u, coefficients, r), then rows and edges
     T *const sm = reinterpret_cast<T *>(g_res_smem);
@@ -695,22 +1039,38 @@ __global__ void __launch_bounds__(kResThreads + 32, 1) k_resident(const __grid_c
     // y of column 0 and w of column nth - 1: [rows + 1][2] behind them
     T *const EC = edge + 3 * er + 2 * lr0;
     // u of the rows beyond the run and of the threads beyond the warp
-    const T *const pS = run == 0 ? HU + c : P - q.P * VEC + (RR - 1) * S;
-    const T *const pN = top ? HU + nth + c : P + q.P * VEC;
+    const T *const pS = !act ? P : run == 0 ? HU + c : P - q.P * VEC + (RR - 1) * S;
+    const T *const pN = !act ? P : top ? HU + nth + c : P + q.P * VEC;
     const T *const pW = sm + (run * q.P + (atw ? q.ncg - 1 : cg - 1)) * VEC + VEC - 1;
     const T *const pE = sm + (run * q.P + (ate ? 0 : cg + 1)) * VEC;
     T *const pX = q.o_x >= 0 ? reinterpret_cast<T *>(g_res_smem + q.o_x) + tid * VEC : q.p + off;
     const int stX = q.o_x >= 0 ? S : nth;
 
-    auto get_E = [&](int rr, T(&x)[VEC]) { V::ldrw(CS ? P + FE + rr * S : q.aE + coff + (size_t)rr * nth, x); };
-    auto get_N = [&](int rr, T(&x)[VEC]) { V::ldrw(CS ? P + FN + rr * S : q.aN + coff + (size_t)rr * nth, x); };
-    auto get_I = [&](int rr, T(&x)[VEC]) { V::ldrw(CS ? P + FI + rr * S : q.invD + coff + (size_t)rr * nth, x); };
-    auto get_D = [&](int rr, T(&x)[VEC]) { V::ldrw(CS ? P + FD + rr * S : q.D + coff + (size_t)rr * nth, x); };
+    // a row's coefficients; in global memory rows beyond the block's read the last one's place
+    const int most = nr > 0 ? nr - 1 : 0;
+    const unsigned cat = act ? coff : (unsigned)q.cslot[cond] * (unsigned)q.n;
+    auto coef = [&](int field, const T *g, int rr, T(&x)[VEC]) {
+        if constexpr (CS) {
+            V::ldrw(P + field + rr * S, x);
+        } else {
+            V::ldrw(g + (cat + (unsigned)(min(rr, most) * nth)), x);
+            const bool none = rr >= nr || (field == FN && last && rr == nr - 1);
+#pragma unroll
+            for (int e = 0; e < VEC; ++e) x[e] = none ? T(0) : x[e];
+        }
+    };
+    auto get_E = [&](int rr, T(&x)[VEC]) { coef(FE, q.aE, rr, x); };
+    auto get_N = [&](int rr, T(&x)[VEC]) { coef(FN, q.aN, rr, x); };
+    auto get_I = [&](int rr, T(&x)[VEC]) { coef(FI, q.invD, rr, x); };
+    auto get_D = [&](int rr, T(&x)[VEC]) { coef(FD, q.D, rr, x); };
+
+    // (the longest runs: no loads of one row moved across another, there are no registers for it)
+    auto row_end = [] {
+        if constexpr (RS) asm volatile("" ::: "memory");
+    };
 
     // rows of a block's halo area: 0, 1 = first and last row of v; 2, 3 = of z
     unsigned long long *const halo = q.halo + (size_t)blockIdx.x * 4 * q.halo_row + c * ((int)sizeof(T) / 4);
-    unsigned ep = q.epoch;
-
     T rg[RS ? 1 : RR][VEC], vz[RR][VEC], aS0[VEC], hS[VEC], hN[VEC];
     auto r_get = [&](int rr, T(&x)[VEC]) {
         if constexpr (RS) {
@@ -761,45 +1121,56 @@ __global__ void __launch_bounds__(kResThreads + 32, 1) k_resident(const __grid_c
         if (!ok) sh.halo_failed = 1;
     };
 
-    // ---- set-up: coefficients, r, x, u
-    for (int i = tid; i < 2 * nth; i += TC) HU[i] = HR[i] = T(0);
-    for (int i = tid; i < nth; i += TC) YR[i] = T(0);
-    bar_sync_n(1, TC);
-    ResAcc<T> acc0;
-    if (act) {
+    if (j0 + lr0 > 0 && act) V::ldrw(q.aN + coff - nth, aS0);
+    if constexpr (kMixed) {
+        // b = r64 / ||r64||, x = 0
+        const double unit = sh.unit;
+        ++ep;
 #pragma unroll
         for (int rr = 0; rr < RR; ++rr) {
-            if (rr >= nr) continue;
-            const size_t go = (size_t)rr * nth;
-            T t[VEC];
-            V::ldrw(q.aE + coff + go, t);
-            if (CS) V::st(P + FE + rr * S, t);
-            if (sege) EY[er + rr * NS] = t[VEC - 1];
-            if (CS) {
-                V::ldrw(q.aN + coff + go, t);
-                V::st(P + FN + rr * S, t);
-                V::ldrw(q.invD + coff + go, t);
-                V::st(P + FI + rr * S, t);
-                V::ldrw(q.D + coff + go, t);
-                V::st(P + FD + rr * S, t);
+            T r[VEC], x[VEC];
+#pragma unroll
+            for (int e = 0; e < VEC; ++e) {
+                r[e] = rr < nr ? (T)(q.r64[off + (size_t)rr * nth + e] * unit) : T(0);
+                x[e] = T(0);
             }
-            // r = b (- A p), or the residual handed in; x = 0 or p
+            r_put(rr, r);
+            if (q.o_x >= 0 || rr < nr) V::st(pX + rr * stX, x);
+            if (hasS && rr == 0) ll_put<VEC>(halo, r, ep);
+            if (hasN && rr == nr - 1) ll_put<VEC>(halo + q.halo_row, r, ep);
+            asm volatile("" ::: "memory");      // (one row's doubles in registers at a time)
+        }
+        fetch(1, 0);
+    } else {
+        // r = b (- A p), or the residual handed in; x = 0 or p; exchange 0: b.b, and r on the
+        // halo rows
+        ResAcc<T> acc;
+        ++ep;
+#pragma unroll
+        for (int rr = 0; rr < RR; ++rr) {
+            const size_t go = (size_t)rr * nth;
             T x[VEC], r[VEC];
 #pragma unroll
-            for (int e = 0; e < VEC; ++e) x[e] = T(0);
+            for (int e = 0; e < VEC; ++e) x[e] = r[e] = T(0);
+            if (rr >= nr) {
+                r_put(rr, r);
+                if (q.o_x >= 0) V::st(pX + rr * stX, x);
+                continue;
+            }
             if (q.mode == kResRestart) {
                 V::ldrw(q.r_in + off + go, r);
                 V::ldrw(q.p + off + go, x);
             } else {
                 V::ldrw(q.b + off + go, r);
-                acc0.add(r, r);
+                acc.add(r, r);
                 if (!q.zero_init) {
                     V::ldrw(q.p + off + go, x);
                     const int j = j0 + lr0 + rr;
                     const T *p = q.p + off + go, *aE = q.aE + coff + go, *aN = q.aN + coff + go;
 #pragma unroll
                     for (int e = 0; e < VEC; ++e) {
-                        const int ie = c + e == nth - 1 ? 1 - nth + e : e + 1, iw = c + e == 0 ? nth - 1 : e - 1;
+                        const int ie = c + e == nth - 1 ? 1 - nth + e : e + 1;
+                        const int iw = c + e == 0 ? nth - 1 : e - 1;
                         T ap = q.D[coff + go + e] * x[e] - aE[e] * p[ie] - aE[iw] * p[iw];
                         if (j < nz - 1) ap -= aN[e] * p[nth + e];
                         if (j > 0) ap -= aN[e - nth] * p[e - nth];
@@ -810,44 +1181,14 @@ __global__ void __launch_bounds__(kResThreads + 32, 1) k_resident(const __grid_c
             r_put(rr, r);
             // (in global memory p itself is x, and a neighbour may still be reading it)
             if (q.o_x >= 0 || (q.mode != kResRestart && q.zero_init)) V::st(pX + rr * stX, x);
-#pragma unroll
-            for (int e = 0; e < VEC; ++e) t[e] = T(0);
-            if (q.mode == kResContinue) V::ldrw(q.u + off + go, t);
-            V::st(P + rr * S, t);
             // the rows that the neighbours keep a copy of
-            if (hasS && rr == 0) ll_put<VEC>(halo, r, ep + 1);
-            if (hasN && rr == nr - 1) ll_put<VEC>(halo + q.halo_row, r, ep + 1);
+            if (hasS && rr == 0) ll_put<VEC>(halo, r, ep);
+            if (hasN && rr == nr - 1) ll_put<VEC>(halo + q.halo_row, r, ep);
         }
-        if (j0 + lr0 > 0) V::ldrw(q.aN + coff - nth, aS0);
-        if (hasS) {
-            T t[VEC];
-            V::ldrw(q.invD + coff - nth, t);
-            V::st(HI + c, t);
-            if (q.mode == kResContinue) {
-                V::ldrw(q.u + off - nth, t);
-                V::st(HU + c, t);
-            }
-        }
-        if (hasN) {
-            T t[VEC];
-            const size_t go = (size_t)nr * nth;
-            V::ldrw(q.invD + coff + go, t);
-            V::st(HI + nth + c, t);
-            V::ldrw(q.aE + coff + go, t);
-            V::st(HE + c, t);
-            if (sege) EY[er + nr * NS] = t[VEC - 1];
-            if (q.mode == kResContinue) {
-                V::ldrw(q.u + off + go, t);
-                V::st(HU + nth + c, t);
-            }
-        }
+        publish(acc.value());
+        fetch(1, 0);
+        bar_sync_n(2, all);
     }
-
-    // exchange 0: b.b, and r on the halo rows
-    publish(acc0.value());
-    ++ep;
-    fetch(1, 0);
-    bar_sync_n(2, all);
 
     bool init = true;
     while (!sh.done) {
@@ -860,7 +1201,6 @@ __global__ void __launch_bounds__(kResThreads + 32, 1) k_resident(const __grid_c
         for (int e = 0; e < VEC; ++e) yN[e] = T(0);
 #pragma unroll
         for (int rr = 0; rr < RR; ++rr) {
-            if (rr >= nr) continue;
             T od[VEC], r[VEC];
             get_I(rr, od);
             r_get(rr, r);
@@ -870,9 +1210,10 @@ __global__ void __launch_bounds__(kResThreads + 32, 1) k_resident(const __grid_c
                 vz[rr][e] = r[e] * od[e];
             }
             r_put(rr, r);
-            if (rr == RR - 1 && !top) V::st(YR + (run + 1) * nth + c, vz[rr]);
-            if (sege) EY[rr * NS] = vz[rr][VEC - 1];
-            if (atw) EC[2 * rr] = vz[rr][0];
+            if (rr == RR - 1 && act && !top) V::st(YR + (run + 1) * nth + c, vz[rr]);
+            if (sege && rr < nr) EY[rr * NS] = vz[rr][VEC - 1];
+            if (atw && rr < nr) EC[2 * rr] = vz[rr][0];
+            row_end();
         }
         if (hasS) {
             T h[VEC], od[VEC];
@@ -909,39 +1250,34 @@ __global__ void __launch_bounds__(kResThreads + 32, 1) k_resident(const __grid_c
             if (act) V::ldrw(YR + run * nth + c, yp);
 #pragma unroll
             for (int rr = 0; rr < RR; ++rr) {
-                T ev[VEC];
-#pragma unroll
-                for (int e = 0; e < VEC; ++e) ev[e] = T(0);
-                if (rr < nr) get_E(rr, ev);
+                const bool in = rr < nr;
+                T ev[VEC], od[VEC], nv[VEC], w[VEC];
+                get_E(rr, ev);
+                get_I(rr, od);
+                get_N(rr, nv);
                 T yW = __shfl_up_sync(0xffffffffu, vz[rr][VEC - 1], 1);
                 T aW = __shfl_up_sync(0xffffffffu, ev[VEC - 1], 1);
-                if (rr < nr) {
-                    if (segw && !atw) {
-                        yW = EYl[rr * NS];
-                        aW = EYl[er + rr * NS];
-                    }
-                    T w[VEC], od[VEC];
-                    get_I(rr, od);
-#pragma unroll
-                    for (int e = 0; e < VEC; ++e) {
-                        T sum = nS[e] * yp[e];
-                        if (e > 0)
-                            sum += ev[e - 1] * vz[rr][e - 1];
-                        else if (!atw)
-                            sum += aW * yW;
-                        if (e == VEC - 1 && ate) sum += ev[e] * EC[2 * rr];
-                        w[e] = vz[rr][e] + od[e] * sum;
-                    }
-                    if (rr == 0 && run > 0) V::st(WR + (run - 1) * nth + c, w);
-                    if (segw) EY[2 * er + rr * NS] = w[0];
-                    if (ate) EC[2 * rr + 1] = w[VEC - 1];
-                    get_N(rr, nS);
-#pragma unroll
-                    for (int e = 0; e < VEC; ++e) {
-                        yp[e] = vz[rr][e];
-                        vz[rr][e] = w[e];
-                    }
+                if (segw) {
+                    yW = in && !atw ? EYl[rr * NS] : T(0);
+                    aW = in && !atw ? EYl[er + rr * NS] : T(0);
                 }
+#pragma unroll
+                for (int e = 0; e < VEC; ++e) {
+                    T sum = nS[e] * yp[e];
+                    sum += (e > 0 ? ev[e - 1] : aW) * (e > 0 ? vz[rr][e - 1] : yW);
+                    if (e == VEC - 1 && ate && in) sum += ev[e] * EC[2 * rr];
+                    w[e] = vz[rr][e] + od[e] * sum;
+                }
+                if (rr == 0 && act && run > 0) V::st(WR + (run - 1) * nth + c, w);
+                if (segw && in) EY[2 * er + rr * NS] = w[0];
+                if (ate && in) EC[2 * rr + 1] = w[VEC - 1];
+#pragma unroll
+                for (int e = 0; e < VEC; ++e) {
+                    yp[e] = in ? vz[rr][e] : yp[e];
+                    nS[e] = in ? nv[e] : nS[e];
+                    vz[rr][e] = w[e];
+                }
+                row_end();
             }
             // w on the row above the block, for z of its last row
             {
@@ -975,40 +1311,36 @@ __global__ void __launch_bounds__(kResThreads + 32, 1) k_resident(const __grid_c
             if (act && !top) V::ldrw(WR + run * nth + c, wN);
 #pragma unroll
             for (int rr = RR - 1; rr >= 0; --rr) {
+                const bool in = rr < nr;
+                T ev[VEC], od[VEC], nv[VEC], z[VEC], r[VEC];
+                r_get(rr, r);
+                get_E(rr, ev);
+                get_I(rr, od);
+                get_N(rr, nv);
                 T wE = __shfl_down_sync(0xffffffffu, vz[rr][0], 1);
-                if (rr < nr) {
-                    T ev[VEC], od[VEC], nv[VEC], z[VEC], r[VEC];
-                    r_get(rr, r);
-                    get_E(rr, ev);
-                    get_I(rr, od);
-                    get_N(rr, nv);
-                    if (sege && !ate) wE = EWr[rr * NS];
-                    const bool north = !(last && rr == nr - 1);
+                if (sege) wE = in && !ate ? EWr[rr * NS] : T(0);
 #pragma unroll
-                    for (int e = 0; e < VEC; ++e) {
-                        T sum = north ? nv[e] * wN[e] : T(0);
-                        if (e < VEC - 1)
-                            sum += ev[e] * vz[rr][e + 1];
-                        else if (!ate)
-                            sum += ev[e] * wE;
-                        if (e == 0 && atw) sum += EYl[er + rr * NS] * EC[2 * rr + 1];
-                        z[e] = vz[rr][e] + od[e] * sum;
-                    }
-#pragma unroll
-                    for (int e = 0; e < VEC; ++e) {
-                        wN[e] = vz[rr][e];
-                        vz[rr][e] = z[e];
-                    }
-                    if (hasS && rr == 0) ll_put<VEC>(halo + 2 * q.halo_row, z, ep);
-                    if (hasN && rr == nr - 1) ll_put<VEC>(halo + 3 * q.halo_row, z, ep);
-                    arz.add(r, z);
-                    arr.add(r, r);
+                for (int e = 0; e < VEC; ++e) {
+                    T sum = nv[e] * wN[e];
+                    // (column nth - 1 has no upper neighbour to the east: wE is 0 there)
+                    sum += ev[e] * (e < VEC - 1 ? vz[rr][e + 1] : wE);
+                    if (e == 0 && atw && in) sum += EYl[er + rr * NS] * EC[2 * rr + 1];
+                    z[e] = vz[rr][e] + od[e] * sum;
                 }
+#pragma unroll
+                for (int e = 0; e < VEC; ++e) {
+                    wN[e] = in ? vz[rr][e] : wN[e];
+                    vz[rr][e] = z[e];
+                }
+                if (hasS && rr == 0) ll_put<VEC>(halo + 2 * q.halo_row, z, ep);
+                if (hasN && rr == nr - 1) ll_put<VEC>(halo + 3 * q.halo_row, z, ep);
+                arz.add(r, z);
+                arr.add(r, r);
+                row_end();
             }
         } else {
 #pragma unroll
             for (int rr = 0; rr < RR; ++rr) {
-                if (rr >= nr) continue;
                 T r[VEC];
                 r_get(rr, r);
                 if (hasS && rr == 0) ll_put<VEC>(halo + 2 * q.halo_row, vz[rr], ep);
@@ -1022,7 +1354,7 @@ __global__ void __launch_bounds__(kResThreads + 32, 1) k_resident(const __grid_c
         if (!init) {
 #pragma unroll
             for (int rr = 0; rr < RR; ++rr) {
-                if (rr >= nr) continue;
+                if (q.o_x < 0 && rr >= nr) continue;
                 T x[VEC], u[VEC];
                 V::ldrw(pX + rr * stX, x);
                 V::ldrw(P + rr * S, u);
@@ -1042,7 +1374,6 @@ __global__ void __launch_bounds__(kResThreads + 32, 1) k_resident(const __grid_c
         const T beta = (T)sh.beta;
 #pragma unroll
         for (int rr = 0; rr < RR; ++rr) {
-            if (rr >= nr) continue;
             T u[VEC];
             V::ldrw(P + rr * S, u);
 #pragma unroll
@@ -1070,69 +1401,102 @@ __global__ void __launch_bounds__(kResThreads + 32, 1) k_resident(const __grid_c
             us[e] = uc[e] = T(0);
             nS[e] = aS0[e];
         }
-        if (act) {
-            V::ldrw(pS, us);
-            V::ldrw(P, uc);
-        }
+        V::ldrw(pS, us);
+        V::ldrw(P, uc);
 #pragma unroll
         for (int rr = 0; rr < RR; ++rr) {
-            T ev[VEC];
-#pragma unroll
-            for (int e = 0; e < VEC; ++e) ev[e] = T(0);
-            if (rr < nr) get_E(rr, ev);
+            T ev[VEC], un[VEC], nv[VEC], D[VEC];
+            get_E(rr, ev);
+            get_N(rr, nv);
+            get_D(rr, D);
+            V::ldrw(rr == RR - 1 || rr == nr - 1 ? pN : P + (rr + 1) * S, un);
             T uW = __shfl_up_sync(0xffffffffu, uc[VEC - 1], 1);
             T uE = __shfl_down_sync(0xffffffffu, uc[0], 1);
             T aW = __shfl_up_sync(0xffffffffu, ev[VEC - 1], 1);
-            if (rr < nr) {
-                T un[VEC], nv[VEC], D[VEC];
-                V::ldrw(rr == RR - 1 || rr == nr - 1 ? pN : P + (rr + 1) * S, un);
-                get_N(rr, nv);
-                get_D(rr, D);
-                if (segw) {
-                    uW = pW[rr * S];
-                    aW = EYl[er + rr * NS];
-                }
-                if (sege) uE = pE[rr * S];
-                if (last && rr == nr - 1) {
-#pragma unroll
-                    for (int e = 0; e < VEC; ++e) nv[e] = T(0);
-                }
-#pragma unroll
-                for (int e = 0; e < VEC; ++e) {
-                    const T xE = e < VEC - 1 ? uc[e + 1] : uE;
-                    const T xW = e > 0 ? uc[e - 1] : uW;
-                    const T a = e > 0 ? ev[e - 1] : aW;
-                    vz[rr][e] = D[e] * uc[e] - ev[e] * xE - a * xW - nv[e] * un[e] - nS[e] * us[e];
-                }
-                auv.add(uc, vz[rr]);
-                if (hasS && rr == 0) ll_put<VEC>(halo, vz[rr], ep);
-                if (hasN && rr == nr - 1) ll_put<VEC>(halo + q.halo_row, vz[rr], ep);
-#pragma unroll
-                for (int e = 0; e < VEC; ++e) {
-                    us[e] = uc[e];
-                    uc[e] = un[e];
-                    nS[e] = nv[e];
-                }
+            if (segw) {
+                uW = rr < nr ? pW[rr * S] : T(0);
+                aW = rr < nr ? EYl[er + rr * NS] : T(0);
             }
+            if (rr >= nr) aW = T(0);        // (the last column's, next to a thread without columns)
+            if (sege) uE = rr < nr ? pE[rr * S] : T(0);
+#pragma unroll
+            for (int e = 0; e < VEC; ++e) {
+                const T xE = e < VEC - 1 ? uc[e + 1] : uE;
+                const T xW = e > 0 ? uc[e - 1] : uW;
+                const T a = e > 0 ? ev[e - 1] : aW;
+                vz[rr][e] = D[e] * uc[e] - ev[e] * xE - a * xW - nv[e] * un[e] - nS[e] * us[e];
+            }
+            auv.add(uc, vz[rr]);
+            if (hasS && rr == 0) ll_put<VEC>(halo, vz[rr], ep);
+            if (hasN && rr == nr - 1) ll_put<VEC>(halo + q.halo_row, vz[rr], ep);
+#pragma unroll
+            for (int e = 0; e < VEC; ++e) {
+                us[e] = uc[e];
+                uc[e] = un[e];
+                nS[e] = rr + 1 < nr ? nv[e] : T(0);
+            }
+            row_end();
         }
         publish(auv.value());
         fetch(1, 0);
         bar_sync_n(2, all);
     }
 
-    // ---- the solution, and the direction of a run to be continued
+    // the solution: x, or p64 += x in its units
 #pragma unroll
     for (int rr = 0; rr < RR; ++rr) {
         if (rr >= nr) continue;
-        T t[VEC];
-        if (q.o_x >= 0) {
-            V::ldrw(pX + rr * stX, t);
-            V::st(q.p + off + (size_t)rr * nth, t);
+        T x[VEC];
+        V::ldrw(pX + rr * stX, x);
+        if constexpr (kMixed) {
+            double *const p = q.p64 + off + (size_t)rr * nth;
+#pragma unroll
+            for (int e = 0; e < VEC; ++e) p[e] = fma(sh.back, (double)x[e], p[e]);
+            asm volatile("" ::: "memory");
+        } else if (q.o_x >= 0) {
+            V::st(q.p + off + (size_t)rr * nth, x);
         }
-        if (q.u) {
-            V::ldrw(P + rr * S, t);
-            V::st(q.u + off + (size_t)rr * nth, t);
+    }
+    return ep;
+}
+
+template <typename T, int VEC, int RR, bool CS>
+__device__ __noinline__ void res_setup(const ResParams<T> &q)
+{
+    ResRows<T, VEC, RR, CS>(q, res_shared<T>()).setup();
+}
+template <typename T, int VEC, int RR, bool CS>
+__device__ __noinline__ void res_residual(const ResParams<T> &q, unsigned ep)
+{
+    ResRows<T, VEC, RR, CS>(q, res_shared<T>()).residual(ep);
+}
+
+template <typename T, int VEC, int RR, bool CS>
+__global__ void __launch_bounds__(kResThreads + 32, 1) k_resident(const __grid_constant__ ResParams<T> q)
+{
+    ResShared<T> &sh = res_shared<T>();
+    const int cond = blockIdx.x / q.bpc, grp = q.groups == 1 ? 0 : cond;
+    if (!((q.mask >> grp) & 1ull)) return;                  // this group does not run
+    if ((int)threadIdx.x >= q.threads) {
+        res_exchange_warp<T>(q, sh, q.sc + grp, grp, q.groups == 1 ? 0 : cond * q.bpc,
+                             q.groups == 1 ? (int)gridDim.x : q.bpc, threadIdx.x & 31);
+        return;
+    }
+    unsigned ep = q.epoch;
+    if constexpr (sizeof(T) == 4) {
+        // FP64 refinements around the FP32 run
+        res_setup<T, VEC, RR, CS>(q);
+#pragma unroll 1
+        for (;;) {
+            res_residual<T, VEC, RR, CS>(q, ++ep);
+            bar_sync_n(2, q.threads + 32);
+            bar_sync_n(2, q.threads + 32);
+            if (sh.stop) break;
+            ep = res_iterate<T, VEC, RR, CS>(q, sh, ep);
         }
+    } else {
+        res_setup<T, VEC, RR, CS>(q);
+        res_iterate<T, VEC, RR, CS>(q, sh, ep);
     }
 }
 

@@ -19,10 +19,10 @@ constexpr int kResVariant = 50000000;   // gmaf_solve_info.kernel_variant: + 100
 // not hold r beside the product.
 __host__ __device__ constexpr bool res_r_shared(int rr, int vec, int size) { return rr * vec * size > 64; }
 
+// FP64 (T = double): one run.  FP32: the whole mixed-precision solve.
 enum ResMode {
     kResFresh = 0,      // r = b - A p (p = 0 with zero_init)
-    kResRestart = 1,    // r handed in, p continued, the norm of b kept from the last run
-    kResContinue = 2    // r = b, p = 0, the recurrence continued with the direction in u
+    kResRestart = 1     // r handed in, p continued, the count and the norm of b kept from the last run
 };
 
 // Kernel parameters.  o_*: byte offsets in shared memory (-1: the array stays in
@@ -31,7 +31,7 @@ template <typename T>
 struct ResParams {
     int nth, nz, bpc, groups;           // bpc blocks a condition; groups: 1 joint system or K
     int threads, P, ncg, nrr, rows;
-    int precond, mode, zero_init, keep_iter, max_iter, guard_limit;
+    int precond, mode, zero_init, max_iter, guard_limit;
     int o_rows, o_edge, o_x;
     unsigned epoch;                     // exchanges of this run are epoch + 1, epoch + 2, ...
     unsigned long long mask;            // groups that run
@@ -39,13 +39,20 @@ struct ResParams {
     const T *D, *invD, *aE, *aN;
     const int *cslot;
     const T *b, *r_in;
-    T *p, *u;                           // u: written at the end (null: not wanted)
+    T *p;                               // (FP32: scratch for x when it does not fit on the SM)
     Scalars *sc;                        // [groups]
-    double eps, cscale;
+    double eps;
+    // FP32: the FP64 system and its refinement
+    const double *D64, *aE64, *aN64, *S64, *scale;   // scale: FP32 matrix = scale A
+    double *p64, *r64;
+    unsigned long long *halo64;         // flagged FP64 rows, [blocks][2]
+    double inner_floor;                 // reduction of a run
+    int continued, max_outer;
     unsigned long long *words;          // [groups][kResGroupWords], zero at the start of the run
     unsigned long long *halo;           // flagged rows, [blocks][4]
     int halo_row;                       // 8-byte words of one flagged row
-    unsigned long long *times;          // ns in A, B and set-up, counts of A and B (added to; or null)
+    unsigned long long *times;          // ns in A, B and set-up, counts of A and B, ns and count
+                                        // of FP64 residuals (added to; or null)
 };
 
 struct ResPlan {
