@@ -1265,8 +1265,15 @@ int solve_joint_device(gmaf_ctx *ctx, int nth, int nz, int K, int nslots, const 
     ResRun<float> rr;
     res_setup<float>(ctx, rr, nth, nz, K, nth % 4 == 0);
     if (rr.on) {
-        if (rr.pl.o_x < 0) GMAF_TRY(ensure(ctx, B_X32, (size_t)N * sizeof(float)));
+        if (rr.pl.tm || rr.pl.o_x < 0) GMAF_TRY(ensure(ctx, B_X32, (size_t)N * sizeof(float)));
         ResParams<float> &q = rr.q;
+        if (rr.pl.tm) {
+            GMAF_TRY(ensure(ctx, B_DBND32, (size_t)nslots * 2 * nth * sizeof(float)));
+            GMAF_TRY(launch_dbnd32((const float *)ctx->buf[B_D32], (const float *)ctx->buf[B_AE32],
+                                   (const float *)ctx->buf[B_AN32], (float *)ctx->buf[B_DBND32], nth, nz,
+                                   nslots, ctx->num_sms, s));
+            q.dbnd = (const float *)ctx->buf[B_DBND32];
+        }
         q.precond = kernel_precond(opts);
         q.max_iter = opts->max_iter;
         q.guard_limit = ctx->loop_guard;

@@ -59,6 +59,20 @@ bool res_plan(int nth, int nz, int K, bool vec_ok, int num_sms, ResPlan *out)
             break;
         }
     }
+    if (!best && sizeof(T) == 4 && vec_ok && nth / 4 <= kResThreads) {
+        // the largest systems (one joint system, 4 columns a thread): with an iteration on 9
+        // conditions of 700 x 300 cells in 33 us against 57 of the phase kernels and of 1024 x
+        // 512 in 39 against 68, whatever fits comes here
+        pl.tm = true;
+        pl.vec = 4;
+        pl.rr = kTmRows;
+        pl.ncg = nth / 4;
+        pl.P = 1;
+        while (pl.P < pl.ncg && pl.P < 32) pl.P *= 2;
+        if (pl.ncg > 32) pl.P = (pl.ncg + 31) / 32 * 32;
+        pl.nrr = (pl.rows + kTmRows - 1) / kTmRows;
+        best = (long long)pl.P * pl.nrr <= kResThreads;
+    }
     if (!best) return false;
     pl.threads = (pl.P * pl.nrr + 31) / 32 * 32;
     // shared memory: u, rows and edges, r for the longest runs; then, as far as there is
@@ -68,21 +82,27 @@ bool res_plan(int nth, int nz, int K, bool vec_ok, int num_sms, ResPlan *out)
     const long long field = (long long)pl.rr * kResThreads * pl.vec * sz;
     const long long rows = (long long)(6 + 2 * pl.nrr) * nth * sz;
     const long long edges = (long long)(pl.rows + 1) * (3 * kResSegs + 2) * sz;
-    const long long need = field * (res_r_shared(pl.rr, pl.vec, sz) ? 2 : 1) + round16(rows) + round16(edges);
+    const bool rs = !pl.tm && res_r_shared(pl.rr, pl.vec, sz);
+    const long long need = field * (rs ? 2 : 1) + round16(rows) + round16(edges);
     if (rows > kMax || edges > kMax || need > kMax) return false;
-    const bool cs = need + 4 * field <= kMax;
-    long long o = field * ((res_r_shared(pl.rr, pl.vec, sz) ? 2 : 1) + (cs ? 4 : 0));
+    const bool cs = !pl.tm && need + 4 * field <= kMax;
+    long long o = field * ((rs ? 2 : 1) + (cs ? 4 : 0));
     pl.o_rows = (int)o;
     o += round16(rows);
     pl.o_edge = (int)o;
     o += round16(edges);
     pl.o_x = -1;
-    if (o + field <= kMax) {
+    if (pl.tm) {
+        // omega/D of as many rows of a run as there is room for
+        pl.o_x = (int)o;
+        pl.ri = (int)std::min<long long>(kTmRows, (kMax - o) / (field / kTmRows));
+        o += pl.ri * (field / kTmRows);
+    } else if (o + field <= kMax) {
         pl.o_x = (int)o;
         o += field;
     }
     pl.smem = (int)o;
-    pl.fn = sz == 4 ? res_kernel_f32(pl.vec, pl.rr, cs) : res_kernel_f64(pl.vec, pl.rr, cs);
+    pl.fn = pl.tm ? res_kernel_tm() : sz == 4 ? res_kernel_f32(pl.vec, pl.rr, cs) : res_kernel_f64(pl.vec, pl.rr, cs);
     if (!pl.fn) return false;
     // flagged rows: four of T, and for FP32 two of doubles behind them
     pl.halo_bytes = (size_t)pl.grid * 4 * nth * 2 * sz + (sz == 4 ? (size_t)pl.grid * 2 * nth * 16 : 0);
@@ -102,6 +122,7 @@ void res_fill(const ResPlan &pl, ResParams<T> *q)
     q->o_rows = pl.o_rows;
     q->o_edge = pl.o_edge;
     q->o_x = pl.o_x;
+    q->ri = pl.ri;
     q->halo_row = q->nth * ((int)sizeof(T) / 4);
     q->halo64 = q->halo + (size_t)pl.grid * 4 * q->halo_row;
 }

@@ -46,6 +46,8 @@ struct ResParams {
     const double *D64, *aE64, *aN64, *S64, *scale;   // scale: FP32 matrix = scale A
     double *p64, *r64;
     unsigned long long *halo64;         // flagged FP64 rows, [blocks][2]
+    const float *dbnd;                  // the largest systems: Dirichlet term of the diagonal, [slots][2][nth]
+    int ri;                             //   and rows of a run whose omega/D is in shared memory
     double inner_floor;                 // reduction of a run
     int continued, max_outer;
     unsigned long long *words;          // [groups][kResGroupWords], zero at the start of the run
@@ -59,7 +61,8 @@ struct ResPlan {
     const void *fn;
     int grid, smem, vec, rr;
     int bpc, threads, P, ncg, nrr, rows;
-    int o_rows, o_edge, o_x;
+    int o_rows, o_edge, o_x, ri;
+    bool tm;                            // the largest systems (k_resident_tm)
     size_t halo_bytes;                  // flagged rows, zero before the first launch
 };
 
@@ -75,6 +78,8 @@ void res_fill(const ResPlan &pl, ResParams<T> *q);
 // Kernel of a plan (compiled for T in a translation unit of its own).
 const void *res_kernel_f32(int vec, int rr, bool cs);
 const void *res_kernel_f64(int vec, int rr, bool cs);
+const void *res_kernel_tm();
+constexpr int kTmRows = 16;             // rows of a run of k_resident_tm
 
 // Cooperative launch; cudaErrorCooperativeLaunchTooLarge when the blocks cannot all
 // be resident (a partitioned GPU): the caller then takes the phase kernels.

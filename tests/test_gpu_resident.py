@@ -145,6 +145,30 @@ def test_grids_beyond_the_resident_solve_take_the_phase_kernels(g, monkeypatch, 
     assert rel_l2(p, ref) <= 1e-10
 
 
+# runs of 16 rows (id 50004160): whole and partial ones, one and two of them a column, rows that
+# are no multiple of a warp's columns, five blocks a condition; then a row of threads
+# too many.  The condition number grows with the square of the rows: up to four times that of the
+# grids above, and the tolerance with it
+@pytest.mark.parametrize("nth,nz,K,precond,fits", [
+    (1024, 512, 9, 1, True), (700, 300, 9, 1, True), (700, 300, 9, 0, True),
+    (2048, 152, 9, 2, True), (2048, 147, 9, 1, True), (128, 1000, 30, 1, True),
+    (1028, 290, 9, 1, False), (1024, 529, 9, 1, False),
+])
+def test_largest_resident_systems_match_phase_kernels(g, monkeypatch, nth, nz, K, precond, fits):
+    _, arrs = system(nth, nz, K, nth + nz)
+    kw = dict(precision=1, precond=precond)
+    p, it, rel, info = solve(g, monkeypatch, nth, nz, K, arrs, **kw)
+    assert info["kernel_variant"] == 50004160 if fits else not resident(info)
+    ref, itr, _, infr = solve(g, monkeypatch, nth, nz, K, arrs, variant=1001004, **kw)
+    assert not resident(infr)
+    assert rel <= 1e-12 and abs(it - itr) <= 2 + itr // 50
+    assert rel_l2(p, ref) <= 4e-10
+    p2, it2, _, _ = solve(g, monkeypatch, nth, nz, K, arrs, **kw)
+    assert it2 == it and torch.equal(p, p2)
+    p3, it3, _, _ = solve(g, monkeypatch, nth, nz, K, arrs, start=p, eps=1e-10, **kw)
+    assert it3 == 0 and torch.equal(p3, p)
+
+
 def test_sources_of_any_scale(g, monkeypatch):
     """The sums over blocks are fixed-point numbers on a scale that follows them: sources
     scaled by powers of two give the scaled solution, bit for bit."""
