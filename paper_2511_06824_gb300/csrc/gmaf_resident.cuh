@@ -440,6 +440,21 @@ __device__ __forceinline__ double res_quotient(double a, double b)
     return fma(y, fma(-b, t, a), t);
 }
 
+// Sums and products are written out as fused operations in the order of the phase kernels
+// (gmaf_pcg_kernels.cuh), so that an FP32 run passes through their numbers: only the sums over
+// the grid, which every scalar is rounded from, are added in another order.  A stopped
+// refinement leaves rounding of 1e-13 in a solution, which a finite-difference Jacobian
+// magnifies by 1e4: it must not depend on which kernels a grid takes.  (Left to the compiler,
+// the two sweeps' sums were fused the other way round; on 9 conditions of 512 x 256 cells the
+// Jacobian moved by up to 2.4e-9.)
+__device__ __forceinline__ float res_fma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ float res_fnma(float a, float b, float c) { return __fmaf_rn(-a, b, c); }
+__device__ __forceinline__ float res_diff(float a, float b, float c, float d) { return __fmaf_rn(a, b, -__fmul_rn(c, d)); }
+// (FP64 keeps the compiler's choice: it leaves no such trace)
+__device__ __forceinline__ double res_fma(double a, double b, double c) { return a * b + c; }
+__device__ __forceinline__ double res_fnma(double a, double b, double c) { return c - a * b; }
+__device__ __forceinline__ double res_diff(double a, double b, double c, double d) { return a * b - c * d; }
+
 // Barrier of the threads that own rows (the exchange warp does not take part).
 __device__ __forceinline__ void bar_sync_n(int id, int threads)
 {
@@ -772,7 +787,7 @@ struct ResAcc<float> {
     {
         float t = 0.0f;
 #pragma unroll
-        for (int e = 0; e < VEC; ++e) t += a[e] * b[e];
+        for (int e = 0; e < VEC; ++e) t = res_fma(a[e], b[e], t);
         s.add_sum(t);
     }
     __device__ __forceinline__ Acc<float> value() const { return s; }
@@ -1264,9 +1279,9 @@ __device__ __forceinline__ unsigned res_iterate(const ResParams<T> &q, ResShared
 #pragma unroll
                 for (int e = 0; e < VEC; ++e) {
                     T sum = nS[e] * yp[e];
-                    sum += (e > 0 ? ev[e - 1] : aW) * (e > 0 ? vz[rr][e - 1] : yW);
-                    if (e == VEC - 1 && ate && in) sum += ev[e] * EC[2 * rr];
-                    w[e] = vz[rr][e] + od[e] * sum;
+                    sum = res_fma(e > 0 ? ev[e - 1] : aW, e > 0 ? vz[rr][e - 1] : yW, sum);
+                    if (e == VEC - 1 && ate && in) sum = res_fma(ev[e], EC[2 * rr], sum);
+                    w[e] = res_fma(od[e], sum, vz[rr][e]);
                 }
                 if (rr == 0 && act && run > 0) V::st(WR + (run - 1) * nth + c, w);
                 if (segw && in) EY[2 * er + rr * NS] = w[0];
@@ -1298,11 +1313,11 @@ __device__ __forceinline__ unsigned res_iterate(const ResParams<T> &q, ResShared
                     for (int e = 0; e < VEC; ++e) {
                         T sum = nS[e] * yp[e];
                         if (e > 0)
-                            sum += ev[e - 1] * yN[e - 1];
+                            sum = res_fma(ev[e - 1], yN[e - 1], sum);
                         else if (!atw)
-                            sum += aW * yW;
-                        if (e == VEC - 1 && ate) sum += ev[e] * EC[2 * nr];
-                        wN[e] = yN[e] + od[e] * sum;
+                            sum = res_fma(aW, yW, sum);
+                        if (e == VEC - 1 && ate) sum = res_fma(ev[e], EC[2 * nr], sum);
+                        wN[e] = res_fma(od[e], sum, yN[e]);
                     }
                 }
             }
@@ -1323,9 +1338,9 @@ __device__ __forceinline__ unsigned res_iterate(const ResParams<T> &q, ResShared
                 for (int e = 0; e < VEC; ++e) {
                     T sum = nv[e] * wN[e];
                     // (column nth - 1 has no upper neighbour to the east: wE is 0 there)
-                    sum += ev[e] * (e < VEC - 1 ? vz[rr][e + 1] : wE);
-                    if (e == 0 && atw && in) sum += EYl[er + rr * NS] * EC[2 * rr + 1];
-                    z[e] = vz[rr][e] + od[e] * sum;
+                    sum = res_fma(ev[e], e < VEC - 1 ? vz[rr][e + 1] : wE, sum);
+                    if (e == 0 && atw && in) sum = res_fma(EYl[er + rr * NS], EC[2 * rr + 1], sum);
+                    z[e] = res_fma(od[e], sum, vz[rr][e]);
                 }
 #pragma unroll
                 for (int e = 0; e < VEC; ++e) {
@@ -1424,7 +1439,10 @@ __device__ __forceinline__ unsigned res_iterate(const ResParams<T> &q, ResShared
                 const T xE = e < VEC - 1 ? uc[e + 1] : uE;
                 const T xW = e > 0 ? uc[e - 1] : uW;
                 const T a = e > 0 ? ev[e - 1] : aW;
-                vz[rr][e] = D[e] * uc[e] - ev[e] * xE - a * xW - nv[e] * un[e] - nS[e] * us[e];
+                T t = res_diff(D[e], uc[e], ev[e], xE);
+                t = res_fnma(a, xW, t);
+                t = res_fnma(nv[e], un[e], t);
+                vz[rr][e] = res_fnma(nS[e], us[e], t);
             }
             auv.add(uc, vz[rr]);
             if (hasS && rr == 0) ll_put<VEC>(halo, vz[rr], ep);

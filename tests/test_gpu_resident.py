@@ -169,6 +169,24 @@ def test_largest_resident_systems_match_phase_kernels(g, monkeypatch, nth, nz, K
     assert it3 == 0 and torch.equal(p3, p)
 
 
+@pytest.mark.parametrize("nth,nz,K", [(96, 48, 9), (132, 45, 9), (256, 128, 9), (512, 256, 9)])
+def test_mixed_runs_pass_through_the_numbers_of_the_phase_kernels(g, monkeypatch, nth, nz, K):
+    """FP32 arithmetic cell by cell is that of the phase kernels (id 604322); only the grid's sums
+    are added in another order, each rounded to FP32 before it is used.  So the first iterations
+    agree but for the FP64 norm of the residual, the factor of x in p, which takes another last bit
+    or two (another FP32 rounding anywhere would show as 1e-10 and more), and converged solutions
+    agree far below the tolerance that stopped them."""
+    _, arrs = system(nth, nz, K, nth)
+    kw = dict(precision=1, eps=1e-13)
+    p, _, _, info = solve(g, monkeypatch, nth, nz, K, arrs, max_iter=3, allow=True, **kw)
+    ref, _, _, infr = solve(g, monkeypatch, nth, nz, K, arrs, max_iter=3, allow=True, variant=604322, **kw)
+    assert resident(info) and infr["kernel_variant"] == 604322
+    assert rel_l2(p, ref) <= 1e-14
+    p, it, _, _ = solve(g, monkeypatch, nth, nz, K, arrs, **kw)
+    ref, itr, _, _ = solve(g, monkeypatch, nth, nz, K, arrs, variant=604322, **kw)
+    assert abs(it - itr) <= 2 and rel_l2(p, ref) <= 5e-12
+
+
 def test_sources_of_any_scale(g, monkeypatch):
     """The sums over blocks are fixed-point numbers on a scale that follows them: sources
     scaled by powers of two give the scaled solution, bit for bit."""
