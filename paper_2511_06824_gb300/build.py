@@ -17,7 +17,7 @@ CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libgmaf.so")
 SOURCES = ["gmaf_api.cu", "gmaf_assemble.cu", "gmaf_pcg.cu", "gmaf_tma.cu", "gmaf_drec.cu",
-           "gmaf_resident.cu", "gmaf_resident_f32.cu", "gmaf_resident_tm.cu",
+           "gmaf_resident.cu", "gmaf_resident_f32.cu", "gmaf_resident_tm.cu", "gmaf_resident_s.cu",
            "gmaf_server.cu", "gmaf_noalloc.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC = os.environ.get("NVCC", "nvcc")

@@ -112,8 +112,8 @@ enum BufId {
     B_CHUNK, B_CHUNKCTR,
     // boundary rows' Dirichlet term of the FP32 diagonal (phase A with the rebuilt diagonal)
     B_DBND32,
-    // resident PCG: exchanged rows, words of the exchanged sums, phase times
-    B_RES, B_RESWORDS, B_RESTIME,
+    // resident PCG: exchanged rows, words of the exchanged sums, phase times, scaled matrix
+    B_RES, B_RESWORDS, B_RESTIME, B_RESCOEF,
     B_COUNT
 };
 

@@ -881,7 +881,8 @@ struct ResRun {
 // The plan and its buffers; off (phase kernels) when the system does not fit, when a
 // phase kernel is asked for, or when the budget has no room for the exchanged words.
 template <typename T>
-static void res_setup(gmaf_ctx *ctx, ResRun<T> &rr, int nth, int nz, int K, bool vec)
+static void res_setup(gmaf_ctx *ctx, ResRun<T> &rr, int nth, int nz, int K, bool vec, long long m,
+                      bool with_d)
 {
     rr.on = false;
     if (ctx->force_variant >= 0 && ctx->force_variant / 10000000 != kResVariant / 10000000) return;
@@ -894,6 +895,7 @@ static void res_setup(gmaf_ctx *ctx, ResRun<T> &rr, int nth, int nz, int K, bool
     if (ensure(ctx, B_RESWORDS, kResRing) != GMAF_OK) return;
     if (ensure(ctx, B_RES, rr.pl.halo_bytes) != GMAF_OK) return;
     if (ctx->phase_timing && ensure(ctx, B_RESTIME, 64) != GMAF_OK) return;
+    if (sizeof(T) == 8 && rr.pl.tm && ensure(ctx, B_RESCOEF, res_scaled_bytes(m, with_d)) != GMAF_OK) return;
     ResParams<T> &q = rr.q;
     q.nth = nth;
     q.nz = nz;
@@ -990,9 +992,9 @@ static int solve_resident64(gmaf_ctx *ctx, ResRun<double> &rr, int K, const int 
         rd[k].nz = q.nz;
         rd[k].K = async ? 1 : K;
         rd[k].n = n;
-        rd[k].D = q.D + c;
-        rd[k].aE = q.aE + c;
-        rd[k].aN = q.aN + c;
+        rd[k].D = q.D64 + c;
+        rd[k].aE = q.aE64 + c;
+        rd[k].aN = q.aN64 + c;
         rd[k].cslot = async ? (const int *)((char *)ctx->buf[B_ASYNC] + o_slot) : q.cslot;
         rd[k].S = S + o;
         rd[k].p = p + o;
@@ -1136,7 +1138,7 @@ int solve_joint_device(gmaf_ctx *ctx, int nth, int nz, int K, int nslots, const 
         const void *ptrs[] = {D, aE, aN, S, p};
         bool vec = nth % 2 == 0;
         for (const void *x : ptrs) vec = vec && aligned16(x);
-        res_setup<double>(ctx, rr, nth, nz, K, vec);
+        res_setup<double>(ctx, rr, nth, nz, K, vec, m, opts->precond == 2);
         if (rr.on) {
             ResParams<double> &q = rr.q;
             q.precond = kernel_precond(opts);
@@ -1152,6 +1154,18 @@ int solve_joint_device(gmaf_ctx *ctx, int nth, int nz, int K, int nslots, const 
             q.b = S;
             q.r_in = nullptr;
             q.p = p;
+            q.D64 = D;
+            q.aE64 = aE;
+            q.aN64 = aN;
+            q.p64 = p;
+            if (rr.pl.tm) {
+                // (x apart from p, which keeps the start until the end)
+                if (rr.pl.o_x < 0) GMAF_TRY(ensure(ctx, B_U0, (size_t)N * sizeof(double)));
+                q.x = (double *)ctx->buf[B_U0];
+                GMAF_TRY(res_scaled(D, aE, aN, opts->precond == 2 ? (const double *)ctx->buf[B_INVD] : nullptr,
+                                    opts->precond == 1 ? opts->omega : 1.0, nth, nz, m, ctx->buf[B_RESCOEF],
+                                    ctx->num_sms, s, &q));
+            }
             bool off = false;
             const int st = solve_resident64(ctx, rr, K, cslot_host, S, p, opts, info, &off);
             if (!off) return st;
@@ -1263,11 +1277,11 @@ int solve_joint_device(gmaf_ctx *ctx, int nth, int nz, int K, int nslots, const 
 
     // the whole refinement in one launch where the system fits on the SMs
     ResRun<float> rr;
-    res_setup<float>(ctx, rr, nth, nz, K, nth % 4 == 0);
+    res_setup<float>(ctx, rr, nth, nz, K, nth % 4 == 0, m, false);
     if (rr.on) {
-        if (rr.pl.tm || rr.pl.o_x < 0) GMAF_TRY(ensure(ctx, B_X32, (size_t)N * sizeof(float)));
+        if (rr.pl.tm == 3 || rr.pl.o_x < 0) GMAF_TRY(ensure(ctx, B_X32, (size_t)N * sizeof(float)));
         ResParams<float> &q = rr.q;
-        if (rr.pl.tm) {
+        if (rr.pl.tm == 3) {
             GMAF_TRY(ensure(ctx, B_DBND32, (size_t)nslots * 2 * nth * sizeof(float)));
             GMAF_TRY(launch_dbnd32((const float *)ctx->buf[B_D32], (const float *)ctx->buf[B_AE32],
                                    (const float *)ctx->buf[B_AN32], (float *)ctx->buf[B_DBND32], nth, nz,
@@ -1283,7 +1297,7 @@ int solve_joint_device(gmaf_ctx *ctx, int nth, int nz, int K, int nslots, const 
         q.aE = (const float *)ctx->buf[B_AE32];
         q.aN = (const float *)ctx->buf[B_AN32];
         q.cslot = cslot;
-        q.p = (float *)ctx->buf[B_X32];
+        q.p = q.x = (float *)ctx->buf[B_X32];
         q.sc = dsc;
         q.D64 = D;
         q.aE64 = aE;

@@ -804,10 +804,8 @@ struct ResRows {
     using V = Vec<T, VEC>;
     static constexpr int S = kResThreads * VEC;     // private fields: [row][thread][VEC]
     static constexpr int NS = kResSegs;
-    static constexpr bool RS = res_r_shared(RR, VEC, sizeof(T));
     static constexpr bool kMixed = sizeof(T) == 4;  // FP32 runs inside FP64 refinement
     static constexpr int FE = RR * S, FN = 2 * RR * S, FI = 3 * RR * S, FD = 4 * RR * S;
-    static constexpr int FR = CS ? 5 * RR * S : RR * S;
 
     const ResParams<T> &q;
     ResShared<T> &sh;
@@ -1007,10 +1005,8 @@ __device__ __forceinline__ unsigned res_iterate(const ResParams<T> &q, ResShared
     using V = Vec<T, VEC>;
     constexpr int S = kResThreads * VEC;            // private fields: [row][thread][VEC]
     constexpr int NS = kResSegs;
-    constexpr bool RS = res_r_shared(RR, VEC, sizeof(T));
     constexpr bool kMixed = sizeof(T) == 4;         // FP32 runs inside FP64 refinement
     constexpr int FE = RR * S, FN = 2 * RR * S, FI = 3 * RR * S, FD = 4 * RR * S;
-    constexpr int FR = CS ? 5 * RR * S : RR * S;
     extern __shared__ __align__(16) unsigned char g_res_smem[];
     const int nth = q.nth, nz = q.nz, TC = q.threads, all = TC + 32;
     int tid;
@@ -1079,29 +1075,16 @@ __device__ __forceinline__ unsigned res_iterate(const ResParams<T> &q, ResShared
     auto get_I = [&](int rr, T(&x)[VEC]) { coef(FI, q.invD, rr, x); };
     auto get_D = [&](int rr, T(&x)[VEC]) { coef(FD, q.D, rr, x); };
 
-    // (the longest runs: no loads of one row moved across another, there are no registers for it)
-    auto row_end = [] {
-        if constexpr (RS) asm volatile("" ::: "memory");
-    };
-
     // rows of a block's halo area: 0, 1 = first and last row of v; 2, 3 = of z
     unsigned long long *const halo = q.halo + (size_t)blockIdx.x * 4 * q.halo_row + c * ((int)sizeof(T) / 4);
-    T rg[RS ? 1 : RR][VEC], vz[RR][VEC], aS0[VEC], hS[VEC], hN[VEC];
+    T rg[RR][VEC], vz[RR][VEC], aS0[VEC], hS[VEC], hN[VEC];
     auto r_get = [&](int rr, T(&x)[VEC]) {
-        if constexpr (RS) {
-            V::ldrw(P + FR + rr * S, x);
-        } else {
 #pragma unroll
-            for (int e = 0; e < VEC; ++e) x[e] = rg[rr][e];
-        }
+        for (int e = 0; e < VEC; ++e) x[e] = rg[rr][e];
     };
     auto r_put = [&](int rr, const T(&x)[VEC]) {
-        if constexpr (RS) {
-            V::st(P + FR + rr * S, x);
-        } else {
 #pragma unroll
-            for (int e = 0; e < VEC; ++e) rg[rr][e] = x[e];
-        }
+        for (int e = 0; e < VEC; ++e) rg[rr][e] = x[e];
     };
 #pragma unroll
     for (int rr = 0; rr < RR; ++rr)
@@ -1228,7 +1211,6 @@ __device__ __forceinline__ unsigned res_iterate(const ResParams<T> &q, ResShared
             if (rr == RR - 1 && act && !top) V::st(YR + (run + 1) * nth + c, vz[rr]);
             if (sege && rr < nr) EY[rr * NS] = vz[rr][VEC - 1];
             if (atw && rr < nr) EC[2 * rr] = vz[rr][0];
-            row_end();
         }
         if (hasS) {
             T h[VEC], od[VEC];
@@ -1292,8 +1274,7 @@ __device__ __forceinline__ unsigned res_iterate(const ResParams<T> &q, ResShared
                     nS[e] = in ? nv[e] : nS[e];
                     vz[rr][e] = w[e];
                 }
-                row_end();
-            }
+                }
             // w on the row above the block, for z of its last row
             {
                 T ev[VEC];
@@ -1351,8 +1332,7 @@ __device__ __forceinline__ unsigned res_iterate(const ResParams<T> &q, ResShared
                 if (hasN && rr == nr - 1) ll_put<VEC>(halo + 3 * q.halo_row, z, ep);
                 arz.add(r, z);
                 arr.add(r, r);
-                row_end();
-            }
+                }
         } else {
 #pragma unroll
             for (int rr = 0; rr < RR; ++rr) {
@@ -1453,7 +1433,6 @@ __device__ __forceinline__ unsigned res_iterate(const ResParams<T> &q, ResShared
                 uc[e] = un[e];
                 nS[e] = rr + 1 < nr ? nv[e] : T(0);
             }
-            row_end();
         }
         publish(auv.value());
         fetch(1, 0);

@@ -15,9 +15,15 @@ constexpr int kResGroupWords = 16;      // 8-byte words of a group of blocks for
 constexpr int kResSegs = kResThreads / 32;   // segments of 32 threads in a row, at most
 constexpr int kResVariant = 50000000;   // gmaf_solve_info.kernel_variant: + 1000 VEC + 10 RR
 
-// Whether a run's r lives in shared memory: with over 64 bytes a thread the registers do
-// not hold r beside the product.
-__host__ __device__ constexpr bool res_r_shared(int rr, int vec, int size) { return rr * vec * size > 64; }
+// Where a kernel keeps r and the product: in registers (0), or, with over 64 bytes a thread, in
+// tensor memory: with the couplings there too (1, runs of 8 rows), or in runs of 16 with the
+// couplings streamed from L2 (FP64: 2, FP32: 3).
+__host__ __device__ constexpr int res_tm(int rr, int vec, int size)
+{
+    return rr * vec * size <= 64 ? 0 : rr == 8 ? 1 : size == 8 ? 2 : 3;
+}
+// Rows of n_theta values that a block of form 1 or 2 keeps in shared memory.
+__host__ __device__ constexpr int res_tm_rows(int nrr, int size) { return size == 8 ? 4 + 3 * nrr : 5 + 4 * nrr; }
 
 // FP64 (T = double): one run.  FP32: the whole mixed-precision solve.
 enum ResMode {
@@ -30,20 +36,24 @@ enum ResMode {
 template <typename T>
 struct ResParams {
     int nth, nz, bpc, groups;           // bpc blocks a condition; groups: 1 joint system or K
-    int threads, P, ncg, nrr, rows;
+    int threads, P, ncg, nrr, rows, nseg;
     int precond, mode, zero_init, max_iter, guard_limit;
-    int o_rows, o_edge, o_x;
+    int o_rows, o_edge, o_x, o_q, o_keep, keep;     // keep: rows of a run whose E stays on the SM
     unsigned epoch;                     // exchanges of this run are epoch + 1, epoch + 2, ...
     unsigned long long mask;            // groups that run
     long long n;
-    const T *D, *invD, *aE, *aN;
+    const T *D, *invD, *aE, *aN;        // (scaled: of s A s; D null where it is the constant dg)
     const int *cslot;
     const T *b, *r_in;
     T *p;                               // (FP32: scratch for x when it does not fit on the SM)
+    // scaled FP64: 1 / s^2, s, and scratch for x; the system is D64 ..., p64
+    const T *Q, *s;
+    T *x;
+    T dg;
     Scalars *sc;                        // [groups]
     double eps;
     // FP32: the FP64 system and its refinement
-    const double *D64, *aE64, *aN64, *S64, *scale;   // scale: FP32 matrix = scale A
+    const double *D64, *aE64, *aN64, *S64, *scale;   // scale: FP32 or scaled matrix: of scale A
     double *p64, *r64;
     unsigned long long *halo64;         // flagged FP64 rows, [blocks][2]
     const float *dbnd;                  // the largest systems: Dirichlet term of the diagonal, [slots][2][nth]
@@ -60,9 +70,9 @@ struct ResParams {
 struct ResPlan {
     const void *fn;
     int grid, smem, vec, rr;
-    int bpc, threads, P, ncg, nrr, rows;
-    int o_rows, o_edge, o_x, ri;
-    bool tm;                            // the largest systems (k_resident_tm)
+    int bpc, threads, P, ncg, nrr, rows, nseg;
+    int o_rows, o_edge, o_x, o_q, o_keep, keep, ri;
+    int tm;                             // res_tm
     size_t halo_bytes;                  // flagged rows, zero before the first launch
 };
 
@@ -80,6 +90,13 @@ const void *res_kernel_f32(int vec, int rr, bool cs);
 const void *res_kernel_f64(int vec, int rr, bool cs);
 const void *res_kernel_tm();
 constexpr int kTmRows = 16;             // rows of a run of k_resident_tm
+const void *res_kernel_s(int size, int rr);
+
+// The scaled FP64 matrix of m cells: coef (res_scaled_bytes) receives aE, aN, Q, s and (with minv)
+// D.  minv: the preconditioner's diagonal, null for w / D.
+size_t res_scaled_bytes(long long m, bool with_d);
+int res_scaled(const double *D, const double *aE, const double *aN, const double *minv, double w, int nth, int nz,
+               long long m, void *coef, int num_sms, cudaStream_t s, ResParams<double> *q);
 
 // Cooperative launch; cudaErrorCooperativeLaunchTooLarge when the blocks cannot all
 // be resident (a partitioned GPU): the caller then takes the phase kernels.

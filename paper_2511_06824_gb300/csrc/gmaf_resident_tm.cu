@@ -1,9 +1,8 @@
 // The resident PCG for the largest systems it takes (FP32 inside FP64 refinement): its
 // vectors in shared and tensor memory.
 //
-// Above 16 cells a thread the registers hold neither r nor the product.  Both then live in
-// the SM's tensor memory (256 KB that no other kernel here uses; each thread has 128 words
-// of its own lane: 64 of the product, 64 of r), u stays in shared memory, and the
+// Runs of 16 rows: r and the product live in the SM's tensor memory (64 words a thread each),
+// u stays in shared memory, and the
 // coefficients and x are streamed from L2, one group of rows ahead of the one worked on.
 // The diagonal is rebuilt from the couplings, as in the phase A of gmaf_drec.cu, to save
 // its traffic.
@@ -12,22 +11,10 @@
 // coefficients' and x's 175 MB from L2 at 4.5 TB/s, and two exchanges of 1.5 us), the
 // phase kernels take 68.3; on 9 of 700 x 300 it is 33.3 against 56.7.
 #include "gmaf_resident.cuh"
+#include "gmaf_tmem.cuh"
 
 namespace gmaf {
 
-constexpr int kTmCols = 512;                // columns of tensor memory (32-bit words a lane): all
-
-__device__ __forceinline__ void tm_alloc(unsigned *slot)
-{
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(smem_u32(slot)),
-                 "n"(kTmCols)
-                 : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
-}
-__device__ __forceinline__ void tm_free(unsigned base)
-{
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(base), "n"(kTmCols) : "memory");
-}
 __device__ __forceinline__ void tm_ld(unsigned at, float (&x)[4])
 {
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];\n"
@@ -44,14 +31,6 @@ __device__ __forceinline__ void tm_wait_ld(float (&x)[4], float (&y)[4])
     asm volatile("tcgen05.wait::ld.sync.aligned;\n"
                  : "+f"(x[0]), "+f"(x[1]), "+f"(x[2]), "+f"(x[3]), "+f"(y[0]), "+f"(y[1]), "+f"(y[2]), "+f"(y[3])::"memory");
 }
-__device__ __forceinline__ void tm_st(unsigned at, const float (&x)[4])
-{
-    asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};\n" ::"r"(at), "f"(x[0]), "f"(x[1]),
-                 "f"(x[2]), "f"(x[3])
-                 : "memory");
-}
-__device__ __forceinline__ void tm_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;\n" ::: "memory"); }
-
 // As res_iterate (whose comments hold here), for runs of kTmRows rows.  tmem: the block's base.
 __device__ __forceinline__ unsigned res_iterate_tm(const ResParams<float> &q, ResShared<float> &sh,
                                                    unsigned ep, unsigned tmem)

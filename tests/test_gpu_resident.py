@@ -135,7 +135,7 @@ def test_resident_solve_matches_the_oracle(g, monkeypatch):
         assert np.linalg.norm(p.cpu().numpy() - po.ravel()) <= 1e-10 * np.linalg.norm(po)
 
 
-@pytest.mark.parametrize("nth,nz,K,precision", [(513, 5, 1, 0), (2052, 3, 1, 1), (512, 257, 16, 0)])
+@pytest.mark.parametrize("nth,nz,K,precision", [(513, 5, 1, 0), (2052, 3, 1, 1), (640, 300, 9, 0)])
 def test_grids_beyond_the_resident_solve_take_the_phase_kernels(g, monkeypatch, nth, nz, K, precision):
     _, arrs = system(nth, nz, K, 5)
     p, it, rel, info = solve(g, monkeypatch, nth, nz, K, arrs, precision=precision, allow=True)
@@ -143,6 +143,40 @@ def test_grids_beyond_the_resident_solve_take_the_phase_kernels(g, monkeypatch, 
                                  variant=1001003 if precision == 0 else 1001004)
     assert not resident(info) and info["status"] == infr["status"]
     assert rel_l2(p, ref) <= 1e-10
+
+
+# runs of 8 rows, and in FP64 of 16: partial runs and partial segments of a row (of one thread
+# only), many runs a column, ASSOR-I's diagonal (not constant in the scaled form), the
+# asynchronized criterion, a warm start
+@pytest.mark.parametrize("nth,nz,K,precision,precond,criterion,rows", [
+    (1000, 250, 4, 0, 1, 0, 8), (700, 300, 4, 0, 2, 0, 8), (512, 250, 9, 0, 1, 1, 8),
+    (60, 1000, 15, 0, 1, 0, 8), (640, 256, 5, 0, 0, 0, 16), (1024, 250, 9, 0, 1, 0, 16),
+    (514, 256, 9, 0, 1, 1, 16),
+    (640, 200, 9, 1, 1, 0, 8), (1028, 127, 9, 1, 1, 0, 8), (2048, 120, 9, 1, 0, 0, 8),
+    (128, 1000, 15, 1, 1, 0, 8),
+])
+def test_resident_runs_in_tensor_memory_match_phase_kernels(g, monkeypatch, nth, nz, K, precision,
+                                                            precond, criterion, rows):
+    _, arrs = system(nth, nz, K, nth + nz)
+    kw = dict(precision=precision, precond=precond, criterion=criterion)
+    forced = 1001003 if precision == 0 else 1001004
+    p, it, rel, info = solve(g, monkeypatch, nth, nz, K, arrs, **kw)
+    ref, itr, _, infr = solve(g, monkeypatch, nth, nz, K, arrs, variant=forced, **kw)
+    assert info["kernel_variant"] == 50000000 + (2000 if precision == 0 else 4000) + 10 * rows
+    assert not resident(infr)
+    assert rel <= (1e-11 if precision == 0 else 1e-12)
+    # (recurrences of thousands of iterations pass the tolerance on a plateau: on 700 x 300 with
+    # ASSOR-I the phase kernels of one and of two columns a lane differ by 19)
+    assert abs(it - itr) <= 2 + itr // 50
+    assert rel_l2(p, ref) <= 4e-10
+    p2, it2, _, _ = solve(g, monkeypatch, nth, nz, K, arrs, **kw)
+    assert it2 == it and torch.equal(p, p2)
+    p3, it3, _, _ = solve(g, monkeypatch, nth, nz, K, arrs, start=p, **{**kw, "eps": 1e-10})
+    assert it3 == 0 and torch.equal(p3, p)
+    start = ref * (1.0 + 1e-3)
+    a, ita, _, _ = solve(g, monkeypatch, nth, nz, K, arrs, start=start, **kw)
+    b, itb, _, _ = solve(g, monkeypatch, nth, nz, K, arrs, start=start, variant=forced, **kw)
+    assert abs(ita - itb) <= 2 + itb // 50 and rel_l2(a, b) <= 4e-10
 
 
 # runs of 16 rows (id 50004160): whole and partial ones, one and two of them a column, rows that
