@@ -11,16 +11,18 @@
 //
 // Host code cannot use the array's name as a device address, so the address is
 // looked up once per device with cudaGetSymbolAddress and passed to the kernels.
-// The loop is driven from the host in chunks (no graph, no events, no pinned
-// staging), so nothing here allocates.  The kernels are the untuned default
-// variants of the joint solver (two columns per lane when n_theta is even and
-// the arrays are 16-byte aligned, else one), with the one-level reduction of
-// the phase sums.
+// Systems that fit on the SMs take the resident PCG (gmaf_resident.cuh), a run in
+// one launch; its kernels are loaded with the array, at the first call.  For the others the loop is driven
+// from the host in chunks (no graph, no events, no pinned staging), so nothing
+// here allocates.  Their kernels are the untuned default variants of the joint
+// solver (two columns per lane when n_theta is even and the arrays are 16-byte
+// aligned, else one), with the one-level reduction of the phase sums.
 #include <mutex>
 
 #include "gmaf_internal.cuh"
 #include "gmaf_pcg_kernels.cuh"
 #include "gmaf_pcg_host.cuh"
+#include "gmaf_resident.h"
 
 namespace gmaf {
 
@@ -42,11 +44,12 @@ static_assert(kNaPart + kNaPartBytes <= kNaVec, "partials slot");
 
 std::mutex g_na_mutex;
 void *g_na_base[kNaMaxDevices];
+bool g_na_coop[kNaMaxDevices];         // the resident kernels are loaded there
 
 size_t round256(size_t b) { return (b + 255) & ~size_t(255); }
 
 // Device address of the scratch array on the current device (looked up once per device).
-int noalloc_base(char **out)
+int noalloc_base(char **out, cudaStream_t s, bool *coop)
 {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
@@ -57,8 +60,19 @@ int noalloc_base(char **out)
         void *ptr = nullptr;
         e = cudaGetSymbolAddress(&ptr, g_noalloc_scratch);
         if (e != cudaSuccess || ptr == nullptr) return cuda_status(e == cudaSuccess ? cudaErrorInvalidSymbol : e);
+        int has = 0;
+        e = cudaDeviceGetAttribute(&has, cudaDevAttrCooperativeLaunch, dev);
+        if (e == cudaSuccess && has) {
+            e = res_preload64(s);
+            if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+            g_na_coop[dev] = e == cudaSuccess;
+            if (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorNotSupported) e = cudaSuccess;
+        }
+        cudaGetLastError();
+        if (e != cudaSuccess) return cuda_status(e);
         g_na_base[dev] = ptr;
     }
+    *coop = g_na_coop[dev];
     *out = (char *)g_na_base[dev];
     return GMAF_OK;
 }
@@ -83,13 +97,14 @@ extern "C" int gmaf_solve_joint_noalloc(const gmaf_grid *grid, int32_t n_cond, c
     if ((long long)nth * nz > (1LL << 31) - 1 || kNaVec + 7 * vec > (size_t)GMAF_NOALLOC_SCRATCH_BYTES)
         return GMAF_OUT_OF_MEMORY;
     char *base = nullptr;
-    int st = noalloc_base(&base);
+    cudaStream_t s = (cudaStream_t)cuda_stream;
+    bool coop = false;
+    int st = noalloc_base(&base, s, &coop);
     if (st != GMAF_OK) return st;
     int dev = 0, num_sms = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&num_sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return cuda_status(e);
-    cudaStream_t s = (cudaStream_t)cuda_stream;
     // Once work is on the stream, an error return first waits for it, so that the
     // call leaves nothing running on the shared array (result ignored: the error
     // being returned is the one that counts).
@@ -160,6 +175,49 @@ extern "C" int gmaf_solve_joint_noalloc(const gmaf_grid *grid, int32_t n_cond, c
     int slots[kMaxCond];
     for (int k = 0; k < K; ++k) slots[k] = k;
 
+    // The resident run's part of the array: omega/D (or ASSOR-I's diagonal), the residual of a
+    // restart, x and the scaled matrix where it has them, words and rows of the exchanges.
+    ResPlan pl{};
+    ResParams<double> q{};
+    bool res = coop && opts->max_iter < (1 << 29) && res_plan<double>(nth, nz, K, vec_ok(h), num_sms, &pl);
+    char *coef = nullptr;
+    if (res) {
+        const bool with_d = opts->precond == 2;
+        size_t o = kNaVec + (!pl.tm || with_d ? 1 : 0) * vec;
+        q.r_in = (const double *)(base + o);
+        o += vec;
+        q.x = (double *)(base + o);
+        if (pl.tm && pl.o_x < 0) o += vec;
+        coef = base + o;
+        if (pl.tm) o += res_scaled_bytes(N, with_d);
+        q.words = (unsigned long long *)(base + o);
+        o += 2 * kResGroupWords * 8;
+        q.halo = (unsigned long long *)(base + o);
+        o += round256(pl.halo_bytes);
+        res = o <= (size_t)GMAF_NOALLOC_SCRATCH_BYTES;
+    }
+    if (res) {
+        q.nth = nth;
+        q.nz = nz;
+        q.n = n;
+        q.groups = 1;
+        q.mask = 1;
+        res_fill<double>(pl, &q);
+        q.precond = h.precond;
+        q.zero_init = opts->zero_init;
+        q.max_iter = opts->max_iter;
+        q.eps = opts->eps;
+        q.mode = kResFresh;
+        q.D = q.D64 = D;
+        q.invD = invD;
+        q.aE = q.aE64 = aE;
+        q.aN = q.aN64 = aN;
+        q.cslot = cslot;
+        q.b = S;
+        q.p = q.p64 = p;
+        q.sc = dsc;
+    }
+
     // The array keeps the previous call's contents: clear the scalars and the
     // reduction tickets, which must start at zero.  The copies below come from
     // pageable (stack) memory and have consumed their sources when they return.
@@ -169,7 +227,28 @@ extern "C" int gmaf_solve_joint_noalloc(const gmaf_grid *grid, int32_t n_cond, c
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(d_desc, &h, sizeof(h), cudaMemcpyHostToDevice, s);
     if (e != cudaSuccess) return fail(e);
-    diag_inverse64(opts, D, aE, aN, nth, nz, N, invD, num_sms, s);
+    if (!res || !pl.tm || opts->precond == 2) diag_inverse64(opts, D, aE, aN, nth, nz, N, invD, num_sms, s);
+    if (res) {
+        e = cudaMemsetAsync(q.words, 0, 2 * kResGroupWords * 8 + round256(pl.halo_bytes), s);
+        if (e != cudaSuccess) return fail(e);
+        if (pl.tm) {
+            st = res_scaled(D, aE, aN, opts->precond == 2 ? invD : nullptr, opts->precond == 1 ? opts->omega : 1.0,
+                            nth, nz, N, coef, num_sms, s, &q);
+            if (st != GMAF_OK) {
+                fail(cudaSuccess);
+                return st;
+            }
+        }
+        e = res_launch<double>(pl, q, s);
+        if (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorNotSupported) {
+            // the blocks cannot all be resident here: the phase kernels
+            cudaGetLastError();
+            res = false;
+            diag_inverse64(opts, D, aE, aN, nth, nz, N, invD, num_sms, s);
+        } else if (e != cudaSuccess) {
+            return fail(e);
+        }
+    }
 
     Scalars hs{}, hr{};
     int restarted = 0;
@@ -177,30 +256,41 @@ extern "C" int gmaf_solve_joint_noalloc(const gmaf_grid *grid, int32_t n_cond, c
     int status = GMAF_NOT_CONVERGED;
     double true_rel = 0.0;
     for (;;) {
-        k_reset<<<1, 32, 0, s>>>(dsc, keep ? 1 : 0);
-        if (init_r) k_init_r<double><<<grid_s, kThreads, 0, s>>>(d_desc);
-        e = launch<double>(ks.b_init, grid_b, d_desc, s, ks.smem_b);
-        if (e == cudaSuccess) e = cudaGetLastError();
-        if (e != cudaSuccess) return fail(e);
-        const int chunk = 16;
-        for (int it = 0; it <= opts->max_iter + chunk; it += chunk) {
-            int done = 0;
-            e = cudaMemcpyAsync(&done, &dsc->done, sizeof(int), cudaMemcpyDeviceToHost, s);
-            if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-            if (e != cudaSuccess) return fail(e);
-            if (done) break;
-            for (int q = 0; q < chunk && e == cudaSuccess; ++q) {
-                e = launch<double>(ks.a, grid_a, d_desc, s, ks.smem_a);
-                if (e == cudaSuccess) e = launch<double>(ks.b, grid_b, d_desc, s, ks.smem_b);
+        if (res) {
+            // (the first run is under way)
+            if (keep) {
+                q.mode = kResRestart;
+                q.epoch = 2u * (unsigned)opts->max_iter + 4u;
+                q.words += kResGroupWords;
+                e = res_launch<double>(pl, q, s);
+                if (e != cudaSuccess) return fail(e);
             }
+        } else {
+            k_reset<<<1, 32, 0, s>>>(dsc, keep ? 1 : 0);
+            if (init_r) k_init_r<double><<<grid_s, kThreads, 0, s>>>(d_desc);
+            e = launch<double>(ks.b_init, grid_b, d_desc, s, ks.smem_b);
+            if (e == cudaSuccess) e = cudaGetLastError();
             if (e != cudaSuccess) return fail(e);
+            const int chunk = 16;
+            for (int it = 0; it <= opts->max_iter + chunk; it += chunk) {
+                int done = 0;
+                e = cudaMemcpyAsync(&done, &dsc->done, sizeof(int), cudaMemcpyDeviceToHost, s);
+                if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+                if (e != cudaSuccess) return fail(e);
+                if (done) break;
+                for (int q = 0; q < chunk && e == cudaSuccess; ++q) {
+                    e = launch<double>(ks.a, grid_a, d_desc, s, ks.smem_a);
+                    if (e == cudaSuccess) e = launch<double>(ks.b, grid_b, d_desc, s, ks.smem_b);
+                }
+                if (e != cudaSuccess) return fail(e);
+            }
+            k_finalize<double><<<grid_s, kThreads, 0, s>>>(d_desc);
         }
-        k_finalize<double><<<grid_s, kThreads, 0, s>>>(d_desc);
         e = cudaMemcpyAsync(&hs, dsc, sizeof(Scalars), cudaMemcpyDeviceToHost, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
         if (e != cudaSuccess) return fail(e);
         // true residual S - A p into r[iter & 1], where a restart reads it
-        rd.r = h.r[hs.iter & 1];
+        rd.r = res ? const_cast<double *>(q.r_in) : h.r[hs.iter & 1];
         e = cudaMemcpyAsync(d_rdesc, &rd, sizeof(rd), cudaMemcpyHostToDevice, s);
         if (e != cudaSuccess) return fail(e);
         k_resid64<<<grid_s, kThreads, 0, s>>>(d_rdesc);

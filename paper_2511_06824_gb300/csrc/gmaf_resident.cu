@@ -84,7 +84,7 @@ static long long round16(long long b) { return (b + 15) / 16 * 16; }
 // x; the tensor memory forms keep x and 1 / s^2 (1), the first rows' aE (2) or omega/D (3).
 static bool layout(ResPlan &pl, int nth, int sz, bool *cs)
 {
-    const int kMax = 226 * 1024;         // of the 227 KB a block can have (a little is static)
+    const int kMax = kResSmem;
     const bool scaled = pl.tm == 1 || pl.tm == 2;
     const long long row = (long long)kResThreads * pl.vec * sz, field = pl.rr * row;
     const long long rows = (long long)(scaled ? res_tm_rows(pl.nrr, sz) : 6 + 2 * pl.nrr) * nth * sz;
@@ -213,6 +213,27 @@ cudaError_t res_launch(const ResPlan &pl, ResParams<T> &q, cudaStream_t s)
     if (e != cudaSuccess) return e;
     void *args[] = {(void *)&q};
     return cudaLaunchCooperativeKernel(pl.fn, dim3(pl.grid), dim3(pl.threads + 32), args, pl.smem, s);
+}
+
+cudaError_t res_preload64(cudaStream_t s)
+{
+    cudaFuncAttributes fa;
+    cudaError_t e = cudaFuncGetAttributes(&fa, (const void *)k_res_scaled);
+    for (int k = 0; k < 18 && e == cudaSuccess; ++k) {
+        const int vec = 1 + (k & 1), rr = 1 << (k >> 2);
+        const void *fn = k >= 16 ? res_kernel_s(8, k == 16 ? 8 : 16) : res_kernel_f64(vec, rr, (k & 2) != 0);
+        if (!fn) continue;
+        ResPlan pl{};
+        pl.fn = fn;
+        pl.grid = 1;
+        pl.threads = 32;
+        pl.smem = kResSmem;
+        ResParams<double> q{};
+        q.bpc = q.groups = 1;           // (mask 0: the group does not run)
+        q.threads = pl.threads;
+        e = res_launch<double>(pl, q, s);
+    }
+    return e;
 }
 
 template bool res_plan<float>(int, int, int, bool, int, ResPlan *);

@@ -11,6 +11,7 @@ namespace gmaf {
 
 constexpr int kResThreads = 512;        // most threads that own rows (one more warp exchanges)
 constexpr int kResMaxBlocks = 160;      // most blocks of a launch (they are counted in a byte)
+constexpr int kResSmem = 225 * 1024;    // shared memory of a block (of 227 KB; 1.1 KB more is static)
 constexpr int kResGroupWords = 16;      // 8-byte words of a group of blocks for its sums
 constexpr int kResSegs = kResThreads / 32;   // segments of 32 threads in a row, at most
 constexpr int kResVariant = 50000000;   // gmaf_solve_info.kernel_variant: + 1000 VEC + 10 RR
@@ -97,6 +98,10 @@ const void *res_kernel_s(int size, int rr);
 size_t res_scaled_bytes(long long m, bool with_d);
 int res_scaled(const double *D, const double *aE, const double *aN, const double *minv, double w, int nth, int nz,
                long long m, void *coef, int num_sms, cudaStream_t s, ResParams<double> *q);
+
+// Loads every FP64 kernel on the current device and launches it once without work, so that later
+// launches allocate neither code nor local memory.
+cudaError_t res_preload64(cudaStream_t s);
 
 // Cooperative launch; cudaErrorCooperativeLaunchTooLarge when the blocks cannot all
 // be resident (a partitioned GPU): the caller then takes the phase kernels.
