@@ -308,14 +308,10 @@ extern "C" int gmaf_solve_joint_noalloc(const gmaf_grid *grid, int32_t n_cond, c
             status = hs.status != 0 ? hs.status : hr.status;
             break;
         }
-        if ((hs.converged || hs.zero_rhs) && true_rel <= 10.0 * opts->eps) {
-            status = GMAF_OK;
-            break;
-        }
-        if (restarted || hs.iter >= opts->max_iter) {
-            status = GMAF_NOT_CONVERGED;
-            break;
-        }
+        const bool end = hs.converged || hs.zero_rhs;
+        status = end && true_rel <= 10.0 * opts->eps ? GMAF_OK : GMAF_NOT_CONVERGED;
+        if (end && true_rel <= (res && !restarted ? res_limit(pl.tm) : 10.0) * opts->eps) break;
+        if (restarted || hs.iter >= opts->max_iter) break;
         restarted = 1;
         keep = true;
         init_r = false;

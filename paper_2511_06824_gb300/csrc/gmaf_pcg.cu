@@ -1037,10 +1037,9 @@ static int solve_resident64(gmaf_ctx *ctx, ResRun<double> &rr, int K, const int 
                 true_rel[k] = 0.0;
             }
             if (h[k].status != 0 || h[G + k].status != 0) continue;
-            if ((h[k].converged || h[k].zero_rhs) && true_rel[k] <= 10.0 * opts->eps) {
-                ok[k] = 1;
-                continue;
-            }
+            const bool end = h[k].converged || h[k].zero_rhs;
+            ok[k] = end && true_rel[k] <= 10.0 * opts->eps;
+            if (end && true_rel[k] <= (restarted[k] ? 10.0 : res_limit(rr.pl.tm)) * opts->eps) continue;
             if (restarted[k] || h[k].iter >= opts->max_iter) continue;
             restarted[k] = 1;
             again |= 1ull << k;

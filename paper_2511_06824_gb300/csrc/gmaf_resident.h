@@ -23,6 +23,13 @@ __host__ __device__ constexpr int res_tm(int rr, int vec, int size)
 {
     return rr * vec * size <= 64 ? 0 : rr == 8 ? 1 : size == 8 ? 2 : 3;
 }
+// How far above the tolerance the true residual of a first FP64 run may be.  In the scaled forms
+// the recurrence is that of a matrix rounded to the last bits and drifts from the true residual
+// (by 4e-14 of the right-hand side on 512 x 256 cells, 2e-13 on 1000 x 250, 1e-11 on 511 x 5,
+// where the unscaled forms drift by a tenth of it), so a run that ends well above is restarted
+// from its true residual, which takes that out; the unscaled forms keep the phase kernels' limit.
+constexpr double res_limit(int tm) { return tm ? 1.25 : 10.0; }
+
 // Rows of n_theta values that a block of form 1 or 2 keeps in shared memory.
 __host__ __device__ constexpr int res_tm_rows(int nrr, int size) { return size == 8 ? 4 + 3 * nrr : 5 + 4 * nrr; }
 
