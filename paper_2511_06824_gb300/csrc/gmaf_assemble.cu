@@ -110,7 +110,9 @@ __device__ __forceinline__ double texture_depth(const Lattice &lt, const Reach &
 {
     const double r2 = __dmul_rn(lt.r, lt.r);
     bool in = false;
-    for (int c = 0; c < z.n; ++c) in = in || __dadd_rn((z.odd >> c) & 1 ? q[1] : q[0], z.dz2[c]) < r2;
+    // (squares: not negative, so that the integers compare as they do, off the FP64 pipe)
+    for (int c = 0; c < z.n; ++c)
+        in = in || __double_as_longlong(__dadd_rn((z.odd >> c) & 1 ? q[1] : q[0], z.dz2[c])) < __double_as_longlong(r2);
     return in ? lt.depth : 0.0;
 }
 
@@ -120,17 +122,19 @@ struct FilmPt {
     double X, Y, rho;
 };
 
-__device__ __forceinline__ FilmPt film_pt(const Geom &g, const double *e, double ct, double st,
-                                          double t)
+__device__ __forceinline__ FilmPt film_at(double Rc, double ex, double ey, double ct, double st)
 {
-    const double Rc = g.Rk + g.c;
-    const double ex = e[0] + (e[2] - e[0]) * t;
-    const double ey = e[1] + (e[3] - e[1]) * t;
     FilmPt f;
     f.X = Rc * ct - ex;
     f.Y = Rc * st - ey;
     f.rho = sqrt(f.X * f.X + f.Y * f.Y);
     return f;
+}
+
+__device__ __forceinline__ FilmPt film_pt(const Geom &g, const double *e, double ct, double st,
+                                          double t)
+{
+    return film_at(g.Rk + g.c, e[0] + (e[2] - e[0]) * t, e[1] + (e[3] - e[1]) * t, ct, st);
 }
 
 // ------------------------------------------------------------------ trig table
@@ -233,7 +237,9 @@ static Batches make_batches(int ncond, const gmaf_state *conds, bool simplified)
 // Lane 0 of a warp works on the column west of the warp's 31 others: its a_E is the
 // neighbour's a_W, so that the diagonal is complete without a second pass.  The
 // results are bitwise those of evaluating every cell and condition by itself.
-// 1024 x 512 x 9 cells of a Picard step's conditions: 1486 us that way, 738 us now.
+// 1024 x 512 x 9 cells of a Picard step's conditions: 1486 us that way, 703 us now (738 before
+// what depends on the row only was formed once a block, and conditions of one film shared a
+// reciprocal).
 
 // a / b, correctly rounded, from y = 1 / b (correctly rounded): the product and two
 // corrections by the residual (Markstein), for a divisor that is the same for all cells.
@@ -244,12 +250,21 @@ __device__ __forceinline__ double quotient(double a, double b, double y)
     return fma(y, fma(-b, t, a), t);
 }
 
+// Far from the ends of the exponent's range, where quotient() is that of the division.
+__device__ __forceinline__ bool mid_range(double x)
+{
+    const int e = (__double2hiint(x) >> 20) & 0x7ff;
+    return e > 300 && e < 1700;
+}
+
 constexpr int kAsmWarps = 4, kAsmRows = 32;
 
 // Per row of a block: the axial coordinate of its centre and north face, and what of the
-// texture is in reach of them.
+// texture is in reach of them; the eccentricities there, and the rates of each condition at
+// the centre.
 struct AsmRow {
-    double tc, tn;
+    double tc, exc, eyc, exn, eyn;
+    double exd[kBatch], eyd[kBatch];
     Reach c, n;
 };
 
@@ -280,7 +295,7 @@ __global__ void __launch_bounds__(kAsmWarps * 32) k_assemble(Geom g, Batches bt,
     if (i >= g.nth) i = g.nth - 1;
 
     const double Ub = -g.v;
-    const double inv12mu = 1.0 / (12.0 * g.mu);
+    const double inv12mu = 1.0 / (12.0 * g.mu), Rc = g.Rk + g.c;
     int contact = 0;
     const double cc = trig[i], sc = trig[g.nth + i];
     const double ce = trig[2 * g.nth + i], se = trig[3 * g.nth + i];
@@ -298,9 +313,22 @@ __global__ void __launch_bounds__(kAsmWarps * 32) k_assemble(Geom g, Batches bt,
                 const int j = j0 + q / 2;
                 const double z = q & 1 ? ((double)j + 1.0) * g.dz : ((double)j + 0.5) * g.dz;
                 AsmRow &r = row[q / 2];
-                (q & 1 ? r.tn : r.tc) = z * g.invL;
+                const double t = z * g.invL;
+                (q & 1 ? r.exn : r.exc) = st[0][0] + (st[0][2] - st[0][0]) * t;
+                (q & 1 ? r.eyn : r.eyc) = st[0][1] + (st[0][3] - st[0][1]) * t;
+                if (!(q & 1)) r.tc = t;
                 lattice_reach(g.lt, z, q & 1 ? r.n : r.c);
             }
+        }
+        __syncthreads();
+        // (the multiply-adds of S are written out, so that it does not depend on how the
+        // compiler pairs these terms)
+        for (int q = tid; q < nb * (j1 - j0); q += blockDim.x) {
+            const int k = q / (j1 - j0);
+            AsmRow &r = row[q - k * (j1 - j0)];
+            const double rest = 1.0 - r.tc;
+            r.exd[k] = __fma_rn(st[k][4], rest, __dmul_rn(st[k][6], r.tc));
+            r.eyd[k] = __fma_rn(st[k][5], rest, __dmul_rn(st[k][7], r.tc));
         }
         __syncthreads();
         if (i0 >= g.nth) continue;                                  // (a whole warp)
@@ -314,9 +342,9 @@ __global__ void __launch_bounds__(kAsmWarps * 32) k_assemble(Geom g, Batches bt,
         }
         for (int j = j0; j < j1; ++j) {
             const AsmRow &rw = row[j - j0];
-            const FilmPt fe = film_pt(g, st[0], ce, se, rw.tc);
-            const FilmPt fn = film_pt(g, st[0], cc, sc, rw.tn);
-            const FilmPt fc = film_pt(g, st[0], cc, sc, rw.tc);
+            const FilmPt fe = film_at(Rc, rw.exc, rw.eyc, ce, se);
+            const FilmPt fn = film_at(Rc, rw.exn, rw.eyn, cc, sc);
+            const FilmPt fc = film_at(Rc, rw.exc, rw.eyc, cc, sc);
             const double he = (fe.rho - g.Rk) + texture_depth(g.lt, rw.c, qe);
             const double hn = (fn.rho - g.Rk) + texture_depth(g.lt, rw.n, qc);
             contact |= (he <= 0.0) | (hn <= 0.0);
@@ -342,15 +370,15 @@ __global__ void __launch_bounds__(kAsmWarps * 32) k_assemble(Geom g, Batches bt,
             const double diag = east + west + north + south_n + aB;
             if (own) {
                 const size_t P = (size_t)j * g.nth + i;
+                const double wedge = __dmul_rn(-(Ub / 2.0), __dsub_rn(hn, hs));
+                // (several conditions: one reciprocal for their quotients)
+                const bool shared = nb > 1 && mid_range(fc.rho);
+                const double inv_rho = shared ? 1.0 / fc.rho : 0.0;
                 for (int k = 0; k < nb; ++k) {
-                    // dh/dt = -(X/rho) dex/dt - (Y/rho) dey/dt at the cell centre; the
-                    // multiply-adds are written out, so that S does not depend on how
-                    // the compiler pairs these terms
-                    const double rest = 1.0 - rw.tc;
-                    const double exd = __fma_rn(st[k][4], rest, __dmul_rn(st[k][6], rw.tc));
-                    const double eyd = __fma_rn(st[k][5], rest, __dmul_rn(st[k][7], rw.tc));
-                    const double hdot = -__fma_rn(fc.X, exd, __dmul_rn(fc.Y, eyd)) / fc.rho;
-                    const double wedge = __dmul_rn(-(Ub / 2.0), __dsub_rn(hn, hs));
+                    // dh/dt = -(X/rho) dex/dt - (Y/rho) dey/dt at the cell centre
+                    const double a = __fma_rn(fc.X, rw.exd[k], __dmul_rn(fc.Y, rw.eyd[k]));
+                    const bool zero = (__double_as_longlong(a) << 1) == 0;
+                    const double hdot = -(shared && (mid_range(a) || zero) ? quotient(a, fc.rho, inv_rho) : a / fc.rho);
                     const double squeeze = __dmul_rn(__dmul_rn(hdot, g.dx), g.dz);
                     S[(size_t)bt.idx[blockIdx.z][k] * (size_t)n + P] =
                         __dadd_rn(__fma_rn(wedge, g.dx, -squeeze), sB);
