@@ -404,9 +404,10 @@ int launch_assemble(const Geom &g, int ncond, const double *conds, const int *co
 {
     const Batches bt = make_batches(ncond, conds_host, simplified);
     const int strips = (g.nth + 31 * kAsmWarps - 1) / (31 * kAsmWarps);
-    // rows a block marches: 32, fewer while there are fewer than about 8 blocks an SM
+    // rows a block marches: 32, fewer while there are fewer than about 4 blocks an SM (512 x 256
+    // x 9: 247 us a call, with 8 blocks an SM 275, with 1 330)
     int rows = kAsmRows;
-    while (rows > 2 && (long long)strips * ((g.nz + rows - 1) / rows) * bt.n < 152 * 8) rows /= 2;
+    while (rows > 2 && (long long)strips * ((g.nz + rows - 1) / rows) * bt.n < 152 * 4) rows /= 2;
     const int segs = (g.nz + rows - 1) / rows;
     const dim3 grid(strips, segs < 65535 ? segs : 65535, bt.n);
     k_assemble<<<grid, kAsmWarps * 32, 0, s>>>(g, bt, conds, coef_slot, D, aE, aN, S, trig, rows,
@@ -636,10 +637,11 @@ int launch_loads(const Geom &g, int ncond, const double *conds, const double *p,
     const Batches bt = make_batches(ncond, conds_host, simplified);
     const int er = g.nz + 1, strips = (g.nth + kLoadThreads - 1) / kLoadThreads;
     // segments of rows: short ones on small grids, so that every SM has work, but no more
-    // blocks a condition than there are partial sums
+    // blocks a condition than there are partial sums (512 x 256 x 9: 116 us a call with 4 blocks
+    // an SM, 134 with 8, 188 with 1)
     const long long most = 2LL * num_sms;
     int rows = kLoadRows;
-    while (rows > 2 && (long long)strips * ((er + rows - 1) / rows) * bt.n < 8LL * num_sms &&
+    while (rows > 2 && (long long)strips * ((er + rows - 1) / rows) * bt.n < 4LL * num_sms &&
            (long long)strips * ((er + rows / 2 - 1) / (rows / 2)) <= most)
         rows /= 2;
     const long long units = (long long)strips * ((er + rows - 1) / rows);
@@ -652,59 +654,57 @@ int launch_loads(const Geom &g, int ncond, const double *conds, const double *p,
 
 // result layout (doubles): [0..11] loads of condition 0, [12..59] J (6 x 8),
 // [60..63] G, [64..71] new state, [72] status (0 ok, -4 singular).
+//
+// One warp: the entries of a step side by side, the 4 x 4 system eliminated a row and column a
+// lane.  All of it is chains of FP64 divisions (570 cycles) and multiply-adds (64): 43 us on one
+// thread, 9 us so.
 __global__ void k_picard(const double *__restrict__ loads, PicardIn in, double dt, double d_e,
                          double d_edot, double L, double *__restrict__ result)
 {
-    if (threadIdx.x != 0) return;
+    __shared__ double F[9][6], J[6][8], Je[4][4], Jd[4][4], G[4], A[4][5];
+    const int lane = threadIdx.x;
     const double *base = in.base, *e_prev = in.e_prev, *F_ext = in.F_ext;
     const bool simp = in.simplified != 0;
     const int K = simp ? 5 : 9;
-    double F[9][6];
-    for (int k = 0; k < K; ++k)
-        for (int c = 0; c < 6; ++c) F[k][c] = loads[k * 12 + c] + loads[k * 12 + 6 + c];
+    for (int q = lane; q < K * 6; q += 32) F[q / 6][q % 6] = loads[q / 6 * 12 + q % 6] + loads[q / 6 * 12 + 6 + q % 6];
+    __syncwarp();
     // load Jacobian by forward differences (Eq. 2.13-2.14); the simplified scheme
     // forms only the rate columns, from its conditions 1..4
-    double J[6][8];
-    for (int r = 0; r < 6; ++r)
-        for (int c = 0; c < 8; ++c) {
-            if (simp)
-                J[r][c] = c < 4 ? 0.0 : (F[1 + (c - 4)][r] - F[0][r]) / d_edot;
-            else
-                J[r][c] = (F[1 + c][r] - F[0][r]) / (c < 4 ? d_e : d_edot);
-        }
-    // generalized force of the linear tilt: (Fx - My/L, Fy + Mx/L, My/L, -Mx/L)
-    auto gen = [L](const double *f, double *gout) {
-        gout[0] = f[0] - f[4] / L;
-        gout[1] = f[1] + f[3] / L;
-        gout[2] = f[4] / L;
-        gout[3] = -f[3] / L;
-    };
-    double G[4];
-    gen(F[0], G);
-    for (int q = 0; q < 4; ++q) G[q] += F_ext[q];
-    double Je[4][4], Jd[4][4];
-    for (int c = 0; c < 4; ++c) {
-        double col[6], gg[4];
-        for (int r = 0; r < 6; ++r) col[r] = J[r][c];
-        gen(col, gg);
-        for (int r = 0; r < 4; ++r) Je[r][c] = gg[r];
-        for (int r = 0; r < 6; ++r) col[r] = J[r][4 + c];
-        gen(col, gg);
-        for (int r = 0; r < 4; ++r) Jd[r][c] = gg[r];
+    for (int q = lane; q < 48; q += 32) {
+        const int r = q / 8, c = q % 8;
+        if (simp)
+            J[r][c] = c < 4 ? 0.0 : (F[1 + (c - 4)][r] - F[0][r]) / d_edot;
+        else
+            J[r][c] = (F[1 + c][r] - F[0][r]) / (c < 4 ? d_e : d_edot);
     }
+    __syncwarp();
+    // generalized force of the linear tilt: (Fx - My/L, Fy + Mx/L, My/L, -Mx/L)
+    auto gen = [L](int r, double fx, double fy, double mx, double my) {
+        const double t = (r == 0 || r == 2 ? my : mx) / L;
+        return r == 0 ? fx - t : r == 1 ? fy + t : r == 2 ? t : -t;
+    };
+    {
+        const int r = lane & 3, c = (lane >> 2) & 3, at = c + (lane < 16 ? 0 : 4);
+        (lane < 16 ? Je : Jd)[r][c] = gen(r, J[0][at], J[1][at], J[3][at], J[4][at]);
+        if (lane < 4) G[r] = gen(r, F[0][0], F[0][1], F[0][3], F[0][4]) + F_ext[r];
+    }
+    __syncwarp();
     // general: (J_edot + dt J_e) delta = -G - J_e (e_prev + dt edot - e);
     // simplified (Eq. 2.20-2.21): J_edot delta = -G
-    double A[4][5];
-    for (int r = 0; r < 4; ++r) {
+    if (lane < 16) {
+        const int r = lane >> 2, c = lane & 3;
+        A[r][c] = simp ? Jd[r][c] : Jd[r][c] + dt * Je[r][c];
+    } else if (lane < 20) {
+        const int r = lane - 16;
         double s = 0.0;
-        for (int c = 0; c < 4; ++c) {
-            A[r][c] = simp ? Jd[r][c] : Jd[r][c] + dt * Je[r][c];
-            if (!simp) s += Je[r][c] * (e_prev[c] + dt * base[4 + c] - base[c]);
-        }
+        if (!simp)
+            for (int c = 0; c < 4; ++c) s += Je[r][c] * (e_prev[c] + dt * base[4 + c] - base[c]);
         A[r][4] = -G[r] - s;
     }
+    __syncwarp();
     int status = 0;
     // Gaussian elimination with partial pivoting
+    const int row = lane / 5, col = lane - 5 * row;
     for (int k = 0; k < 4 && status == 0; ++k) {
         int best = k;
         for (int r = k + 1; r < 4; ++r)
@@ -713,36 +713,41 @@ __global__ void k_picard(const double *__restrict__ loads, PicardIn in, double d
             status = -4;
             break;
         }
-        if (best != k)
-            for (int c = 0; c < 5; ++c) {
-                const double t = A[k][c];
-                A[k][c] = A[best][c];
-                A[best][c] = t;
-            }
-        for (int r = k + 1; r < 4; ++r) {
-            const double f = A[r][k] / A[k][k];
-            for (int c = k; c < 5; ++c) A[r][c] -= f * A[k][c];
+        double a = 0.0;
+        if (lane < 20) a = A[row == k ? best : row == best ? k : row][col];
+        __syncwarp();
+        if (lane < 20) A[row][col] = a;
+        __syncwarp();
+        if (lane < 20 && row > k && col >= k) {
+            const double f = A[row][k] / A[k][k];
+            a -= f * A[k][col];
         }
+        __syncwarp();
+        if (lane < 20) A[row][col] = a;
+        __syncwarp();
     }
+    for (int q = lane; q < 12; q += 32) result[q] = loads[q];
+    for (int q = lane; q < 48; q += 32) result[12 + q] = J[q / 8][q % 8];
+    if (lane < 4) result[60 + lane] = G[lane];
     double delta[4] = {0, 0, 0, 0};
     if (status == 0) {
+#pragma unroll
         for (int r = 3; r >= 0; --r) {
             double s = A[r][4];
+#pragma unroll
             for (int c = r + 1; c < 4; ++c) s -= A[r][c] * delta[c];
             delta[r] = s / A[r][r];
         }
     }
-    for (int q = 0; q < 12; ++q) result[q] = loads[q];
-    for (int r = 0; r < 6; ++r)
-        for (int c = 0; c < 8; ++c) result[12 + r * 8 + c] = J[r][c];
-    for (int q = 0; q < 4; ++q) result[60 + q] = G[q];
+#pragma unroll
     for (int q = 0; q < 4; ++q) {
+        if (lane != q) continue;
         const double ed = base[4 + q] + delta[q];
         result[64 + 4 + q] = ed;
         // general: e = e_prev + dt edot_new; simplified: e += dt delta (Eq. 2.22)
         result[64 + q] = simp ? base[q] + dt * delta[q] : e_prev[q] + dt * ed;
     }
-    result[72] = (double)status;
+    if (lane == 0) result[72] = (double)status;
 }
 
 int launch_picard_update(const double *loads, const PicardIn &in, double dt, double d_e,
