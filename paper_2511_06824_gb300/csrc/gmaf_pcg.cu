@@ -1305,6 +1305,8 @@ int solve_joint_device(gmaf_ctx *ctx, int nth, int nz, int K, int nslots, const 
         q.scale = &dsc_outer->scale;
         q.p64 = p;
         q.r64 = (double *)ctx->buf[B_R64];
+        q.pairs64 = nth % 2 == 0;
+        for (const double *a : {D, aE, aN, S, (const double *)p}) q.pairs64 = q.pairs64 && aligned16(a);
         q.continued = ctx->mixed_restart ? 0 : 1;
         q.inner_floor = q.continued ? ctx->reliable_delta : ctx->inner_floor;
         q.max_outer = q.continued ? kMaxOuterContinued : kMaxOuterRestart;

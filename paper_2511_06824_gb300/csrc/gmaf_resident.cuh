@@ -942,21 +942,37 @@ struct ResRows {
         }
     }
 
+    // VEC doubles from global memory: 16 bytes at a time where every row allows it.
+    __device__ __forceinline__ void ld64(const double *p, double (&x)[VEC]) const
+    {
+        if (VEC > 1 && q.pairs64) {
+#pragma unroll
+            for (int e = 0; e + 1 < VEC; e += 2) {
+                const double2 t = *reinterpret_cast<const double2 *>(p + e);
+                x[e] = t.x;
+                x[e + 1] = t.y;
+            }
+        } else {
+#pragma unroll
+            for (int e = 0; e < VEC; ++e) x[e] = p[e];
+        }
+    }
+
     // Mixed precision: this thread's rows of r64 = S - A p64, and the warps' sums of r64 r64 and
-    // S S.  The rows of the blocks below and above come as flagged words.
+    // S S.  The rows of the blocks below and above come as flagged words.  A row of p serves three
+    // rows' equations from registers, its neighbours' columns come by shuffle: 5 values a cell are
+    // loaded, not 11 (1024 x 512 x 9 cells: 145 us before, 123 us so; its FP64 operations take 70).
     __device__ __forceinline__ void residual(unsigned ep)
     {
-        double *const p64 = q.p64 + off;
+        const double *const p64 = q.p64 + off;
         unsigned long long *const row64 = q.halo64 + ((size_t)blockIdx.x * 2 * nth + c) * 2;
         double pS64[VEC], pN64[VEC], rr = 0.0, ss = 0.0;
         if (hasS) {
-#pragma unroll
-            for (int e = 0; e < VEC; ++e) pS64[e] = p64[e];
+            ld64(p64, pS64);
             ll_put<VEC>(row64, pS64, ep);
         }
         if (hasN) {
-#pragma unroll
-            for (int e = 0; e < VEC; ++e) pN64[e] = p64[(size_t)(nr - 1) * nth + e];
+            ld64(p64 + (size_t)(nr - 1) * nth, pN64);
             ll_put<VEC>(row64 + 2 * nth, pN64, ep);
         }
         bar_sync_n(1, TC);                          // p64 of the block's other threads
@@ -966,21 +982,76 @@ struct ResRows {
         if (hasS) ok = ll_get<VEC>(row64 - 2 * nth, pS64, ep);
         if (hasN) ok = ll_get<VEC>(row64 + 4 * nth, pN64, ep) && ok;
         if (!ok) sh.halo_failed = 1;
+        // p on this row and the one below, a_N of the row below
+        double pc[VEC], ps[VEC], nS[VEC];
+#pragma unroll
+        for (int e = 0; e < VEC; ++e) {
+            pc[e] = nS[e] = 0.0;
+            ps[e] = pS64[e];
+        }
+        const int jl = j0 + lr0;
+        if (act) {
+            ld64(p64, pc);
+            if (jl > 0) ld64(q.aN64 + coff - nth, nS);
+            if (jl > 0 && !hasS) ld64(p64 - nth, ps);
+        }
+        __syncwarp();
 #pragma unroll 1
-        for (int k = 0; k < nr; ++k) {
-            const int j = j0 + lr0 + k;
+        for (int k = 0; k < RR; ++k) {
+            const int j = jl + k;
+            const bool in = k < nr;
             const size_t go = (size_t)k * nth;
-            const double *p = p64 + go, *aE = q.aE64 + coff + go, *aN = q.aN64 + coff + go;
+            double pn[VEC], aE[VEC], aN[VEC], D[VEC], S[VEC];
+#pragma unroll
+            for (int e = 0; e < VEC; ++e) aE[e] = aN[e] = D[e] = S[e] = pn[e] = 0.0;
+            double pW = 0.0, pE = 0.0, aW = 0.0;
+            if (in) {
+                ld64(q.aE64 + coff + go, aE);
+                ld64(q.aN64 + coff + go, aN);
+                ld64(q.D64 + coff + go, D);
+                ld64(q.S64 + off + go, S);
+                if (hasN && k == nr - 1) {
+#pragma unroll
+                    for (int e = 0; e < VEC; ++e) pn[e] = pN64[e];
+                } else if (j < nz - 1) {
+                    ld64(p64 + go + nth, pn);
+                }
+                if (segw) {
+                    const int iw = atw ? nth - 1 : -1;
+                    pW = p64[go + iw];
+                    aW = q.aE64[coff + go + iw];
+                }
+                if (sege) pE = p64[go + (ate ? 1 - nth + VEC - 1 : VEC)];
+            }
+            const double wp = __shfl_up_sync(0xffffffffu, pc[VEC - 1], 1);
+            const double wa = __shfl_up_sync(0xffffffffu, aE[VEC - 1], 1);
+            const double ep_ = __shfl_down_sync(0xffffffffu, pc[0], 1);
+            if (!segw) {
+                pW = wp;
+                aW = wa;
+            }
+            if (!sege) pE = ep_;
+            if (in) {
+                double r64[VEC];
+#pragma unroll
+                for (int e = 0; e < VEC; ++e) {
+                    double ap = D[e] * pc[e] - aE[e] * (e < VEC - 1 ? pc[e + 1] : pE) -
+                                (e > 0 ? aE[e - 1] : aW) * (e > 0 ? pc[e - 1] : pW);
+                    if (j < nz - 1) ap -= aN[e] * pn[e];
+                    if (j > 0) ap -= nS[e] * ps[e];
+                    const double rv = S[e] - ap;
+                    r64[e] = rv;
+                    rr = fma(rv, rv, rr);
+                    ss = fma(S[e], S[e], ss);
+                }
+#pragma unroll
+                for (int e = 0; e < VEC; ++e) q.r64[off + go + e] = r64[e];
+            }
 #pragma unroll
             for (int e = 0; e < VEC; ++e) {
-                const int ie = c + e == nth - 1 ? 1 - nth + e : e + 1, iw = c + e == 0 ? nth - 1 : e - 1;
-                double ap = q.D64[coff + go + e] * p[e] - aE[e] * p[ie] - aE[iw] * p[iw];
-                if (j < nz - 1) ap -= aN[e] * (hasN && k == nr - 1 ? pN64[e] : p[nth + e]);
-                if (j > 0) ap -= aN[e - nth] * (hasS && k == 0 ? pS64[e] : p[e - nth]);
-                const double s = q.S64[off + go + e], rv = s - ap;
-                q.r64[off + go + e] = rv;
-                rr = fma(rv, rv, rr);
-                ss = fma(s, s, ss);
+                ps[e] = pc[e];
+                pc[e] = pn[e];
+                nS[e] = aN[e];
             }
         }
         const double x[2] = {rr, ss};

@@ -68,6 +68,7 @@ struct ResParams {
     int ri;                             //   and rows of a run whose omega/D is in shared memory
     double inner_floor;                 // reduction of a run
     int continued, max_outer;
+    int pairs64;                        // the rows of the FP64 arrays start on 16-byte boundaries
     unsigned long long *words;          // [groups][kResGroupWords], zero at the start of the run
     unsigned long long *halo;           // flagged rows, [blocks][4]
     int halo_row;                       // 8-byte words of one flagged row
