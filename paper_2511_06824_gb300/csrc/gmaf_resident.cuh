@@ -311,12 +311,12 @@ __device__ __forceinline__ ResLimbs res_limbs(const ResTerm<float> &t, int e)
 // exchange before.  Words of one kind are added to again only after an exchange of
 // another kind, which no block completes before all have read these.
 
-enum ResWord { kWordUV = 0, kWordRZ = 4, kWordMaxCount = 8, kWordMax = 9, kWordR64 = 12 };
+enum ResWord { kWordUV = 0, kWordRZ = 4, kWordMaxCount = 8, kWordMax = 9, kWordMeet = 11, kWordR64 = 12 };
 static_assert(kWordR64 + 4 <= kResGroupWords, "words of a group");
 
 struct ResSums {
     unsigned long long *w;              // the group's words (zero at the start of the run)
-    unsigned long long prev[10], prev_max;
+    unsigned long long prev[10], prev_max, prev_meet;
     int nb, e[5];                       // blocks; exponent expected of u.v, r.z, r.r, and of
                                         // r.r and S.S in FP64 (0: not known)
     unsigned turn;
@@ -349,6 +349,20 @@ __device__ __forceinline__ bool res_max_exp(ResSums &x, const int (&mine)[NV], i
         }
     }
     return false;
+}
+
+// All blocks of the group have come, and what their threads stored before is visible.
+__device__ __forceinline__ bool res_meet(ResSums &x, int lane)
+{
+    __threadfence();
+    __syncwarp();
+    if (lane == 0) res_red(x.w + kWordMeet, 1ull);
+    bool ok = false;
+    for (unsigned k = 0; k < kResSpin && !ok; ++k)
+        ok = ll_ld1(x.w + kWordMeet) - x.prev_meet == (unsigned long long)x.nb;
+    x.prev_meet += (unsigned long long)x.nb;
+    __threadfence();
+    return __all_sync(0xffffffffu, ok) != 0;
 }
 
 // The totals over the group's blocks of NV values, of which each lane holds one term
@@ -476,6 +490,7 @@ struct ResShared {
     ResTerm<T> part[2][kResThreads / 32];           // the warps' sums
     ResTerm<double> part64[2][kResThreads / 32];    // (of the FP64 residual)
     double alpha, beta;
+    double red64[kThreads / 32];        // (norm of the FP64 residual)
     double unit, back;                  // mixed precision: 1 / ||r64||; scale ||r64||, which takes x to p
     int done, stop, halo_failed;
 };
@@ -662,11 +677,25 @@ struct ResExchange {
             {
                 const ResTerm<double> mine[2] = {gather64(0), gather64(1)};
                 double tot[2];
-                if (!res_totals<2, double>(sums, 2, mine, lane, tot) || sh.halo_failed) {
+                bool ok = res_totals<2, double>(sums, 2, mine, lane, tot) && !sh.halo_failed;
+                // ||r64|| in the order of k_resid64, to the last bit: it is the unit of the FP32
+                // run and the factor of x in p (see res_norm_warps)
+                double nn = tot[0];
+                if (q.grid64) {
+                    ok = res_meet(sums, lane) && ok;
+                    bar_sync_n(2, all);
+                    bar_sync_n(2, all);
+                    ok = res_meet(sums, lane) && ok;
+                    bar_sync_n(2, all);
+                    bar_sync_n(2, all);
+                    nn = 0.0;
+                    for (int w = 0; w < kThreads / 32; ++w) nn += sh.red64[w];
+                }
+                rnorm = sqrt(nn);
+                if (!ok) {
                     verdict = GMAF_TIMEOUT;
                     stop = true;
                 } else {
-                    rnorm = sqrt(tot[0]);
                     const double nS = sqrt(tot[1]);
                     true_rel = nS > 0.0 ? rnorm / nS : 0.0;
                     if (!finite_d(tot[0]) || !finite_d(tot[1]) || !finite_d(true_rel)) {
@@ -716,7 +745,7 @@ struct ResExchange {
             if (status != 0) verdict = status;
             stop = status != 0 || seg == 0;     // (the row threads still add x to p)
             if (stop) {
-                bar_sync_n(2, all);             // the residual's sums: not wanted
+                for (int k = 0; k < (q.grid64 ? 5 : 1); ++k) bar_sync_n(2, all);    // the residual's sums: not wanted
                 if (lane == 0) sh.stop = 1;
                 bar_sync_n(2, all);
                 break;
@@ -1533,10 +1562,70 @@ __device__ __noinline__ void res_setup(const ResParams<T> &q)
 {
     ResRows<T, VEC, RR, CS>(q, res_shared<T>()).setup();
 }
+// The norm of r64 as k_resid64 adds it up: a run of the refinement then works on the numbers that
+// it would have with the phase kernels, bit for bit (the last bit of the norm is a bit of p, whose
+// rounding is all that r64 is made of towards the end; with the norm as the blocks' exact sum a
+// Picard step's Jacobian on 512 x 256 cells moved by 1e-10 to 1e-9, so it does by 1e-12).  First the sums of that kernel's warps,
+// then, in every block, what its blocks and its last block add.
+static __device__ __noinline__ void res_norm_warps(const ResParams<float> &q)
+{
+    const int warps = q.threads >> 5, lane = threadIdx.x & 31, total = q.grid64 * (kThreads / 32);
+    const long long N = q.n * (long long)(gridDim.x / q.bpc), stride = (long long)q.grid64 * kThreads;
+    for (int w = blockIdx.x * warps + (threadIdx.x >> 5); w < total; w += gridDim.x * warps) {
+        double s = 0.0;
+        for (long long g = (long long)w * 32 + lane; g < N; g += 4 * stride) {
+            double v[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) v[k] = g + k * stride < N ? __ldcg(q.r64 + g + k * stride) : 0.0;
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                if (g + k * stride < N) s = fma(v[k], v[k], s);
+        }
+        s = warp_sum_d(s);
+        if (lane == 0) __stcg(q.warps64 + w, s);
+    }
+    __threadfence();
+}
+static __device__ __noinline__ void res_norm_total(const ResParams<float> &q, double *red)
+{
+    constexpr int W = kThreads / 32;
+    const int warps = q.threads >> 5, lane = threadIdx.x & 31;
+    for (int w = threadIdx.x >> 5; w < W; w += warps) {
+        double s = 0.0;
+        for (int b = w * 32 + lane; b < q.grid64; b += kThreads) {
+            double x[W], t = 0.0;
+#pragma unroll
+            for (int k = 0; k < W; ++k) x[k] = __ldcg(q.warps64 + b * W + k);
+#pragma unroll
+            for (int k = 0; k < W; ++k) t += x[k];
+            s += t;
+        }
+        s = warp_sum_d(s);
+        if (lane == 0) red[w] = s;
+    }
+}
+
 template <typename T, int VEC, int RR, bool CS>
 __device__ __noinline__ void res_residual(const ResParams<T> &q, unsigned ep)
 {
     ResRows<T, VEC, RR, CS>(q, res_shared<T>()).residual(ep);
+}
+
+// The meetings of the row threads with refine() between a residual and the next run.
+__device__ __forceinline__ void res_decide(const ResParams<float> &q, ResShared<float> &sh)
+{
+    const int all = q.threads + 32;
+    if (q.grid64) {
+        __threadfence();
+        bar_sync_n(2, all);
+        bar_sync_n(2, all);
+        res_norm_warps(q);
+        bar_sync_n(2, all);
+        bar_sync_n(2, all);
+        res_norm_total(q, sh.red64);
+    }
+    bar_sync_n(2, all);
+    bar_sync_n(2, all);
 }
 
 template <typename T, int VEC, int RR, bool CS>
@@ -1557,8 +1646,7 @@ __global__ void __launch_bounds__(kResThreads + 32, 1) k_resident(const __grid_c
 #pragma unroll 1
         for (;;) {
             res_residual<T, VEC, RR, CS>(q, ++ep);
-            bar_sync_n(2, q.threads + 32);
-            bar_sync_n(2, q.threads + 32);
+            res_decide(q, sh);
             if (sh.stop) break;
             ep = res_iterate<T, VEC, RR, CS>(q, sh, ep);
         }

@@ -562,8 +562,7 @@ static __global__ void __launch_bounds__(kResThreads + 32, 1) k_resident_tm(cons
 #pragma unroll 1
     for (;;) {
         res_residual<T, 4, kTmRows, false>(q, ++ep);
-        bar_sync_n(2, q.threads + 32);
-        bar_sync_n(2, q.threads + 32);
+        res_decide(q, sh);
         if (sh.stop) break;
         ep = res_iterate_tm(q, sh, ep, tmem);
     }
