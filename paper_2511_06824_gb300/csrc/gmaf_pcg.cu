@@ -1305,8 +1305,7 @@ int solve_joint_device(gmaf_ctx *ctx, int nth, int nz, int K, int nslots, const 
         q.scale = &dsc_outer->scale;
         q.p64 = p;
         q.r64 = (double *)ctx->buf[B_R64];
-        // (runs of 16 rows rebuild the diagonal and so have numbers of their own)
-        q.grid64 = rr.pl.tm == 3 ? 0 : gs;
+        q.grid64 = gs;
         GMAF_TRY(ensure(ctx, B_PART, (size_t)gs * (kThreads / 32) * sizeof(double)));
         q.warps64 = (double *)ctx->buf[B_PART];
         q.pairs64 = nth % 2 == 0;

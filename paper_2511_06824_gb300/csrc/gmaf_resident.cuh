@@ -505,7 +505,8 @@ __device__ __forceinline__ ResShared<T> &res_shared()
 
 // The warp that takes no rows: adds the block's sums, exchanges them, updates the
 // scalars (finish_a and finish_b of the phase kernels) and decides when to stop.
-template <typename T>
+// NORM: ||r64|| in k_resid64's order (res_norm_warps).
+template <typename T, bool NORM>
 struct ResExchange {
     const ResParams<T> &q;
     ResShared<T> &sh;
@@ -681,7 +682,7 @@ struct ResExchange {
                 // ||r64|| in the order of k_resid64, to the last bit: it is the unit of the FP32
                 // run and the factor of x in p (see res_norm_warps)
                 double nn = tot[0];
-                if (q.grid64) {
+                if constexpr (NORM) {
                     ok = res_meet(sums, lane) && ok;
                     bar_sync_n(2, all);
                     bar_sync_n(2, all);
@@ -745,7 +746,7 @@ struct ResExchange {
             if (status != 0) verdict = status;
             stop = status != 0 || seg == 0;     // (the row threads still add x to p)
             if (stop) {
-                for (int k = 0; k < (q.grid64 ? 5 : 1); ++k) bar_sync_n(2, all);    // the residual's sums: not wanted
+                for (int k = 0; k < (NORM ? 5 : 1); ++k) bar_sync_n(2, all);    // the residual's sums: not wanted
                 if (lane == 0) sh.stop = 1;
                 bar_sync_n(2, all);
                 break;
@@ -760,11 +761,11 @@ struct ResExchange {
     }
 };
 
-template <typename T>
+template <typename T, bool NORM = true>
 __device__ __forceinline__ void res_exchange_warp(const ResParams<T> &q, ResShared<T> &sh, Scalars *sc,
                                                   int grp, int g0, int nb, int lane)
 {
-    ResExchange<T> x{q, sh, q.threads + 32, q.threads / 32, lane};
+    ResExchange<T, NORM> x{q, sh, q.threads + 32, q.threads / 32, lane};
     x.sums = ResSums{};
     x.sums.w = q.words + (size_t)grp * kResGroupWords;
     x.sums.nb = nb;
@@ -1566,7 +1567,8 @@ __device__ __noinline__ void res_setup(const ResParams<T> &q)
 // it would have with the phase kernels, bit for bit (the last bit of the norm is a bit of p, whose
 // rounding is all that r64 is made of towards the end; with the norm as the blocks' exact sum a
 // Picard step's Jacobian on 512 x 256 cells moved by 1e-10 to 1e-9, so it does by 1e-12).  First the sums of that kernel's warps,
-// then, in every block, what its blocks and its last block add.
+// then, in every block, what its blocks and its last block add: 16 us a refinement on 256 x 128 x 9
+// cells, 19 on 512 x 256 x 9 (several warps of that kernel at a time: no faster).
 static __device__ __noinline__ void res_norm_warps(const ResParams<float> &q)
 {
     const int warps = q.threads >> 5, lane = threadIdx.x & 31, total = q.grid64 * (kThreads / 32);
@@ -1612,10 +1614,11 @@ __device__ __noinline__ void res_residual(const ResParams<T> &q, unsigned ep)
 }
 
 // The meetings of the row threads with refine() between a residual and the next run.
+template <bool NORM>
 __device__ __forceinline__ void res_decide(const ResParams<float> &q, ResShared<float> &sh)
 {
     const int all = q.threads + 32;
-    if (q.grid64) {
+    if constexpr (NORM) {
         __threadfence();
         bar_sync_n(2, all);
         bar_sync_n(2, all);
@@ -1646,7 +1649,7 @@ __global__ void __launch_bounds__(kResThreads + 32, 1) k_resident(const __grid_c
 #pragma unroll 1
         for (;;) {
             res_residual<T, VEC, RR, CS>(q, ++ep);
-            res_decide(q, sh);
+            res_decide<true>(q, sh);
             if (sh.stop) break;
             ep = res_iterate<T, VEC, RR, CS>(q, sh, ep);
         }

@@ -68,7 +68,7 @@ struct ResParams {
     int ri;                             //   and rows of a run whose omega/D is in shared memory
     double inner_floor;                 // reduction of a run
     int continued, max_outer;
-    int grid64;                         // blocks of k_resid64 on this system (0: not asked for), and sums of
+    int grid64;                         // blocks of k_resid64 on this system, and sums of
     double *warps64;                    // its warps: the norm is added up in that kernel's order
     int pairs64;                        // the rows of the FP64 arrays start on 16-byte boundaries
     unsigned long long *words;          // [groups][kResGroupWords], zero at the start of the run

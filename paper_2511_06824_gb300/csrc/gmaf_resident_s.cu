@@ -793,7 +793,7 @@ static __global__ void __launch_bounds__(kResThreads + 32, 1) k_resident_s(const
 #pragma unroll 1
         for (;;) {
             res_residual<T, 4, RR, false>(q, ++ep);
-            res_decide(q, sh);
+            res_decide<true>(q, sh);
             if (sh.stop) break;
             ep = res_iterate_s<T, RR, TM>(q, sh, ep, tmem);
         }

@@ -7,7 +7,7 @@
 // The diagonal is rebuilt from the couplings, as in the phase A of gmaf_drec.cu, to save
 // its traffic.
 //
-// On 9 conditions of 1024 x 512 cells an iteration takes 39.4 us (A 16.7, B 21.6: the
+// On 9 conditions of 1024 x 512 cells an iteration takes 37 to 39 us (A 16.8, B 21.2: the
 // coefficients' and x's 175 MB from L2 at 4.5 TB/s, and two exchanges of 1.5 us), the
 // phase kernels take 68.3; on 9 of 700 x 300 it is 33.3 against 56.7.
 #include "gmaf_resident.cuh"
@@ -538,7 +538,7 @@ static __global__ void __launch_bounds__(kResThreads + 32, 1) k_resident_tm(cons
     ResShared<T> &sh = res_shared<T>();
     __shared__ unsigned s_tmem;
     if ((int)threadIdx.x >= q.threads) {
-        res_exchange_warp<T>(q, sh, q.sc, 0, 0, (int)gridDim.x, threadIdx.x & 31);
+        res_exchange_warp<T, false>(q, sh, q.sc, 0, 0, (int)gridDim.x, threadIdx.x & 31);
         return;
     }
     // omega/D of the first rows stays in shared memory
@@ -562,7 +562,7 @@ static __global__ void __launch_bounds__(kResThreads + 32, 1) k_resident_tm(cons
 #pragma unroll 1
     for (;;) {
         res_residual<T, 4, kTmRows, false>(q, ++ep);
-        res_decide(q, sh);
+        res_decide<false>(q, sh);
         if (sh.stop) break;
         ep = res_iterate_tm(q, sh, ep, tmem);
     }
