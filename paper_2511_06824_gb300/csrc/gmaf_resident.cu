@@ -7,16 +7,17 @@
 
 namespace gmaf {
 
-const void *res_kernel_f64(int vec, int rr, bool cs)
+ResKernel res_kernel_f64(int vec, int rr, bool cs)
 {
-#define GMAF_RES(V, R)                                                              \
-    if (vec == V && rr == R)                                                        \
-        return cs ? (const void *)k_resident<double, V, R, true>                    \
-                  : (const void *)k_resident<double, V, R, false>;
+#define GMAF_RES(V, R)                                              \
+    if (vec == V && rr == R) {                                      \
+        if (cs) GMAF_RES_KERNEL((k_resident<double, V, R, true>));  \
+        GMAF_RES_KERNEL((k_resident<double, V, R, false>));         \
+    }
     GMAF_RES(1, 1) GMAF_RES(1, 2) GMAF_RES(1, 4) GMAF_RES(1, 8)
     GMAF_RES(2, 1) GMAF_RES(2, 2) GMAF_RES(2, 4)
 #undef GMAF_RES
-    return nullptr;
+    return {};
 }
 
 // ------------------------------------------------------------------ scaled matrix
@@ -164,13 +165,13 @@ bool res_plan(int nth, int nz, int K, bool vec_ok, int num_sms, ResPlan *out)
             t.nseg = (int)((ncg + 31) / 32);
             bool cs = false;
             if (!layout(t, nth, sz, &cs)) continue;
-            t.fn = t.tm == 3   ? res_kernel_tm()
-                   : t.tm      ? res_kernel_s(sz, rr)
-                   : sz == 4   ? res_kernel_f32(vec, rr, cs)
-                               : res_kernel_f64(vec, rr, cs);
+            t.k = t.tm == 3   ? res_kernel_tm()
+                  : t.tm      ? res_kernel_s(sz, rr)
+                  : sz == 4   ? res_kernel_f32(vec, rr, cs)
+                              : res_kernel_f64(vec, rr, cs);
             const long long warps = ((long long)P * t.nrr + 31) / 32;
             const long long cells = (warps + 3) / 4 * vec * rr;
-            if (t.fn && (!best || cells < best)) {
+            if (t.k.fn && (!best || cells < best)) {
                 best = cells;
                 pl = t;
             }
@@ -209,10 +210,9 @@ void res_fill(const ResPlan &pl, ResParams<T> *q)
 template <typename T>
 cudaError_t res_launch(const ResPlan &pl, ResParams<T> &q, cudaStream_t s)
 {
-    cudaError_t e = cudaFuncSetAttribute(pl.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, pl.smem);
-    if (e != cudaSuccess) return e;
+    smem_optin(*pl.k.opted, pl.k.fn, kResSmem);
     void *args[] = {(void *)&q};
-    return cudaLaunchCooperativeKernel(pl.fn, dim3(pl.grid), dim3(pl.threads + 32), args, pl.smem, s);
+    return cudaLaunchCooperativeKernel(pl.k.fn, dim3(pl.grid), dim3(pl.threads + 32), args, pl.smem, s);
 }
 
 cudaError_t res_preload64(cudaStream_t s)
@@ -221,10 +221,9 @@ cudaError_t res_preload64(cudaStream_t s)
     cudaError_t e = cudaFuncGetAttributes(&fa, (const void *)k_res_scaled);
     for (int k = 0; k < 18 && e == cudaSuccess; ++k) {
         const int vec = 1 + (k & 1), rr = 1 << (k >> 2);
-        const void *fn = k >= 16 ? res_kernel_s(8, k == 16 ? 8 : 16) : res_kernel_f64(vec, rr, (k & 2) != 0);
-        if (!fn) continue;
         ResPlan pl{};
-        pl.fn = fn;
+        pl.k = k >= 16 ? res_kernel_s(8, k == 16 ? 8 : 16) : res_kernel_f64(vec, rr, (k & 2) != 0);
+        if (!pl.k.fn) continue;
         pl.grid = 1;
         pl.threads = 32;
         pl.smem = kResSmem;

@@ -1659,4 +1659,11 @@ __global__ void __launch_bounds__(kResThreads + 32, 1) k_resident(const __grid_c
     }
 }
 
+// Returns a kernel, named in parentheses, with its record of devices.
+#define GMAF_RES_KERNEL(fn)                                                                          \
+    do {                                                                                             \
+        static std::atomic<unsigned long long> opted{0};                                             \
+        return ResKernel{(const void *)fn, &opted};                                                  \
+    } while (0)
+
 }  // namespace gmaf

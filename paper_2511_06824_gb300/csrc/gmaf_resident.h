@@ -3,6 +3,7 @@
 // allocation-free solve (gmaf_noalloc.cu).  Internal; not part of the ABI.
 #pragma once
 
+#include <atomic>
 #include <cstddef>
 
 #include "gmaf_internal.cuh"
@@ -78,8 +79,16 @@ struct ResParams {
                                         // of FP64 residuals (added to; or null)
 };
 
-struct ResPlan {
+// A kernel and the devices on which it is opted in to kResSmem.  (The attribute is the kernel's,
+// not the launch's: set to a plan's own size before each launch, it was lowered between another
+// thread's setting and launch, which then failed.)
+struct ResKernel {
     const void *fn;
+    std::atomic<unsigned long long> *opted;
+};
+
+struct ResPlan {
+    ResKernel k;
     int grid, smem, vec, rr;
     int bpc, threads, P, ncg, nrr, rows, nseg;
     int o_rows, o_edge, o_x, o_q, o_keep, keep, ri;
@@ -97,11 +106,11 @@ template <typename T>
 void res_fill(const ResPlan &pl, ResParams<T> *q);
 
 // Kernel of a plan (compiled for T in a translation unit of its own).
-const void *res_kernel_f32(int vec, int rr, bool cs);
-const void *res_kernel_f64(int vec, int rr, bool cs);
-const void *res_kernel_tm();
+ResKernel res_kernel_f32(int vec, int rr, bool cs);
+ResKernel res_kernel_f64(int vec, int rr, bool cs);
+ResKernel res_kernel_tm();
 constexpr int kTmRows = 16;             // rows of a run of k_resident_tm
-const void *res_kernel_s(int size, int rr);
+ResKernel res_kernel_s(int size, int rr);
 
 // The scaled FP64 matrix of m cells: coef (res_scaled_bytes) receives aE, aN, Q, s and (with minv)
 // D.  minv: the preconditioner's diagonal, null for w / D.

@@ -804,10 +804,11 @@ static __global__ void __launch_bounds__(kResThreads + 32, 1) k_resident_s(const
     if (threadIdx.x < 32) tm_free(tmem);
 }
 
-const void *res_kernel_s(int size, int rr)
+ResKernel res_kernel_s(int size, int rr)
 {
-    if (size == 4) return (const void *)k_resident_s<float, 8, 1>;
-    return rr == 8 ? (const void *)k_resident_s<double, 8, 1> : (const void *)k_resident_s<double, 16, 2>;
+    if (size == 4) GMAF_RES_KERNEL((k_resident_s<float, 8, 1>));
+    if (rr == 8) GMAF_RES_KERNEL((k_resident_s<double, 8, 1>));
+    GMAF_RES_KERNEL((k_resident_s<double, 16, 2>));
 }
 
 }  // namespace gmaf

@@ -570,6 +570,6 @@ static __global__ void __launch_bounds__(kResThreads + 32, 1) k_resident_tm(cons
     if (threadIdx.x < 32) tm_free(tmem);
 }
 
-const void *res_kernel_tm() { return (const void *)k_resident_tm; }
+ResKernel res_kernel_tm() { GMAF_RES_KERNEL((k_resident_tm)); }
 
 }  // namespace gmaf

@@ -1,0 +1,89 @@
+"""Where the resident PCG ends or has to give way: whatever it cannot do, the phase kernels do,
+with the results that they had, and what one call does leaves others as they were."""
+import threading
+
+import numpy as np
+import pytest
+
+import oracle
+from paper_2511_06824_gb300 import inputs
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+PHYS = inputs.phys_vector()
+
+
+@pytest.fixture(scope="module")
+def g():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2511_06824_gb300 import build, gmaf
+    build.build()
+    gmaf.load()
+    return gmaf
+
+
+def resident(info):
+    """Whether the solve took the resident kernel (ids 50000000 + 1000 VEC + 10 RR)."""
+    return info["kernel_variant"] // 10000000 == 5
+
+
+def system(nth, nz, K, seed):
+    rng = np.random.default_rng(seed)
+    tex = inputs.dimple_texture(rng)
+    st, *arrs = oracle.assemble_joint(nth, nz, PHYS, tex, [inputs.random_state(rng) for _ in range(K)])
+    assert st == 0
+    return [torch.from_numpy(np.ascontiguousarray(a).ravel()).cuda() for a in arrs]
+
+
+def solve(g, nth, nz, K, arrs, budget=0, start=None, allow=None, **opts):
+    """Status, iterations, true residual, details and solution, in a context of its own."""
+    p = torch.full((K * nth * nz,), 5.0, dtype=torch.float64, device="cuda")
+    if start is not None:
+        p.copy_(start)
+        opts["zero_init"] = 0
+    with g.Context(hbm_budget_bytes=budget) as c:
+        st, it, rel = g.gmaf_solve_joint(c.handle, nth, nz, K, *arrs, p, g.solver_opts(**{"eps": 1e-10, **opts}),
+                                         allow=allow or (g.GMAF_OK,))
+        info = g.gmaf_last_solve_info(c.handle)
+    return st, it, rel, info, p
+
+
+def rel_l2(a, b):
+    return float(torch.linalg.norm(a - b) / torch.linalg.norm(b))
+
+
+def test_threads_with_contexts_of_their_own(g):
+    """Threads, each with a context and a stream, solve grids that take the same kernel with
+    different amounts of shared memory, over and over: no launch fails, and every result is bit for
+    bit that of the solve alone."""
+    shapes = [(60, 40, 9), (128, 64, 4), (512, 304, 1), (60, 40, 2)]
+    kw = dict(eps=1e-6, max_iter=2)
+    arrs = [system(*s, 3) for s in shapes]
+    refs = [solve(g, *s, a, allow=(g.GMAF_NOT_CONVERGED,), **kw)[4] for s, a in zip(shapes, arrs)]
+    failed = []
+
+    def work(q):
+        try:
+            stream = torch.cuda.Stream()
+            p = torch.zeros_like(refs[q])
+            torch.cuda.synchronize()
+            with g.Context(stream=stream.cuda_stream) as c:
+                for _ in range(4000):
+                    st, _, _ = g.gmaf_solve_joint(c.handle, *shapes[q], *arrs[q], p, g.solver_opts(**kw),
+                                                  allow=tuple(range(-8, 1)))
+                    if st != g.GMAF_NOT_CONVERGED:
+                        failed.append((q, g.status_string(st)))
+                        break
+                if not resident(g.gmaf_last_solve_info(c.handle)) or not torch.equal(p, refs[q]):
+                    failed.append((q, "result"))
+        except Exception as e:                      # noqa: BLE001
+            failed.append((q, repr(e)))
+
+    ts = [threading.Thread(target=work, args=(q,)) for q in range(len(shapes))]
+    for t in ts:
+        t.start()
+    for t in ts:
+        t.join()
+    assert not failed, failed
