@@ -289,6 +289,14 @@ extern "C" int gmaf_solve_joint_noalloc(const gmaf_grid *grid, int32_t n_cond, c
         e = cudaMemcpyAsync(&hs, dsc, sizeof(Scalars), cudaMemcpyDeviceToHost, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
         if (e != cudaSuccess) return fail(e);
+        if (res && hs.status == kResBeyond) {
+            // not for the resident run: the phase kernels, from p
+            res = keep = false;
+            init_r = true;
+            restarted = 0;
+            diag_inverse64(opts, D, aE, aN, nth, nz, N, invD, num_sms, s);
+            continue;
+        }
         // true residual S - A p into r[iter & 1], where a restart reads it
         rd.r = res ? const_cast<double *>(q.r_in) : h.r[hs.iter & 1];
         e = cudaMemcpyAsync(d_rdesc, &rd, sizeof(rd), cudaMemcpyHostToDevice, s);

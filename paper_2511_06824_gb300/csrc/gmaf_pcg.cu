@@ -908,7 +908,7 @@ static void res_setup(gmaf_ctx *ctx, ResRun<T> &rr, int nth, int nz, int K, bool
 }
 
 // One launch; max_iter - start iterations at most.  *off: the blocks cannot all be
-// resident here, nothing was launched.
+// resident here, nothing was launched; the phase kernels take the solve.
 template <typename T>
 static int res_run(gmaf_ctx *ctx, ResRun<T> &rr, long long most_iterations, bool *off)
 {
@@ -962,7 +962,8 @@ static int res_run(gmaf_ctx *ctx, ResRun<T> &rr, long long most_iterations, bool
 // FP64, either criterion: the joint system is one group of blocks, under the
 // asynchronized criterion each condition is one (its own scalars, its own end).
 // After a run each group gets the FP64 true-residual check, and once, if that
-// fails, a restart from the true residual.
+// fails, a restart from the true residual.  *off: the phase kernels have to solve
+// the system (from p, where that is the start).
 static int solve_resident64(gmaf_ctx *ctx, ResRun<double> &rr, int K, const int *cslot_host,
                             const double *S, double *p, const gmaf_solver_opts *opts,
                             gmaf_solve_info *info, bool *off)
@@ -1030,6 +1031,10 @@ static int solve_resident64(gmaf_ctx *ctx, ResRun<double> &rr, int K, const int 
         unsigned long long again = 0;
         for (int k = 0; k < G; ++k) {
             if (!((ran >> k) & 1ull)) continue;
+            if (h[k].status == kResBeyond) {
+                *off = true;
+                return GMAF_OK;
+            }
             true_rel[k] = h[G + k].true_rel;
             if (h[k].zero_rhs) {
                 GMAF_CUDA(cudaMemsetAsync(p + (long long)k * n, 0,
@@ -1168,6 +1173,7 @@ int solve_joint_device(gmaf_ctx *ctx, int nth, int nz, int K, int nslots, const 
             bool off = false;
             const int st = solve_resident64(ctx, rr, K, cslot_host, S, p, opts, info, &off);
             if (!off) return st;
+            GMAF_CUDA(cudaMemsetAsync(dsc_outer, 0, sizeof(Scalars), s));
         }
         const int bufs[] = {B_R0, B_R1, B_U0, B_U1, B_Z, B_V};
         for (int b : bufs) GMAF_TRY(ensure(ctx, b, (size_t)N * sizeof(double)));
@@ -1315,8 +1321,8 @@ int solve_joint_device(gmaf_ctx *ctx, int nth, int nz, int K, int nslots, const 
         q.max_outer = q.continued ? kMaxOuterContinued : kMaxOuterRestart;
         bool off = false;
         GMAF_TRY(res_run<float>(ctx, rr, (long long)opts->max_iter + 2 * q.max_outer, &off));
-        if (!off) {
-            GMAF_TRY(read_scalars(ctx, dsc, hsc));
+        if (!off) GMAF_TRY(read_scalars(ctx, dsc, hsc));
+        if (!off && hsc->status != kResBeyond) {
             inf.iterations = hsc->iter;
             inf.iterations_sum = hsc->iter * K;
             inf.outer_iterations = hsc->guard;
@@ -1328,6 +1334,7 @@ int solve_joint_device(gmaf_ctx *ctx, int nth, int nz, int K, int nslots, const 
             *info = inf;
             return inf.status;
         }
+        if (opts->zero_init) GMAF_CUDA(cudaMemsetAsync(p, 0, (size_t)N * sizeof(double), s));
     }
     for (int b : {B_B32, B_X32, B_R032, B_R132, B_U032, B_U132, B_Z32, B_V32})
         GMAF_TRY(ensure(ctx, b, (size_t)N * sizeof(float)));

@@ -171,7 +171,11 @@ __device__ __forceinline__ void res_warp_sums(const double (&x)[NV], ResTerm<dou
 {
     int e[NV];
 #pragma unroll
-    for (int q = 0; q < NV; ++q) e[q] = __reduce_max_sync(0xffffffffu, res_exp(x[q]));
+    for (int q = 0; q < NV; ++q) {
+        // (1 where there are subnormal numbers only, whose sum is not formed: see res_totals)
+        const bool some = (((unsigned)__double2hiint(x[q]) << 1) | (unsigned)__double2loint(x[q])) != 0u;
+        e[q] = __reduce_max_sync(0xffffffffu, max(res_exp(x[q]), some ? 1 : 0));
+    }
     long long v[NV];
 #pragma unroll
     for (int q = 0; q < NV; ++q) {
@@ -220,17 +224,18 @@ __device__ __forceinline__ void res_warp_sums(const Acc<float> (&x)[NV], ResTerm
     }
 }
 
-// The biased exponent (as of a double) of a term's leading bit; 0: zero, 0x7ff: not finite.
+// The biased exponent (as of a double) of a term's leading bit; 0: zero, 1: perhaps less than that
+// exponent, 0x7ff: not finite.
 __device__ __forceinline__ int res_term_exp(const ResTerm<double> &t)
 {
     if (t.e == 0x7ff) return 0x7ff;
-    if (t.v == 0) return 0;
+    if (t.v == 0) return t.e == 1 ? 1 : 0;
     return max(1, t.e - 54 + 63 - __clzll(t.v < 0 ? -t.v : t.v));
 }
 __device__ __forceinline__ int res_term_exp(const ResTerm<float> &t)
 {
     const int e = (__float_as_uint(t.hi) >> 23) & 0xff;
-    return e == 0 ? 0 : (e == 0xff ? 0x7ff : e + 896);
+    return e == 0 ? (t.hi != 0.0f ? 1 : 0) : (e == 0xff ? 0x7ff : e + 896);
 }
 
 struct ResLimbs {
@@ -365,11 +370,14 @@ __device__ __forceinline__ bool res_meet(ResSums &x, int lane)
     return __all_sync(0xffffffffu, ok) != 0;
 }
 
-// The totals over the group's blocks of NV values, of which each lane holds one term
-// (in every lane); false if some block never came.  Values that are not finite or huge
-// give NaN, ones next to zero give zero.
+// The totals over the group's blocks of NV values, of which each lane holds one term (in every
+// lane).  Returns 0, GMAF_TIMEOUT if some block never came, or kResBeyond if the terms of a value
+// leave the range of exponents that the fixed-point numbers are formed in, 2^-942 to 2^1006 (zero
+// and what is not finite do not: they give 0 and NaN).
+constexpr int kResMinExp = 80, kResMaxExp = 2030;
+
 template <int NV, typename T>
-__device__ __forceinline__ bool res_totals(ResSums &x, int kind, const ResTerm<T> (&term)[NV], int lane,
+__device__ __forceinline__ int res_totals(ResSums &x, int kind, const ResTerm<T> (&term)[NV], int lane,
                                            double (&tot)[NV])
 {
     // kind 0: u.v; 1: r.z and r.r; 2: the FP64 residual's and source's
@@ -384,13 +392,16 @@ __device__ __forceinline__ bool res_totals(ResSums &x, int kind, const ResTerm<T
             int ex[NV];
 #pragma unroll
             for (int q = 0; q < NV; ++q) ex[q] = __reduce_max_sync(0xffffffffu, res_term_exp(term[q]));
-            if (!res_max_exp<NV>(x, ex, e, lane)) return false;
+            if (!res_max_exp<NV>(x, ex, e, lane)) return GMAF_TIMEOUT;
+#pragma unroll
+            for (int q = 0; q < NV; ++q)
+                if ((e[q] > 0 && e[q] <= kResMinExp) || (e[q] >= kResMaxExp && e[q] < 0x7ff)) return kResBeyond;
         }
         int en[NV];
         unsigned long long word = 0;
 #pragma unroll
         for (int q = 0; q < NV; ++q) {
-            en[q] = e[q] > 80 && e[q] < 2030 ? e[q] : 1023;
+            en[q] = e[q] > kResMinExp && e[q] < kResMaxExp ? e[q] : 1023;
             const ResLimbs l = res_limbs(term[q], en[q]);
             const unsigned l0 = __reduce_add_sync(0xffffffffu, (unsigned)l.lo & 0xffffffu);
             const int l1 = __reduce_add_sync(0xffffffffu, (int)(l.lo >> 24));
@@ -414,7 +425,7 @@ __device__ __forceinline__ bool res_totals(ResSums &x, int kind, const ResTerm<T
                 mine = mine && ((d[q] - prev[q]) & 0xffull) == (unsigned long long)x.nb;
             ok = __all_sync(0xffffffffu, mine);
         }
-        if (!ok) return false;
+        if (!ok) return GMAF_TIMEOUT;
         bool good = true;
 #pragma unroll
         for (int q = 0; q < NV; ++q) {
@@ -428,17 +439,24 @@ __device__ __forceinline__ bool res_totals(ResSums &x, int kind, const ResTerm<T
         if (!known || good) {
 #pragma unroll
             for (int q = 0; q < NV; ++q) {
-                if (e[q] <= 80 || e[q] >= 2030)
-                    tot[q] = e[q] <= 80 ? 0.0 : __longlong_as_double(0x7ff8000000000000ll);
+                if (e[q] == 0) tot[q] = 0.0;
+                if (e[q] == 0x7ff) tot[q] = __longlong_as_double(0x7ff8000000000000ll);
                 // (what the next total of the kind is expected to be)
                 e[q] = res_exp(tot[q]);
-                if (e[q] <= 80 || e[q] >= 2030) e[q] = 0;
+                if (e[q] <= kResMinExp || e[q] >= kResMaxExp) e[q] = 0;
             }
-            return true;
+            return 0;
         }
         known = false;
     }
-    return false;
+    return GMAF_TIMEOUT;
+}
+
+// Whether ||r||^2 stays in that range down to the tolerance (or to 1e-20, which no residual
+// reaches): bb is ||b||^2.  If not, the phase kernels take the system from the start.
+__device__ __forceinline__ bool res_in_range(double bb, double eps)
+{
+    return bb == 0.0 || res_exp(bb) + 2 * (max(res_exp(eps), 1023 - 67) - 1023) > kResMinExp + 40;
 }
 
 // a / b by Newton's iteration on the reciprocal from a single-precision start and one
@@ -554,8 +572,9 @@ struct ResExchange {
             {
                 const ResTerm<T> mine[2] = {gather(0), gather(1)};
                 double tot[2], beta = 0.0;
-                if (!res_totals<2, T>(sums, 1, mine, lane, tot) || sh.halo_failed) {
-                    status = GMAF_TIMEOUT;
+                const int got = res_totals<2, T>(sums, 1, mine, lane, tot);
+                if (got || sh.halo_failed) {
+                    status = got ? got : GMAF_TIMEOUT;
                     done = 1;
                 } else {
                     const double rz = tot[0], rr = tot[1];
@@ -610,8 +629,9 @@ struct ResExchange {
                 const ResTerm<T> mine[1] = {gather(0)};
                 double tot[1];
                 ++guard;
-                if (!res_totals<1, T>(sums, 0, mine, lane, tot) || sh.halo_failed) {
-                    status = GMAF_TIMEOUT;
+                const int got = res_totals<1, T>(sums, 0, mine, lane, tot);
+                if (got || sh.halo_failed) {
+                    status = got ? got : GMAF_TIMEOUT;
                     done = 1;
                 } else if (res_exp(tot[0]) == 0x7ff || __double_as_longlong(tot[0]) <= 0 ||
                            res_exp(d) == 0x7ff) {
@@ -641,16 +661,19 @@ struct ResExchange {
         {
             const ResTerm<T> mine[1] = {gather(0)};
             double tot[1];
-            const bool got = res_totals<1, T>(sums, 0, mine, lane, tot);
+            const int got = res_totals<1, T>(sums, 0, mine, lane, tot);
             sums.e[0] = 0;
-            if (!got) {
-                status = GMAF_TIMEOUT;
+            if (got) {
+                status = got;
                 done = 1;
             } else if (q.mode != kResRestart) {
                 normS = sqrt(tot[0]);
                 zero_rhs = tot[0] == 0.0;
                 if (!finite_d(tot[0])) {
                     status = GMAF_NONFINITE;
+                    done = 1;
+                } else if (!res_in_range(tot[0], q.eps)) {
+                    status = kResBeyond;
                     done = 1;
                 }
             }
@@ -678,29 +701,33 @@ struct ResExchange {
             {
                 const ResTerm<double> mine[2] = {gather64(0), gather64(1)};
                 double tot[2];
-                bool ok = res_totals<2, double>(sums, 2, mine, lane, tot) && !sh.halo_failed;
+                int got = res_totals<2, double>(sums, 2, mine, lane, tot);
+                if (!got && sh.halo_failed) got = GMAF_TIMEOUT;
                 // ||r64|| in the order of k_resid64, to the last bit: it is the unit of the FP32
                 // run and the factor of x in p (see res_norm_warps)
                 double nn = tot[0];
                 if constexpr (NORM) {
-                    ok = res_meet(sums, lane) && ok;
+                    if (!res_meet(sums, lane) && !got) got = GMAF_TIMEOUT;
                     bar_sync_n(2, all);
                     bar_sync_n(2, all);
-                    ok = res_meet(sums, lane) && ok;
+                    if (!res_meet(sums, lane) && !got) got = GMAF_TIMEOUT;
                     bar_sync_n(2, all);
                     bar_sync_n(2, all);
                     nn = 0.0;
                     for (int w = 0; w < kThreads / 32; ++w) nn += sh.red64[w];
                 }
                 rnorm = sqrt(nn);
-                if (!ok) {
-                    verdict = GMAF_TIMEOUT;
+                if (got) {
+                    verdict = got;
                     stop = true;
                 } else {
                     const double nS = sqrt(tot[1]);
                     true_rel = nS > 0.0 ? rnorm / nS : 0.0;
                     if (!finite_d(tot[0]) || !finite_d(tot[1]) || !finite_d(true_rel)) {
                         verdict = GMAF_NONFINITE;
+                        stop = true;
+                    } else if (outer == 0 && !res_in_range(tot[1], q.eps)) {
+                        verdict = kResBeyond;
                         stop = true;
                     } else if (nS == 0.0 || true_rel <= q.eps) {
                         verdict = GMAF_OK;

@@ -34,6 +34,10 @@ constexpr double res_limit(int tm) { return tm ? 1.25 : 10.0; }
 // Rows of n_theta values that a block of form 1 or 2 keeps in shared memory.
 __host__ __device__ constexpr int res_tm_rows(int nrr, int size) { return size == 8 ? 4 + 3 * nrr : 5 + 4 * nrr; }
 
+// Scalars.status of a run that the phase kernels have to take over (not a status of the ABI): a sum
+// of squares outside the range that the exchange forms sums in.
+constexpr int kResBeyond = 1;
+
 // FP64 (T = double): one run.  FP32: the whole mixed-precision solve.
 enum ResMode {
     kResFresh = 0,      // r = b - A p (p = 0 with zero_init)

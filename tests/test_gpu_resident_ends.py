@@ -87,3 +87,32 @@ def test_threads_with_contexts_of_their_own(g):
     for t in ts:
         t.join()
     assert not failed, failed
+
+
+# norms whose squares are subnormal, just above that, where only the residual's are, and next to
+# the largest double
+@pytest.mark.parametrize("power", [-520, -485, -440, 505])
+@pytest.mark.parametrize("precision,criterion", [(0, 0), (0, 1), (1, 0)])
+def test_sources_at_the_ends_of_the_range(g, monkeypatch, power, precision, criterion):
+    """The sums over blocks are fixed-point numbers whose scale is a normal exponent some way from
+    either end: beyond, the phase kernels solve the system, from the same start."""
+    nth, nz, K = 64, 20, 3
+    D, aE, aN, S = system(nth, nz, K, 9)
+    unit = 2.0 ** -np.floor(np.log2(float(D.max())))            # a diagonal of order one
+    S = S * 2.0 ** (power - np.floor(np.log2(float(torch.linalg.norm(S)))))
+    arrs = [D * unit, aE * unit, aN * unit, S]
+    start = 0.5 * S
+    kw = dict(precision=precision, criterion=criterion, start=start, max_iter=20000,
+              allow=(g.GMAF_OK, g.GMAF_NOT_CONVERGED, g.GMAF_NONFINITE))
+    monkeypatch.setenv("GMAF_NO_TUNE", "1")
+    a = solve(g, nth, nz, K, arrs, **kw)
+    monkeypatch.setenv("GMAF_VARIANT", "604322" if precision else "2322")
+    b = solve(g, nth, nz, K, arrs, **kw)
+    assert not resident(b[3])
+    assert a[0] == b[0] and bool(a[4].any())
+    if resident(a[3]):
+        assert rel_l2(a[4], b[4]) <= 1e-8
+    else:
+        assert a[1] == b[1] and torch.equal(a[4], b[4])
+    if power == -440:
+        assert a[0] == g.GMAF_OK

@@ -1,0 +1,52 @@
+"""Where the resident run of the allocation-free solve ends or gives way, as gmaf_solve_joint's does.
+
+The file name puts it after the test that first loads the scratch array."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2511_06824_gb300 import inputs
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+PHYS = inputs.phys_vector()
+
+
+@pytest.fixture(scope="module")
+def g():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2511_06824_gb300 import build, gmaf
+    build.build()
+    gmaf.load()
+    return gmaf
+
+
+def system(nth, nz, K, seed):
+    rng = np.random.default_rng(seed)
+    tex = inputs.dimple_texture(rng)
+    st, *arrs = oracle.assemble_joint(nth, nz, PHYS, tex, [inputs.random_state(rng) for _ in range(K)])
+    assert st == 0
+    return [torch.from_numpy(np.ascontiguousarray(a).ravel()).cuda() for a in arrs]
+
+
+@pytest.mark.parametrize("power", [-520, -485, -440, 505])
+def test_sources_at_the_ends_of_the_range(g, monkeypatch, power):
+    """Where sums of squares leave the range of the resident run's sums, the phase kernels solve the
+    system from the same start, as in gmaf_solve_joint."""
+    nth, nz, K = 64, 20, 3
+    D, aE, aN, S = system(nth, nz, K, 9)
+    unit = 2.0 ** -np.floor(np.log2(float(D.max())))            # a diagonal of order one
+    S = S * 2.0 ** (power - np.floor(np.log2(float(torch.linalg.norm(S)))))
+    arrs = [D * unit, aE * unit, aN * unit, S]
+    opts = g.solver_opts(eps=1e-10, zero_init=0, max_iter=20000)
+    allow = (g.GMAF_OK, g.GMAF_NOT_CONVERGED, g.GMAF_NONFINITE)
+    monkeypatch.setenv("GMAF_VARIANT", "2322")
+    p, q = 0.5 * S, 0.5 * S
+    with g.Context() as c:
+        st, it, rel = g.gmaf_solve_joint(c.handle, nth, nz, K, *arrs, p, opts, allow=allow)
+    stq, itq, relq = g.gmaf_solve_joint_noalloc(nth, nz, K, *arrs, q, opts, allow=allow)
+    assert stq == st and itq == it and bool(q.any())
+    if st == g.GMAF_OK and power > -500:
+        assert float(torch.linalg.norm(p - q) / torch.linalg.norm(p)) <= 1e-8
