@@ -140,15 +140,26 @@ __device__ __forceinline__ bool ll_get(const unsigned long long *p, double (&x)[
 // Within a warp (FP64) the scale is that of the largest term, 54 bits below its leading
 // one: the quantum is half the last bit of the largest term, so the error is at most
 // that of a chain of double additions.  FP32 keeps the two-float form of RowAcc through
-// the warp's butterfly.  Across warps and blocks a value is an 80-bit integer in two
-// limbs (44 bits and the rest), scaled so that the total expected (the last total of
-// its kind) has 67 bits: a total may grow by 2^13, and one that shrank below 2^-12 of
-// it would keep less than 54 bits; then, and the first time, the blocks first agree on
-// the largest exponent among their terms.
+// the warp's butterfly.  Across warps and blocks a value is an integer in two limbs (42
+// bits and the rest), scaled so that the total expected (the last total of its kind) has
+// 71 bits.  A warp's term may have 76; a total that shrank below 2^-8 of the expected one
+// is formed again, as each warp's term is cut off at the lowest bit (FP32: both its parts)
+// and all of them together may be short by 2^12.4 of it: 2^-49 of a total of 63 bits.  Then,
+// and the first time, the blocks first agree on the largest exponent among their terms.
 
-constexpr int kResTop = 66;             // bit of the leading digit of the expected total
-constexpr int kResLimb = 44;            // bits of the low limb
+constexpr int kResTop = 70;             // bit of the leading digit of the expected total
+constexpr int kResTermBits = 76;        // most bits of a term
+constexpr int kResShrink = 8;           // most bits by which a total may fall short of the expected one
+constexpr int kResLimb = 42;            // bits of the low limb
 constexpr unsigned long long kResLimbMask = (1ull << kResLimb) - 1;
+// Words of the exchange: the low limb beside a count of 8 bits, the rest beside two.  The sum over
+// all blocks and warps (of FP32's two parts each) has to fit, with its sign.
+constexpr long long kResTerms = 2ll * kResMaxBlocks * (kResThreads / 32);
+static_assert(kResMaxBlocks < 256, "blocks are counted in a byte");
+static_assert(kResTerms < 1ll << (55 - kResLimb), "low limbs");
+static_assert(kResTerms < 1ll << (47 - (kResTermBits - kResLimb)), "high limbs");
+// (and within a block, added up in pieces of 24 bits of 32 by integer reductions over a warp)
+static_assert(kResTermBits - kResLimb - 24 < 26 && kResLimb - 24 < 26, "limbs of a block");
 
 __device__ __forceinline__ int res_exp(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
 
@@ -245,7 +256,7 @@ struct ResLimbs {
 // m 2^up in units of the lowest bit (m of `bits` bits), added with its sign.
 __device__ __forceinline__ void res_limbs_add(ResLimbs &x, unsigned long long m, int up, bool neg, int bits)
 {
-    const bool over = (up + bits > kResTop + 14 || up > 63) && m != 0;
+    const bool over = (up + bits > kResTermBits || up > 63) && m != 0;
     const int left = min(max(up, 0), 63);
     m = over ? 0ull : m >> min(max(-up, 0), 63);
     const unsigned long long low = m << left, high = left ? m >> (64 - left) : 0ull;
@@ -255,7 +266,7 @@ __device__ __forceinline__ void res_limbs_add(ResLimbs &x, unsigned long long m,
     x.lo += neg ? -lo : lo;
     x.top += neg ? -top : top;
 }
-// (top 2^44 + lo) 2^(e - 1089), e - 1089 the weight of the lowest bit, rounded to a double.
+// (top 2^kResLimb + lo) 2^(e - 1023 - kResTop), the lowest bit's weight, rounded to a double.
 __device__ __forceinline__ double res_value(long long top, long long lo, int e)
 {
     top += lo >> kResLimb;
@@ -432,7 +443,7 @@ __device__ __forceinline__ int res_totals(ResSums &x, int kind, const ResTerm<T>
             const long long lo = (long long)(d[2 * q] - prev[2 * q]) >> 8;
             const unsigned long long t = d[2 * q + 1] - prev[2 * q + 1];
             tot[q] = res_value((long long)t >> 16, lo, en[q]);
-            good = good && ((t >> 8) & 0xffull) == 0 && res_exp(tot[q]) >= e[q] - 12;
+            good = good && ((t >> 8) & 0xffull) == 0 && res_exp(tot[q]) >= e[q] - kResShrink;
             prev[2 * q] = d[2 * q];
             prev[2 * q + 1] = d[2 * q + 1];
         }

@@ -116,3 +116,21 @@ def test_sources_at_the_ends_of_the_range(g, monkeypatch, power, precision, crit
         assert a[1] == b[1] and torch.equal(a[4], b[4])
     if power == -440:
         assert a[0] == g.GMAF_OK
+
+
+@pytest.mark.parametrize("fill", [0.95, 0.5, 0.999])
+def test_sums_with_the_largest_low_limbs(g, monkeypatch, fill):
+    """152 full blocks whose warps all have the same sum of squares, its bits below the 22 leading
+    ones `fill` of the most they can be: the low halves of the blocks' fixed-point sums are then as
+    large as they get.  ||r|| / ||b|| of a start, without an iteration, to rounding."""
+    nth, nz, K = 512, 304, 1
+    D, aE, aN, _ = system(nth, nz, K, 4)
+    # 64 cells a warp: a sum of 1 + fill / 2^22
+    S = torch.full((K * nth * nz,), float(np.sqrt((1.0 + fill * 2.0 ** -22) / 64.0)), dtype=torch.float64, device="cuda")
+    start = torch.linspace(0.0, 1.0, K * nth * nz, dtype=torch.float64, device="cuda") / float(D.max())
+    kw = dict(start=start, max_iter=0, allow=(g.GMAF_NOT_CONVERGED,))
+    a = solve(g, nth, nz, K, [D, aE, aN, S], **kw)[3]
+    monkeypatch.setenv("GMAF_VARIANT", "1001003")
+    b = solve(g, nth, nz, K, [D, aE, aN, S], **kw)[3]
+    assert resident(a) and not resident(b)
+    assert abs(a["rel_residual"] / b["rel_residual"] - 1.0) <= 1e-13
