@@ -7,6 +7,7 @@
 #include <new>
 
 #include "gmaf_internal.cuh"
+#include "gmaf_resident.h"
 
 namespace gmaf {
 
@@ -160,6 +161,7 @@ int gmaf_create(gmaf_ctx **out, size_t hbm_budget_bytes, void *cuda_stream)
     const char *lg = std::getenv("GMAF_LOOP_GUARD");
     c->loop_guard = lg ? std::atoi(lg) : 0;
     if (c->loop_guard < 0) c->loop_guard = 0;
+    c->res_polls = res_polls();
     *out = c;
     return GMAF_OK;
 }

@@ -166,6 +166,8 @@ struct gmaf_ctx {
     double reliable_delta;         // continued recurrence: residual reduction between two refinements
     unsigned res_epoch;            // resident PCG: last exchange number used in B_RES,
     size_t res_ring;               //   words of B_RESWORDS used since they were cleared
+    unsigned res_polls;            // polls before one of its waits runs out (GMAF_RESIDENT_POLLS can lower it)
+    int res_skip;                  // solves that leave it out, after one whose wait ran out
     int loop_guard;                // GMAF_LOOP_GUARD: fixed loop-guard limit (0: max_iter + 4)
 };
 

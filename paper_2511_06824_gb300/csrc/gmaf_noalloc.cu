@@ -202,6 +202,7 @@ extern "C" int gmaf_solve_joint_noalloc(const gmaf_grid *grid, int32_t n_cond, c
         q.n = n;
         q.groups = 1;
         q.mask = 1;
+        q.polls = res_polls();
         res_fill<double>(pl, &q);
         q.precond = h.precond;
         q.zero_init = opts->zero_init;
@@ -289,7 +290,7 @@ extern "C" int gmaf_solve_joint_noalloc(const gmaf_grid *grid, int32_t n_cond, c
         e = cudaMemcpyAsync(&hs, dsc, sizeof(Scalars), cudaMemcpyDeviceToHost, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
         if (e != cudaSuccess) return fail(e);
-        if (res && hs.status == kResBeyond) {
+        if (res && res_gives_way(hs.status)) {
             // not for the resident run: the phase kernels, from p
             res = keep = false;
             init_r = true;

@@ -871,6 +871,10 @@ static int solve_async64(gmaf_ctx *ctx, int nth, int nz, int K, const int *cslot
 
 constexpr size_t kResRing = 64 * 1024;
 
+// Solves that take the phase kernels after one whose blocks waited too long for each other: what
+// kept some of them off the GPU may still be there, and a wait that runs out takes about 2 s.
+constexpr int kResSkip = 64;
+
 template <typename T>
 struct ResRun {
     bool on = false;
@@ -879,12 +883,17 @@ struct ResRun {
 };
 
 // The plan and its buffers; off (phase kernels) when the system does not fit, when a
-// phase kernel is asked for, or when the budget has no room for the exchanged words.
+// phase kernel is asked for, when the budget has no room for the exchanged words, or for
+// a while after a run whose blocks did not all come.
 template <typename T>
 static void res_setup(gmaf_ctx *ctx, ResRun<T> &rr, int nth, int nz, int K, bool vec, long long m,
                       bool with_d)
 {
     rr.on = false;
+    if (ctx->res_skip > 0) {
+        --ctx->res_skip;
+        return;
+    }
     if (ctx->force_variant >= 0 && ctx->force_variant / 10000000 != kResVariant / 10000000) return;
     if (!res_plan<T>(nth, nz, K, vec, ctx->num_sms, &rr.pl)) return;
     int coop = 0;
@@ -902,6 +911,7 @@ static void res_setup(gmaf_ctx *ctx, ResRun<T> &rr, int nth, int nz, int K, bool
     q.n = (long long)nth * nz;
     q.groups = 1;
     q.mask = ~0ull;
+    q.polls = ctx->res_polls;
     q.halo = (unsigned long long *)ctx->buf[B_RES];
     res_fill<T>(rr.pl, &q);
     rr.on = true;
@@ -1031,7 +1041,8 @@ static int solve_resident64(gmaf_ctx *ctx, ResRun<double> &rr, int K, const int 
         unsigned long long again = 0;
         for (int k = 0; k < G; ++k) {
             if (!((ran >> k) & 1ull)) continue;
-            if (h[k].status == kResBeyond) {
+            if (res_gives_way(h[k].status)) {
+                if (h[k].status == kResLate) ctx->res_skip = kResSkip;
                 *off = true;
                 return GMAF_OK;
             }
@@ -1322,7 +1333,8 @@ int solve_joint_device(gmaf_ctx *ctx, int nth, int nz, int K, int nslots, const 
         bool off = false;
         GMAF_TRY(res_run<float>(ctx, rr, (long long)opts->max_iter + 2 * q.max_outer, &off));
         if (!off) GMAF_TRY(read_scalars(ctx, dsc, hsc));
-        if (!off && hsc->status != kResBeyond) {
+        if (!off && hsc->status == kResLate) ctx->res_skip = kResSkip;
+        if (!off && !res_gives_way(hsc->status)) {
             inf.iterations = hsc->iter;
             inf.iterations_sum = hsc->iter * K;
             inf.outer_iterations = hsc->guard;

@@ -4,6 +4,7 @@
 #include "gmaf_pcg_host.cuh"
 
 #include <algorithm>
+#include <cstdlib>
 
 namespace gmaf {
 
@@ -78,6 +79,13 @@ int res_scaled(const double *D, const double *aE, const double *aN, const double
 }
 
 // ------------------------------------------------------------------ launch shapes
+
+unsigned res_polls()
+{
+    const char *v = std::getenv("GMAF_RESIDENT_POLLS");
+    const long long n = v ? std::atoll(v) : 0;
+    return n >= 1 && n < (long long)kResPolls ? (unsigned)n : kResPolls;
+}
 
 static long long round16(long long b) { return (b + 15) / 16 * 16; }
 

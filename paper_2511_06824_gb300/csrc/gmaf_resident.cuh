@@ -22,8 +22,13 @@
 // result does not depend on scheduling.  A block can write a word again only
 // after an exchange that its readers entered after they had read it (v rows and u.v
 // before the exchange of z, z rows and r.z before the next exchange of v).  All
-// blocks are resident (cooperative launch); a wait that is not met after kResSpin
-// polls ends the run with GMAF_TIMEOUT.
+// blocks are resident (cooperative launch), but other work on the GPU may keep some of
+// them from running.  A wait that is not met after ResParams::polls polls (of about a
+// microsecond) ends the run with kResLate, and the phase kernels, whose blocks wait for
+// nothing, take the system.  A block that gives up adds no more sums, so the others give up
+// too; where it did so in the last exchange of theirs, what they found is measured by the FP64
+// residual after all, in mixed precision by the next one of the run, which is not formed without
+// it.
 //
 // Threads: lane groups of P threads (a power of two or a multiple of 32) cover a
 // row, VEC columns each; every group marches a run of RR rows.  West and east
@@ -38,8 +43,6 @@
 #include "gmaf_resident.h"
 
 namespace gmaf {
-
-constexpr unsigned kResSpin = 1u << 21;     // polls (of about a microsecond) before a wait gives up
 
 // ------------------------------------------------------------------ flagged words
 
@@ -88,11 +91,11 @@ __device__ __forceinline__ void ll_put(unsigned long long *p, const double (&x)[
         ll_st2(p + 2 * q, ll_word((unsigned)__double2loint(x[q]), ep),
                ll_word((unsigned)__double2hiint(x[q]), ep));
 }
-// Polls until every word carries ep; false if that never happened.
+// Polls until every word carries ep, `polls` times at most; false if that never happened.
 template <int VEC>
-__device__ __forceinline__ bool ll_get(const unsigned long long *p, float (&x)[VEC], unsigned ep)
+__device__ __forceinline__ bool ll_get(const unsigned long long *p, float (&x)[VEC], unsigned ep, unsigned polls)
 {
-    for (unsigned k = 0; k < kResSpin; ++k) {
+    for (unsigned k = 0; k < polls; ++k) {
         unsigned long long w[VEC];
         bool ok = true;
         if constexpr (VEC == 1) {
@@ -112,9 +115,9 @@ __device__ __forceinline__ bool ll_get(const unsigned long long *p, float (&x)[V
     return false;
 }
 template <int VEC>
-__device__ __forceinline__ bool ll_get(const unsigned long long *p, double (&x)[VEC], unsigned ep)
+__device__ __forceinline__ bool ll_get(const unsigned long long *p, double (&x)[VEC], unsigned ep, unsigned polls)
 {
-    for (unsigned k = 0; k < kResSpin; ++k) {
+    for (unsigned k = 0; k < polls; ++k) {
         unsigned long long lo[VEC], hi[VEC];
         bool ok = true;
 #pragma unroll
@@ -345,7 +348,7 @@ __device__ __forceinline__ void res_red(unsigned long long *p, unsigned long lon
 
 // The largest exponent of each of NV values over the group's blocks.
 template <int NV>
-__device__ __forceinline__ bool res_max_exp(ResSums &x, const int (&mine)[NV], int *e, int lane)
+__device__ __forceinline__ bool res_max_exp(ResSums &x, const int (&mine)[NV], int *e, int lane, unsigned polls)
 {
     ++x.turn;
     if (lane == 0) {
@@ -355,26 +358,26 @@ __device__ __forceinline__ bool res_max_exp(ResSums &x, const int (&mine)[NV], i
         __threadfence();
         res_red(x.w + kWordMaxCount, 1ull);
     }
-    for (unsigned k = 0; k < kResSpin; ++k) {
-        if (ll_ld1(x.w + kWordMaxCount) - x.prev_max == (unsigned long long)x.nb) {
-            x.prev_max += (unsigned long long)x.nb;
-            __threadfence();
+    // (all lanes leave together: the caller goes on with operations of the whole warp)
+    bool ok = false;
+    for (unsigned k = 0; k < polls && !ok; ++k)
+        ok = __all_sync(0xffffffffu, ll_ld1(x.w + kWordMaxCount) - x.prev_max == (unsigned long long)x.nb) != 0;
+    if (!ok) return false;
+    x.prev_max += (unsigned long long)x.nb;
+    __threadfence();
 #pragma unroll
-            for (int q = 0; q < NV; ++q) e[q] = (int)(ll_ld1(x.w + kWordMax + q) & 0xffffull);
-            return true;
-        }
-    }
-    return false;
+    for (int q = 0; q < NV; ++q) e[q] = (int)(ll_ld1(x.w + kWordMax + q) & 0xffffull);
+    return true;
 }
 
 // All blocks of the group have come, and what their threads stored before is visible.
-__device__ __forceinline__ bool res_meet(ResSums &x, int lane)
+__device__ __forceinline__ bool res_meet(ResSums &x, int lane, unsigned polls)
 {
     __threadfence();
     __syncwarp();
     if (lane == 0) res_red(x.w + kWordMeet, 1ull);
     bool ok = false;
-    for (unsigned k = 0; k < kResSpin && !ok; ++k)
+    for (unsigned k = 0; k < polls && !ok; ++k)
         ok = ll_ld1(x.w + kWordMeet) - x.prev_meet == (unsigned long long)x.nb;
     x.prev_meet += (unsigned long long)x.nb;
     __threadfence();
@@ -382,14 +385,14 @@ __device__ __forceinline__ bool res_meet(ResSums &x, int lane)
 }
 
 // The totals over the group's blocks of NV values, of which each lane holds one term (in every
-// lane).  Returns 0, GMAF_TIMEOUT if some block never came, or kResBeyond if the terms of a value
+// lane).  Returns 0, kResLate if some block never came, or kResBeyond if the terms of a value
 // leave the range of exponents that the fixed-point numbers are formed in, 2^-942 to 2^1006 (zero
 // and what is not finite do not: they give 0 and NaN).
 constexpr int kResMinExp = 80, kResMaxExp = 2030;
 
 template <int NV, typename T>
 __device__ __forceinline__ int res_totals(ResSums &x, int kind, const ResTerm<T> (&term)[NV], int lane,
-                                           double (&tot)[NV])
+                                          unsigned polls, double (&tot)[NV])
 {
     // kind 0: u.v; 1: r.z and r.r; 2: the FP64 residual's and source's
     unsigned long long *const w = x.w + (kind == 0 ? kWordUV : kind == 1 ? kWordRZ : kWordR64);
@@ -403,7 +406,7 @@ __device__ __forceinline__ int res_totals(ResSums &x, int kind, const ResTerm<T>
             int ex[NV];
 #pragma unroll
             for (int q = 0; q < NV; ++q) ex[q] = __reduce_max_sync(0xffffffffu, res_term_exp(term[q]));
-            if (!res_max_exp<NV>(x, ex, e, lane)) return GMAF_TIMEOUT;
+            if (!res_max_exp<NV>(x, ex, e, lane, polls)) return kResLate;
 #pragma unroll
             for (int q = 0; q < NV; ++q)
                 if ((e[q] > 0 && e[q] <= kResMinExp) || (e[q] >= kResMaxExp && e[q] < 0x7ff)) return kResBeyond;
@@ -427,7 +430,7 @@ __device__ __forceinline__ int res_totals(ResSums &x, int kind, const ResTerm<T>
         if (lane < 2 * NV) res_red(w + lane, word);
         unsigned long long d[2 * NV];
         bool ok = false;
-        for (unsigned k = 0; k < kResSpin && !ok; ++k) {
+        for (unsigned k = 0; k < polls && !ok; ++k) {
             bool mine = true;
 #pragma unroll
             for (int q = 0; q < NV; ++q) ll_ld2(w + 2 * q, d[2 * q], d[2 * q + 1]);
@@ -436,7 +439,7 @@ __device__ __forceinline__ int res_totals(ResSums &x, int kind, const ResTerm<T>
                 mine = mine && ((d[q] - prev[q]) & 0xffull) == (unsigned long long)x.nb;
             ok = __all_sync(0xffffffffu, mine);
         }
-        if (!ok) return GMAF_TIMEOUT;
+        if (!ok) return kResLate;
         bool good = true;
 #pragma unroll
         for (int q = 0; q < NV; ++q) {
@@ -460,7 +463,7 @@ __device__ __forceinline__ int res_totals(ResSums &x, int kind, const ResTerm<T>
         }
         known = false;
     }
-    return GMAF_TIMEOUT;
+    return kResLate;
 }
 
 // Whether ||r||^2 stays in that range down to the tolerance (or to 1e-20, which no residual
@@ -524,6 +527,14 @@ struct ResShared {
     int done, stop, halo_failed;
 };
 
+// Before the threads part: row threads may find a halo row missing before the exchange warp runs.
+template <typename T>
+__device__ __forceinline__ void res_clear(ResShared<T> &sh)
+{
+    if (threadIdx.x == 0) sh.done = sh.stop = sh.halo_failed = 0;
+    __syncthreads();
+}
+
 // (one object per block: a function's own shared variable)
 template <typename T>
 __device__ __forceinline__ ResShared<T> &res_shared()
@@ -566,6 +577,14 @@ struct ResExchange {
         return t;
     }
 
+    // res_totals; kResLate if a row of a neighbour is missing.
+    template <int NV, typename U>
+    __device__ __forceinline__ int totals(int kind, const ResTerm<U> (&mine)[NV], double (&tot)[NV])
+    {
+        const int got = res_totals<NV, U>(sums, kind, mine, lane, q.polls, tot);
+        return got ? got : sh.halo_failed ? kResLate : 0;
+    }
+
     // One PCG run from the residual that the row threads hold, to ||r|| <= eps normS or
     // max_iter (of the running count).  cscale > 0: a continued recurrence (mixed
     // precision), whose old direction is cscale times smaller in the new units.
@@ -583,9 +602,9 @@ struct ResExchange {
             {
                 const ResTerm<T> mine[2] = {gather(0), gather(1)};
                 double tot[2], beta = 0.0;
-                const int got = res_totals<2, T>(sums, 1, mine, lane, tot);
-                if (got || sh.halo_failed) {
-                    status = got ? got : GMAF_TIMEOUT;
+                const int got = totals<2, T>(1, mine, tot);
+                if (got) {
+                    status = got;
                     done = 1;
                 } else {
                     const double rz = tot[0], rr = tot[1];
@@ -640,9 +659,9 @@ struct ResExchange {
                 const ResTerm<T> mine[1] = {gather(0)};
                 double tot[1];
                 ++guard;
-                const int got = res_totals<1, T>(sums, 0, mine, lane, tot);
-                if (got || sh.halo_failed) {
-                    status = got ? got : GMAF_TIMEOUT;
+                const int got = totals<1, T>(0, mine, tot);
+                if (got) {
+                    status = got;
                     done = 1;
                 } else if (res_exp(tot[0]) == 0x7ff || __double_as_longlong(tot[0]) <= 0 ||
                            res_exp(d) == 0x7ff) {
@@ -672,7 +691,7 @@ struct ResExchange {
         {
             const ResTerm<T> mine[1] = {gather(0)};
             double tot[1];
-            const int got = res_totals<1, T>(sums, 0, mine, lane, tot);
+            const int got = totals<1, T>(0, mine, tot);
             sums.e[0] = 0;
             if (got) {
                 status = got;
@@ -712,16 +731,15 @@ struct ResExchange {
             {
                 const ResTerm<double> mine[2] = {gather64(0), gather64(1)};
                 double tot[2];
-                int got = res_totals<2, double>(sums, 2, mine, lane, tot);
-                if (!got && sh.halo_failed) got = GMAF_TIMEOUT;
+                int got = sh.halo_failed ? kResLate : totals<2, double>(2, mine, tot);
                 // ||r64|| in the order of k_resid64, to the last bit: it is the unit of the FP32
                 // run and the factor of x in p (see res_norm_warps)
                 double nn = tot[0];
                 if constexpr (NORM) {
-                    if (!res_meet(sums, lane) && !got) got = GMAF_TIMEOUT;
+                    if (!got && !res_meet(sums, lane, q.polls)) got = kResLate;
                     bar_sync_n(2, all);
                     bar_sync_n(2, all);
-                    if (!res_meet(sums, lane) && !got) got = GMAF_TIMEOUT;
+                    if (!got && !res_meet(sums, lane, q.polls)) got = kResLate;
                     bar_sync_n(2, all);
                     bar_sync_n(2, all);
                     nn = 0.0;
@@ -782,6 +800,7 @@ struct ResExchange {
             stalled = q.continued && !converged;
             ++outer;
             if (status != 0) verdict = status;
+            if (lane == 0 && status == kResLate) sh.halo_failed = 1;    // (the row threads wait no further)
             stop = status != 0 || seg == 0;     // (the row threads still add x to p)
             if (stop) {
                 for (int k = 0; k < (NORM ? 5 : 1); ++k) bar_sync_n(2, all);    // the residual's sums: not wanted
@@ -811,7 +830,6 @@ __device__ __forceinline__ void res_exchange_warp(const ResParams<T> &q, ResShar
     x.d = x.normS = x.rr_last = x.alpha = 0.0;
     x.timed = q.times != nullptr && lane == 0 && blockIdx.x == 0;
     x.t_mark = x.timed ? res_time() : 0ull;
-    if (lane == 0) sh.done = sh.stop = sh.halo_failed = 0;
     if constexpr (sizeof(T) == 4) {
         x.refine(sc);
     } else {
@@ -1043,12 +1061,14 @@ struct ResRows {
             ld64(p64 + (size_t)(nr - 1) * nth, pN64);
             ll_put<VEC>(row64 + 2 * nth, pN64, ep);
         }
+        // (a run that ended late waits no further)
+        const unsigned polls = sh.halo_failed ? 1u : q.polls;
         bar_sync_n(1, TC);                          // p64 of the block's other threads
 #pragma unroll
         for (int e = 0; e < VEC; ++e) pS64[e] = pN64[e] = 0.0;
         bool ok = true;
-        if (hasS) ok = ll_get<VEC>(row64 - 2 * nth, pS64, ep);
-        if (hasN) ok = ll_get<VEC>(row64 + 4 * nth, pN64, ep) && ok;
+        if (hasS) ok = ll_get<VEC>(row64 - 2 * nth, pS64, ep, polls);
+        if (hasN) ok = ll_get<VEC>(row64 + 4 * nth, pN64, ep, polls) && ok;
         if (!ok) sh.halo_failed = 1;
         // p on this row and the one below, a_N of the row below
         double pc[VEC], ps[VEC], nS[VEC];
@@ -1253,8 +1273,8 @@ __device__ __forceinline__ unsigned res_iterate(const ResParams<T> &q, ResShared
     // the neighbours' rows: `s`, the last row of the block below, `n`, the first of the one above
     auto fetch = [&](int s, int n) {
         bool ok = true;
-        if (hasS) ok = ll_get<VEC>(halo + (s - 4) * q.halo_row, hS, ep);
-        if (hasN) ok = ll_get<VEC>(halo + (n + 4) * q.halo_row, hN, ep) && ok;
+        if (hasS) ok = ll_get<VEC>(halo + (s - 4) * q.halo_row, hS, ep, q.polls);
+        if (hasN) ok = ll_get<VEC>(halo + (n + 4) * q.halo_row, hN, ep, q.polls) && ok;
         if (!ok) sh.halo_failed = 1;
     };
 
@@ -1675,6 +1695,7 @@ __global__ void __launch_bounds__(kResThreads + 32, 1) k_resident(const __grid_c
     ResShared<T> &sh = res_shared<T>();
     const int cond = blockIdx.x / q.bpc, grp = q.groups == 1 ? 0 : cond;
     if (!((q.mask >> grp) & 1ull)) return;                  // this group does not run
+    res_clear(sh);
     if ((int)threadIdx.x >= q.threads) {
         res_exchange_warp<T>(q, sh, q.sc + grp, grp, q.groups == 1 ? 0 : cond * q.bpc,
                              q.groups == 1 ? (int)gridDim.x : q.bpc, threadIdx.x & 31);

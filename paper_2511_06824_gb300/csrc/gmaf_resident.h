@@ -34,9 +34,15 @@ constexpr double res_limit(int tm) { return tm ? 1.25 : 10.0; }
 // Rows of n_theta values that a block of form 1 or 2 keeps in shared memory.
 __host__ __device__ constexpr int res_tm_rows(int nrr, int size) { return size == 8 ? 4 + 3 * nrr : 5 + 4 * nrr; }
 
-// Scalars.status of a run that the phase kernels have to take over (not a status of the ABI): a sum
-// of squares outside the range that the exchange forms sums in.
-constexpr int kResBeyond = 1;
+// Scalars.status of a run that the phase kernels have to take over (not statuses of the ABI): a sum
+// of squares outside the range that the exchange forms sums in; a wait for another block that ran out.
+constexpr int kResBeyond = 1, kResLate = 2;
+inline bool res_gives_way(int status) { return status > 0; }
+
+// Polls of about a microsecond before a wait runs out, unless the host sets fewer: about 2 s.
+constexpr unsigned kResPolls = 1u << 21;
+// The limit: GMAF_RESIDENT_POLLS (fault injection: a test can make a wait run out) or kResPolls.
+unsigned res_polls();
 
 // FP64 (T = double): one run.  FP32: the whole mixed-precision solve.
 enum ResMode {
@@ -52,6 +58,7 @@ struct ResParams {
     int threads, P, ncg, nrr, rows, nseg;
     int precond, mode, zero_init, max_iter, guard_limit;
     int o_rows, o_edge, o_x, o_q, o_keep, keep;     // keep: rows of a run whose E stays on the SM
+    unsigned polls;                     // limit of a wait
     unsigned epoch;                     // exchanges of this run are epoch + 1, epoch + 2, ...
     unsigned long long mask;            // groups that run
     long long n;

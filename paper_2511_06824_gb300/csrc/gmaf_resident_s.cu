@@ -294,8 +294,8 @@ __device__ __forceinline__ unsigned res_iterate_s(const ResParams<T> &q, ResShar
     // the neighbours' rows: `s`, the last row of the block below, `n`, the first of the one above
     auto fetch = [&](int s, int n) {
         bool ok = true;
-        if (hasS) ok = ll_get<VEC>(halo + (s - 4) * q.halo_row, hS, ep);
-        if (hasN) ok = ll_get<VEC>(halo + (n + 4) * q.halo_row, hN, ep) && ok;
+        if (hasS) ok = ll_get<VEC>(halo + (s - 4) * q.halo_row, hS, ep, q.polls);
+        if (hasN) ok = ll_get<VEC>(halo + (n + 4) * q.halo_row, hN, ep, q.polls) && ok;
         if (!ok) sh.halo_failed = 1;
         __syncwarp();
     };
@@ -776,6 +776,7 @@ static __global__ void __launch_bounds__(kResThreads + 32, 1) k_resident_s(const
     __shared__ unsigned s_tmem;
     const int cond = blockIdx.x / q.bpc, grp = q.groups == 1 ? 0 : cond;
     if (!((q.mask >> grp) & 1ull)) return;                  // this group does not run
+    res_clear(sh);
     if ((int)threadIdx.x >= q.threads) {
         res_exchange_warp<T>(q, sh, q.sc + grp, grp, q.groups == 1 ? 0 : cond * q.bpc,
                              q.groups == 1 ? (int)gridDim.x : q.bpc, threadIdx.x & 31);

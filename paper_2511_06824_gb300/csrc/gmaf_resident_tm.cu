@@ -112,8 +112,8 @@ __device__ __forceinline__ unsigned res_iterate_tm(const ResParams<float> &q, Re
     if (j0 + lr0 > 0 && act) V::ldrw(q.aN + coff - nth, aS0);
     auto fetch = [&](int s, int n) {
         bool ok = true;
-        if (hasS) ok = ll_get<VEC>(halo + (s - 4) * q.halo_row, hS, ep);
-        if (hasN) ok = ll_get<VEC>(halo + (n + 4) * q.halo_row, hN, ep) && ok;
+        if (hasS) ok = ll_get<VEC>(halo + (s - 4) * q.halo_row, hS, ep, q.polls);
+        if (hasN) ok = ll_get<VEC>(halo + (n + 4) * q.halo_row, hN, ep, q.polls) && ok;
         if (!ok) sh.halo_failed = 1;
         __syncwarp();
     };
@@ -537,6 +537,7 @@ static __global__ void __launch_bounds__(kResThreads + 32, 1) k_resident_tm(cons
     using T = float;
     ResShared<T> &sh = res_shared<T>();
     __shared__ unsigned s_tmem;
+    res_clear(sh);
     if ((int)threadIdx.x >= q.threads) {
         res_exchange_warp<T, false>(q, sh, q.sc, 0, 0, (int)gridDim.x, threadIdx.x & 31);
         return;

@@ -134,3 +134,29 @@ def test_sums_with_the_largest_low_limbs(g, monkeypatch, fill):
     b = solve(g, nth, nz, K, [D, aE, aN, S], **kw)[3]
     assert resident(a) and not resident(b)
     assert abs(a["rel_residual"] / b["rel_residual"] - 1.0) <= 1e-13
+
+
+@pytest.mark.parametrize("nth,nz,K,precision,criterion,forced", [
+    (64, 32, 1, 0, 0, 2322), (132, 45, 9, 1, 0, 604322), (130, 45, 9, 0, 1, 2322),
+    (512, 250, 9, 0, 0, 2322), (640, 200, 9, 1, 0, 604322), (700, 300, 9, 1, 0, 604322),
+])
+def test_a_wait_that_runs_out_gives_way_to_the_phase_kernels(g, monkeypatch, nth, nz, K, precision,
+                                                             criterion, forced):
+    """A block that waits longer than the limit (here one poll) ends the resident run, as it would
+    when other work kept some of the blocks off the GPU: the phase kernels then solve the system,
+    from the start that was given, and the context goes on."""
+    arrs = system(nth, nz, K, 8)
+    kw = dict(precision=precision, criterion=criterion, eps=1e-8)
+    monkeypatch.setenv("GMAF_NO_TUNE", "1")
+    monkeypatch.setenv("GMAF_RESIDENT_POLLS", "1")
+    p = torch.full((K * nth * nz,), 5.0, dtype=torch.float64, device="cuda")
+    with g.Context() as c:
+        for _ in range(2):
+            st, it, _ = g.gmaf_solve_joint(c.handle, nth, nz, K, *arrs, p, g.solver_opts(**kw))
+            assert st == 0 and g.gmaf_last_solve_info(c.handle)["kernel_variant"] == forced
+    monkeypatch.delenv("GMAF_RESIDENT_POLLS")
+    monkeypatch.setenv("GMAF_VARIANT", str(forced))
+    ref = solve(g, nth, nz, K, arrs, **kw)
+    assert it == ref[1] and torch.equal(p, ref[4])
+    monkeypatch.delenv("GMAF_VARIANT")
+    assert resident(solve(g, nth, nz, K, arrs, **kw)[3])

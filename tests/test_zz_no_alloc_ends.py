@@ -50,3 +50,22 @@ def test_sources_at_the_ends_of_the_range(g, monkeypatch, power):
     assert stq == st and itq == it and bool(q.any())
     if st == g.GMAF_OK and power > -500:
         assert float(torch.linalg.norm(p - q) / torch.linalg.norm(p)) <= 1e-8
+
+
+@pytest.mark.parametrize("nth,nz,K", [(64, 32, 1), (512, 250, 9)])
+def test_a_wait_that_runs_out_gives_way_to_the_phase_kernels(g, monkeypatch, nth, nz, K):
+    """A resident run whose blocks wait longer than the limit (here one poll) ends, and the phase
+    kernels solve the system; the next call takes the resident run again."""
+    arrs = system(nth, nz, K, 8)
+    opts = g.solver_opts(eps=1e-8)
+    p, q, r = (torch.full((K * nth * nz,), 3.0, dtype=torch.float64, device="cuda") for _ in range(3))
+    monkeypatch.setenv("GMAF_VARIANT", "2322")
+    with g.Context() as c:
+        st, it, rel = g.gmaf_solve_joint(c.handle, nth, nz, K, *arrs, p, opts)
+    monkeypatch.setenv("GMAF_RESIDENT_POLLS", "1")
+    stq, itq, relq = g.gmaf_solve_joint_noalloc(nth, nz, K, *arrs, q, opts)
+    monkeypatch.delenv("GMAF_RESIDENT_POLLS")
+    str_, itr, relr = g.gmaf_solve_joint_noalloc(nth, nz, K, *arrs, r, opts)
+    assert st == stq == str_ == 0 and itq == it and abs(itr - it) <= 2 and relq <= 1e-7
+    assert float(torch.linalg.norm(p - q) / torch.linalg.norm(p)) <= 1e-10
+    assert not torch.equal(q, r) and float(torch.linalg.norm(p - r) / torch.linalg.norm(p)) <= 1e-6
