@@ -20,20 +20,26 @@ int cuda_status(cudaError_t e)
 
 // Grow buffer `id` to at least `bytes` within the context's budget.  Contents
 // are not preserved.
-int ensure(gmaf_ctx *ctx, int id, size_t bytes)
+static int release(gmaf_ctx *ctx, int id)
+{
+    if (!ctx->buf[id]) return GMAF_OK;
+    cudaError_t e = cudaStreamSynchronize(ctx->stream);
+    if (e != cudaSuccess) return cuda_status(e);
+    cudaFree(ctx->buf[id]);
+    ctx->held -= ctx->bytes[id];
+    ctx->buf[id] = nullptr;
+    ctx->bytes[id] = 0;
+    return GMAF_OK;
+}
+
+static int ensure_one(gmaf_ctx *ctx, int id, size_t bytes)
 {
     if (bytes == 0) bytes = 16;
     if (ctx->bytes[id] >= bytes) return GMAF_OK;
     const size_t grow = bytes - ctx->bytes[id];
     if (ctx->budget && ctx->held + grow > ctx->budget) return GMAF_OUT_OF_MEMORY;
-    if (ctx->buf[id]) {
-        cudaError_t e = cudaStreamSynchronize(ctx->stream);
-        if (e != cudaSuccess) return cuda_status(e);
-        cudaFree(ctx->buf[id]);
-        ctx->held -= ctx->bytes[id];
-        ctx->buf[id] = nullptr;
-        ctx->bytes[id] = 0;
-    }
+    const int st = release(ctx, id);
+    if (st != GMAF_OK) return st;
     void *p = nullptr;
     cudaError_t e = cudaMalloc(&p, bytes);
     if (e != cudaSuccess) {
@@ -48,6 +54,32 @@ int ensure(gmaf_ctx *ctx, int id, size_t bytes)
     ctx->buf[id] = p;
     ctx->bytes[id] = bytes;
     ctx->held += bytes;
+    return GMAF_OK;
+}
+
+int ensure(gmaf_ctx *ctx, int id, size_t bytes)
+{
+    int st = ensure_one(ctx, id, bytes);
+    if (st != GMAF_OUT_OF_MEMORY) return st;
+    bool any = false;
+    for (int r = B_RES; r <= B_RESPART; ++r) {
+        any = any || ctx->buf[r];
+        if ((st = release(ctx, r)) != GMAF_OK) return st;
+    }
+    ctx->res_ring = 0;
+    return any ? ensure_one(ctx, id, bytes) : GMAF_OUT_OF_MEMORY;
+}
+
+int ensure_all(gmaf_ctx *ctx, const BufNeed *need, int count)
+{
+    size_t grow = 0;
+    for (int k = 0; k < count; ++k)
+        if (need[k].bytes > ctx->bytes[need[k].id]) grow += need[k].bytes - ctx->bytes[need[k].id];
+    if (ctx->budget && ctx->held + grow > ctx->budget) return GMAF_OUT_OF_MEMORY;
+    for (int k = 0; k < count; ++k) {
+        const int st = ensure_one(ctx, need[k].id, need[k].bytes);
+        if (st != GMAF_OK) return st;
+    }
     return GMAF_OK;
 }
 

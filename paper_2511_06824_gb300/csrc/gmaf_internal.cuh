@@ -112,8 +112,9 @@ enum BufId {
     B_CHUNK, B_CHUNKCTR,
     // boundary rows' Dirichlet term of the FP32 diagonal (phase A with the rebuilt diagonal)
     B_DBND32,
-    // resident PCG: exchanged rows, words of the exchanged sums, phase times, scaled matrix
-    B_RES, B_RESWORDS, B_RESTIME, B_RESCOEF,
+    // resident PCG: exchanged rows, words of the exchanged sums, phase times, scaled matrix,
+    // descriptors and partial sums of its FP64 residuals
+    B_RES, B_RESWORDS, B_RESTIME, B_RESCOEF, B_RESDESC, B_RESPART,
     B_COUNT
 };
 
@@ -202,7 +203,16 @@ inline void smem_optin(std::atomic<unsigned long long> &done, const void *fn, si
         cudaGetLastError();
 }
 
+// At least `bytes` in a buffer of the context.  What only the resident PCG uses gives way when the
+// budget or the GPU has no room left: the phase kernels need less.
 int ensure(gmaf_ctx *ctx, int id, size_t bytes);
+// All of several buffers, without that: GMAF_OUT_OF_MEMORY, and nothing allocated, if the budget has
+// no room for them together.
+struct BufNeed {
+    int id;
+    size_t bytes;
+};
+int ensure_all(gmaf_ctx *ctx, const BufNeed *need, int count);
 int cuda_status(cudaError_t e);
 bool geom_valid(const gmaf_grid *g, const gmaf_physics *ph, const gmaf_texture *tex);
 bool opts_valid(const gmaf_solver_opts *o);

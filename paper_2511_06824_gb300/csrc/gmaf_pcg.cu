@@ -875,6 +875,9 @@ constexpr size_t kResRing = 64 * 1024;
 // kept some of them off the GPU may still be there, and a wait that runs out takes about 2 s.
 constexpr int kResSkip = 64;
 
+// B_RESDESC: descriptors, then the coefficient slot of a condition by itself.
+static size_t res_desc_slot() { return align256((size_t)kMaxCond * sizeof(ResidDesc)); }
+
 template <typename T>
 struct ResRun {
     bool on = false;
@@ -882,12 +885,12 @@ struct ResRun {
     ResParams<T> q{};
 };
 
-// The plan and its buffers; off (phase kernels) when the system does not fit, when a
-// phase kernel is asked for, when the budget has no room for the exchanged words, or for
-// a while after a run whose blocks did not all come.
+// The plan and its buffers (part: of the partial sums); off (phase kernels) when the system does
+// not fit, when a phase kernel is asked for, when the budget has no room for the buffers, or for a
+// while after a run whose blocks did not all come.
 template <typename T>
 static void res_setup(gmaf_ctx *ctx, ResRun<T> &rr, int nth, int nz, int K, bool vec, long long m,
-                      bool with_d)
+                      int nslots, bool with_d, size_t part)
 {
     rr.on = false;
     if (ctx->res_skip > 0) {
@@ -901,10 +904,20 @@ static void res_setup(gmaf_ctx *ctx, ResRun<T> &rr, int nth, int nz, int K, bool
         cudaGetLastError();
         return;
     }
-    if (ensure(ctx, B_RESWORDS, kResRing) != GMAF_OK) return;
-    if (ensure(ctx, B_RES, rr.pl.halo_bytes) != GMAF_OK) return;
-    if (ctx->phase_timing && ensure(ctx, B_RESTIME, 64) != GMAF_OK) return;
-    if (sizeof(T) == 8 && rr.pl.tm && ensure(ctx, B_RESCOEF, res_scaled_bytes(m, with_d)) != GMAF_OK) return;
+    BufNeed need[8] = {{B_RESWORDS, kResRing}, {B_RES, rr.pl.halo_bytes}, {B_RESPART, part}};
+    int n = 3;
+    const size_t N = (size_t)nth * nz * K;
+    if (ctx->phase_timing) need[n++] = {B_RESTIME, 64};
+    if (sizeof(T) == 8) {
+        need[n++] = {B_RESDESC, res_desc_slot() + 256};
+        if (rr.pl.tm) need[n++] = {B_RESCOEF, res_scaled_bytes(m, with_d)};
+        // (x apart from p, which keeps the start until the end)
+        if (rr.pl.tm && rr.pl.o_x < 0) need[n++] = {B_U0, N * sizeof(double)};
+    } else {
+        if (rr.pl.tm == 3 || rr.pl.o_x < 0) need[n++] = {B_X32, N * sizeof(float)};
+        if (rr.pl.tm == 3) need[n++] = {B_DBND32, (size_t)nslots * 2 * nth * sizeof(float)};
+    }
+    if (ensure_all(ctx, need, n) != GMAF_OK) return;
     ResParams<T> &q = rr.q;
     q.nth = nth;
     q.nz = nz;
@@ -990,11 +1003,9 @@ static int solve_resident64(gmaf_ctx *ctx, ResRun<double> &rr, int K, const int 
     q.sc = gsc;
     q.mode = kResFresh;
     // descriptors of the residuals: condition k, or the joint system
-    const size_t o_slot = align256((size_t)kMaxCond * sizeof(ResidDesc));
-    GMAF_TRY(ensure(ctx, B_ASYNC, o_slot + 256));
-    ResidDesc *d_rd = (ResidDesc *)ctx->buf[B_ASYNC];
+    ResidDesc *d_rd = (ResidDesc *)ctx->buf[B_RESDESC];
+    int *d_slot0 = (int *)((char *)ctx->buf[B_RESDESC] + res_desc_slot());
     const int gs = stream_grid(async ? n : n * K, ctx->num_sms);
-    GMAF_TRY(ensure(ctx, B_PART, (size_t)2 * gs * G * sizeof(double)));
     std::vector<ResidDesc> rd(G);
     for (int k = 0; k < G; ++k) {
         const long long o = (long long)k * n, c = async ? (long long)cslot_host[k] * n : 0;
@@ -1006,14 +1017,14 @@ static int solve_resident64(gmaf_ctx *ctx, ResRun<double> &rr, int K, const int 
         rd[k].D = q.D64 + c;
         rd[k].aE = q.aE64 + c;
         rd[k].aN = q.aN64 + c;
-        rd[k].cslot = async ? (const int *)((char *)ctx->buf[B_ASYNC] + o_slot) : q.cslot;
+        rd[k].cslot = async ? d_slot0 : q.cslot;
         rd[k].S = S + o;
         rd[k].p = p + o;
         rd[k].sc = rsc + k;
-        rd[k].partials = (double *)ctx->buf[B_PART] + (size_t)2 * gs * k;
+        rd[k].partials = (double *)ctx->buf[B_RESPART] + (size_t)2 * gs * k;
     }
     GMAF_CUDA(cudaMemsetAsync(gsc, 0, (size_t)2 * G * sizeof(Scalars), s));
-    if (async) GMAF_CUDA(cudaMemsetAsync((char *)ctx->buf[B_ASYNC] + o_slot, 0, sizeof(int), s));
+    if (async) GMAF_CUDA(cudaMemsetAsync(d_slot0, 0, sizeof(int), s));
     std::vector<Scalars> h(2 * G);
     std::vector<int> restarted(G, 0), ok(G, 0);
     std::vector<double> true_rel(G, 0.0);
@@ -1063,7 +1074,11 @@ static int solve_resident64(gmaf_ctx *ctx, ResRun<double> &rr, int K, const int 
         ran = again;
         if (ran) {
             // restart those from S - A p
-            GMAF_TRY(ensure(ctx, B_R0, (size_t)n * K * sizeof(double)));
+            const BufNeed need{B_R0, (size_t)n * K * sizeof(double)};
+            if (ensure_all(ctx, &need, 1) != GMAF_OK) {
+                *off = true;
+                return GMAF_OK;
+            }
             for (int k = 0; k < G; ++k) rd[k].r = (double *)ctx->buf[B_R0] + (long long)k * n;
             GMAF_TRY(residuals());
             q.r_in = (const double *)ctx->buf[B_R0];
@@ -1153,7 +1168,9 @@ int solve_joint_device(gmaf_ctx *ctx, int nth, int nz, int K, int nslots, const 
         const void *ptrs[] = {D, aE, aN, S, p};
         bool vec = nth % 2 == 0;
         for (const void *x : ptrs) vec = vec && aligned16(x);
-        res_setup<double>(ctx, rr, nth, nz, K, vec, m, opts->precond == 2);
+        // (partial sums of the residuals, of each condition or of the joint system)
+        const size_t part = opts->criterion == 1 ? (size_t)2 * K * stream_grid(n, ctx->num_sms) : (size_t)2 * gs;
+        res_setup<double>(ctx, rr, nth, nz, K, vec, m, nslots, opts->precond == 2, part * sizeof(double));
         if (rr.on) {
             ResParams<double> &q = rr.q;
             q.precond = kernel_precond(opts);
@@ -1174,8 +1191,6 @@ int solve_joint_device(gmaf_ctx *ctx, int nth, int nz, int K, int nslots, const 
             q.aN64 = aN;
             q.p64 = p;
             if (rr.pl.tm) {
-                // (x apart from p, which keeps the start until the end)
-                if (rr.pl.o_x < 0) GMAF_TRY(ensure(ctx, B_U0, (size_t)N * sizeof(double)));
                 q.x = (double *)ctx->buf[B_U0];
                 GMAF_TRY(res_scaled(D, aE, aN, opts->precond == 2 ? (const double *)ctx->buf[B_INVD] : nullptr,
                                     opts->precond == 1 ? opts->omega : 1.0, nth, nz, m, ctx->buf[B_RESCOEF],
@@ -1293,12 +1308,11 @@ int solve_joint_device(gmaf_ctx *ctx, int nth, int nz, int K, int nslots, const 
 
     // the whole refinement in one launch where the system fits on the SMs
     ResRun<float> rr;
-    res_setup<float>(ctx, rr, nth, nz, K, nth % 4 == 0, m, false);
+    res_setup<float>(ctx, rr, nth, nz, K, nth % 4 == 0, m, nslots, false,
+                     (size_t)gs * (kThreads / 32) * sizeof(double));
     if (rr.on) {
-        if (rr.pl.tm == 3 || rr.pl.o_x < 0) GMAF_TRY(ensure(ctx, B_X32, (size_t)N * sizeof(float)));
         ResParams<float> &q = rr.q;
         if (rr.pl.tm == 3) {
-            GMAF_TRY(ensure(ctx, B_DBND32, (size_t)nslots * 2 * nth * sizeof(float)));
             GMAF_TRY(launch_dbnd32((const float *)ctx->buf[B_D32], (const float *)ctx->buf[B_AE32],
                                    (const float *)ctx->buf[B_AN32], (float *)ctx->buf[B_DBND32], nth, nz,
                                    nslots, ctx->num_sms, s));
@@ -1323,8 +1337,7 @@ int solve_joint_device(gmaf_ctx *ctx, int nth, int nz, int K, int nslots, const 
         q.p64 = p;
         q.r64 = (double *)ctx->buf[B_R64];
         q.grid64 = gs;
-        GMAF_TRY(ensure(ctx, B_PART, (size_t)gs * (kThreads / 32) * sizeof(double)));
-        q.warps64 = (double *)ctx->buf[B_PART];
+        q.warps64 = (double *)ctx->buf[B_RESPART];
         q.pairs64 = nth % 2 == 0;
         for (const double *a : {D, aE, aN, S, (const double *)p}) q.pairs64 = q.pairs64 && aligned16(a);
         q.continued = ctx->mixed_restart ? 0 : 1;

@@ -160,3 +160,42 @@ def test_a_wait_that_runs_out_gives_way_to_the_phase_kernels(g, monkeypatch, nth
     assert it == ref[1] and torch.equal(p, ref[4])
     monkeypatch.delenv("GMAF_VARIANT")
     assert resident(solve(g, nth, nz, K, arrs, **kw)[3])
+
+
+# a small system that takes the resident run, and a large one with the budget that the phase kernels
+# need for it; the first one's scaled matrix, with ASSOR-I's diagonal, takes more than that
+@pytest.mark.parametrize("small,large,forced,opts", [
+    ((256, 128, 4), (1000, 250, 4), 2322, dict(precond=2)),
+    ((512, 250, 9), (640, 300, 9), 2322, {}),
+    ((256, 128, 9), (640, 300, 9), 2322, dict(criterion=1)),
+    ((512, 250, 9), (1028, 290, 9), 604322, dict(precision=1)),
+    ((640, 200, 9), (700, 300, 9), 604322, dict(precision=1)),
+])
+def test_budgets_that_were_enough_still_are(g, monkeypatch, small, large, forced, opts):
+    """A budget of what the phase kernels hold, to the byte: the solve succeeds, also after a smaller
+    one in the same context, and stays within it."""
+    sizes = (small, large)
+    arrs = [system(*s, 2) for s in sizes]
+    ps = [torch.zeros_like(a[3]) for a in arrs]
+    o = g.solver_opts(eps=1e-6, **opts)
+    monkeypatch.setenv("GMAF_NO_TUNE", "1")
+    monkeypatch.setenv("GMAF_VARIANT", str(forced))
+    with g.Context() as c:
+        for k in (0, 1):
+            g.gmaf_solve_joint(c.handle, *sizes[k], *arrs[k], ps[k], o)
+            if opts.get("criterion", 0) == 0:
+                assert g.gmaf_last_solve_info(c.handle)["kernel_variant"] == forced
+        held = g.gmaf_workspace_bytes(c.handle)
+    refs = [p.clone() for p in ps]
+    monkeypatch.delenv("GMAF_VARIANT")
+    with g.Context() as c:
+        g.gmaf_solve_joint(c.handle, *sizes[0], *arrs[0], ps[0], o)
+        assert resident(g.gmaf_last_solve_info(c.handle))
+    for order in ((1,), (0, 1, 0, 1)):
+        with g.Context(hbm_budget_bytes=held) as c:
+            for k in order:
+                ps[k].fill_(7.0)
+                st, _, _ = g.gmaf_solve_joint(c.handle, *sizes[k], *arrs[k], ps[k], o, allow=tuple(range(-8, 1)))
+                assert st == 0, (order, k, g.status_string(st))
+                assert g.gmaf_workspace_bytes(c.handle) <= held
+                assert rel_l2(ps[k], refs[k]) <= 1e-3
