@@ -253,7 +253,7 @@ extern "C" int gmaf_solve_joint_noalloc(const gmaf_grid *grid, int32_t n_cond, c
 
     Scalars hs{}, hr{};
     int restarted = 0;
-    bool keep = false, init_r = true;
+    bool keep = false, init_r = true, good = false;
     int status = GMAF_NOT_CONVERGED;
     double true_rel = 0.0;
     for (;;) {
@@ -290,12 +290,15 @@ extern "C" int gmaf_solve_joint_noalloc(const gmaf_grid *grid, int32_t n_cond, c
         e = cudaMemcpyAsync(&hs, dsc, sizeof(Scalars), cudaMemcpyDeviceToHost, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
         if (e != cudaSuccess) return fail(e);
-        if (res && res_gives_way(hs.status)) {
-            // not for the resident run: the phase kernels, from p
-            res = keep = false;
+        // not for the resident run: the phase kernels, from p
+        auto give_way = [&] {
+            res = keep = good = false;
             init_r = true;
             restarted = 0;
             diag_inverse64(opts, D, aE, aN, nth, nz, N, invD, num_sms, s);
+        };
+        if (res && !good && res_gives_way(hs.status)) {
+            give_way();
             continue;
         }
         // true residual S - A p into r[iter & 1], where a restart reads it
@@ -307,6 +310,17 @@ extern "C" int gmaf_solve_joint_noalloc(const gmaf_grid *grid, int32_t n_cond, c
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
         if (e != cudaSuccess) return fail(e);
         true_rel = hr.true_rel;
+        if (good) {
+            // a good solution, restarted: better now, or what it was
+            if (hr.status == 0 && true_rel <= 10.0 * opts->eps) {
+                status = GMAF_OK;
+                break;
+            }
+            e = cudaMemsetAsync(dsc_res, 0, sizeof(Scalars), s);
+            if (e != cudaSuccess) return fail(e);
+            give_way();
+            continue;
+        }
         if (hs.zero_rhs) {
             e = cudaMemsetAsync(p, 0, (size_t)N * sizeof(double), s);
             if (e == cudaSuccess) e = cudaStreamSynchronize(s);
@@ -321,6 +335,8 @@ extern "C" int gmaf_solve_joint_noalloc(const gmaf_grid *grid, int32_t n_cond, c
         status = end && true_rel <= 10.0 * opts->eps ? GMAF_OK : GMAF_NOT_CONVERGED;
         if (end && true_rel <= (res && !restarted ? res_limit(pl.tm) : 10.0) * opts->eps) break;
         if (restarted || hs.iter >= opts->max_iter) break;
+        good = status == GMAF_OK;
+        q.optional = good ? 1 : 0;
         restarted = 1;
         keep = true;
         init_r = false;

@@ -984,8 +984,8 @@ static int res_run(gmaf_ctx *ctx, ResRun<T> &rr, long long most_iterations, bool
 
 // FP64, either criterion: the joint system is one group of blocks, under the
 // asynchronized criterion each condition is one (its own scalars, its own end).
-// After a run each group gets the FP64 true-residual check, and once, if that
-// fails, a restart from the true residual.  *off: the phase kernels have to solve
+// After a run each group gets the FP64 true-residual check, and once, if that fails (or, in the
+// scaled forms, is not close), a restart from the true residual.  *off: the phase kernels have to solve
 // the system (from p, where that is the start).
 static int solve_resident64(gmaf_ctx *ctx, ResRun<double> &rr, int K, const int *cslot_host,
                             const double *S, double *p, const gmaf_solver_opts *opts,
@@ -1027,7 +1027,8 @@ static int solve_resident64(gmaf_ctx *ctx, ResRun<double> &rr, int K, const int 
     if (async) GMAF_CUDA(cudaMemsetAsync(d_slot0, 0, sizeof(int), s));
     std::vector<Scalars> h(2 * G);
     std::vector<int> restarted(G, 0), ok(G, 0);
-    std::vector<double> true_rel(G, 0.0);
+    std::vector<double> true_rel(G, 0.0), first_rel(G, 0.0);
+    q.optional = 0;
     unsigned long long ran = G == 64 ? ~0ull : (1ull << G) - 1;
     for (int pass = 0; ran; ++pass) {
         q.mask = ran;
@@ -1049,9 +1050,21 @@ static int solve_resident64(gmaf_ctx *ctx, ResRun<double> &rr, int K, const int 
             return GMAF_OK;
         };
         GMAF_TRY(residuals());
-        unsigned long long again = 0;
+        unsigned long long again = 0, may = 0;
         for (int k = 0; k < G; ++k) {
             if (!((ran >> k) & 1ull)) continue;
+            if ((q.optional >> k) & 1ull) {
+                // a good solution, restarted: better now, or what it was
+                if (h[k].status == kResLate) ctx->res_skip = kResSkip;
+                if (h[G + k].status != 0 || !(h[G + k].true_rel <= 10.0 * opts->eps)) {
+                    *off = true;
+                    return GMAF_OK;
+                }
+                true_rel[k] = h[G + k].true_rel;
+                if (!h[k].converged) h[k].rel = first_rel[k];
+                h[k].status = 0;
+                continue;
+            }
             if (res_gives_way(h[k].status)) {
                 if (h[k].status == kResLate) ctx->res_skip = kResSkip;
                 *off = true;
@@ -1068,17 +1081,21 @@ static int solve_resident64(gmaf_ctx *ctx, ResRun<double> &rr, int K, const int 
             ok[k] = end && true_rel[k] <= 10.0 * opts->eps;
             if (end && true_rel[k] <= (restarted[k] ? 10.0 : res_limit(rr.pl.tm)) * opts->eps) continue;
             if (restarted[k] || h[k].iter >= opts->max_iter) continue;
-            restarted[k] = 1;
             again |= 1ull << k;
+            if (ok[k]) may |= 1ull << k;
+            first_rel[k] = h[k].rel;
         }
         ran = again;
+        q.optional = may;
         if (ran) {
             // restart those from S - A p
             const BufNeed need{B_R0, (size_t)n * K * sizeof(double)};
             if (ensure_all(ctx, &need, 1) != GMAF_OK) {
-                *off = true;
-                return GMAF_OK;
+                *off = ran != may;
+                if (*off) return GMAF_OK;
+                break;
             }
+            for (int k = 0; k < G; ++k) restarted[k] = (int)((ran >> k) & 1ull);
             for (int k = 0; k < G; ++k) rd[k].r = (double *)ctx->buf[B_R0] + (long long)k * n;
             GMAF_TRY(residuals());
             q.r_in = (const double *)ctx->buf[B_R0];

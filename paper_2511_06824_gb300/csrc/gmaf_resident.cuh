@@ -524,7 +524,7 @@ struct ResShared {
     double alpha, beta;
     double red64[kThreads / 32];        // (norm of the FP64 residual)
     double unit, back;                  // mixed precision: 1 / ||r64||; scale ||r64||, which takes x to p
-    int done, stop, halo_failed;
+    int done, stop, halo_failed;        // done: 1 converged, 2 not
 };
 
 // Before the threads part: row threads may find a halo row missing before the exchange warp runs.
@@ -605,7 +605,7 @@ struct ResExchange {
                 const int got = totals<2, T>(1, mine, tot);
                 if (got) {
                     status = got;
-                    done = 1;
+                    done = 2;
                 } else {
                     const double rz = tot[0], rr = tot[1];
                     rr_last = rr;
@@ -624,20 +624,20 @@ struct ResExchange {
                         done = 1;
                     } else if (!fin) {
                         status = GMAF_NONFINITE;
-                        done = 1;
+                        done = 2;
                     } else if (__double_as_longlong(rr) <= thr2 && sqrt(rr) / normS <= eps) {
                         // (Eq. 3.9; the root and the quotient are formed only near the tolerance)
                         converged = 1;
                         done = 1;
                     } else if (iter >= max_iter) {
-                        done = 1;
+                        done = 2;
                     }
                     if (init || !done) d = rz;
                     // loop guard: never more products than iterations (a host-set limit can lower it)
                     if (!init && guard > (q.guard_limit > 0 ? (long long)q.guard_limit
                                                             : (long long)max_iter + 4)) {
                         status = GMAF_TIMEOUT;
-                        done = 1;
+                        done = 2;
                     }
                 }
                 if (lane == 0) {
@@ -662,11 +662,11 @@ struct ResExchange {
                 const int got = totals<1, T>(0, mine, tot);
                 if (got) {
                     status = got;
-                    done = 1;
+                    done = 2;
                 } else if (res_exp(tot[0]) == 0x7ff || __double_as_longlong(tot[0]) <= 0 ||
                            res_exp(d) == 0x7ff) {
                     status = GMAF_NONFINITE;
-                    done = 1;
+                    done = 2;
                 } else {
                     alpha = res_quotient(d, tot[0]);
                 }
@@ -695,16 +695,16 @@ struct ResExchange {
             sums.e[0] = 0;
             if (got) {
                 status = got;
-                done = 1;
+                done = 2;
             } else if (q.mode != kResRestart) {
                 normS = sqrt(tot[0]);
                 zero_rhs = tot[0] == 0.0;
                 if (!finite_d(tot[0])) {
                     status = GMAF_NONFINITE;
-                    done = 1;
+                    done = 2;
                 } else if (!res_in_range(tot[0], q.eps)) {
                     status = kResBeyond;
-                    done = 1;
+                    done = 2;
                 }
             }
         }

@@ -29,6 +29,8 @@ __host__ __device__ constexpr int res_tm(int rr, int vec, int size)
 // (by 4e-14 of the right-hand side on 512 x 256 cells, 2e-13 on 1000 x 250, 1e-11 on 511 x 5,
 // where the unscaled forms drift by a tenth of it), so a run that ends well above is restarted
 // from its true residual, which takes that out; the unscaled forms keep the phase kernels' limit.
+// (Below ten times the tolerance the first run's solution is good, and stays if the restart finds no
+// room for its residual or no iterations left.)
 constexpr double res_limit(int tm) { return tm ? 1.25 : 10.0; }
 
 // Rows of n_theta values that a block of form 1 or 2 keeps in shared memory.
@@ -61,6 +63,8 @@ struct ResParams {
     unsigned polls;                     // limit of a wait
     unsigned epoch;                     // exchanges of this run are epoch + 1, epoch + 2, ...
     unsigned long long mask;            // groups that run
+    unsigned long long optional;        // scaled: groups whose p is within the limit already: a restart
+                                        // that ends without meeting the tolerance leaves it
     long long n;
     const T *D, *invD, *aE, *aN;        // (scaled: of s A s; D null where it is the constant dg)
     const int *cslot;

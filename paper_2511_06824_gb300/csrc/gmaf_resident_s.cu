@@ -755,8 +755,10 @@ __device__ __forceinline__ unsigned res_iterate_s(const ResParams<T> &q, ResShar
     {
         const double back = kMixed ? sh.back : *q.scale;
         const bool from0 = !kMixed && q.zero_init && q.mode != kResRestart;
+        // (a restart that may be left out, and did not get there: p stays what it was)
+        const bool leave = !kMixed && sh.done == 2 && ((q.optional >> (q.groups == 1 ? 0 : blockIdx.x / q.bpc)) & 1ull);
 #pragma unroll 1
-        for (int rr = 0; rr < nr; ++rr) {
+        for (int rr = 0; rr < (leave ? 0 : nr); ++rr) {
             T x[VEC], s[VEC];
             V::ldrw(pX + rr * stX, x);
             if constexpr (kScaled) V::ldrw(q.s + (w.coff + (unsigned)(rr * nth)), s);

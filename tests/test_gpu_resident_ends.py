@@ -199,3 +199,30 @@ def test_budgets_that_were_enough_still_are(g, monkeypatch, small, large, forced
                 assert st == 0, (order, k, g.status_string(st))
                 assert g.gmaf_workspace_bytes(c.handle) <= held
                 assert rel_l2(ps[k], refs[k]) <= 1e-3
+
+
+# grids and tolerances at which a scaled run ends between 1.25 and 10 times its tolerance
+@pytest.mark.parametrize("nth,nz,K,eps,criterion", [
+    (512, 250, 9, 3e-14, 0), (1000, 250, 4, 1e-13, 0), (1000, 250, 4, 4e-14, 0), (1024, 250, 9, 5e-14, 0),
+    (1000, 250, 4, 1e-13, 1), (1000, 250, 4, 5e-14, 1),
+])
+def test_a_restart_that_is_cut_off_takes_nothing_back(g, nth, nz, K, eps, criterion):
+    """A first run that ends within ten times the tolerance is the solution, whether or not there
+    are iterations left for the restart that would bring it closer."""
+    arrs = system(nth, nz, K, nth)
+    kw = dict(eps=eps, criterion=criterion, allow=(g.GMAF_OK, g.GMAF_NOT_CONVERGED))
+    end = solve(g, nth, nz, K, arrs, **kw)
+    assert end[0] == 0 and end[3]["restarts"] >= 1
+    # the first run's count: the smallest budget that is enough
+    lo, hi = 1, end[1]
+    while lo < hi:
+        mid = (lo + hi) // 2
+        lo, hi = (lo, mid) if solve(g, nth, nz, K, arrs, max_iter=mid, **kw)[0] == 0 else (mid + 1, hi)
+    first = solve(g, nth, nz, K, arrs, max_iter=lo, **kw)
+    assert first[0] == 0 and first[2] <= 10.0 * eps
+    for more in (1, 2, 5, 20):
+        st, it, rel, info, p = solve(g, nth, nz, K, arrs, max_iter=lo + more, **kw)
+        assert st == 0 and rel <= first[2], (more, info)
+        assert criterion == 1 or rel < first[2] or torch.equal(p, first[4])
+    for more in range(1, min(40, lo)):
+        assert solve(g, nth, nz, K, arrs, max_iter=lo - more, **kw)[0] == g.GMAF_NOT_CONVERGED

@@ -69,3 +69,31 @@ def test_a_wait_that_runs_out_gives_way_to_the_phase_kernels(g, monkeypatch, nth
     assert st == stq == str_ == 0 and itq == it and abs(itr - it) <= 2 and relq <= 1e-7
     assert float(torch.linalg.norm(p - q) / torch.linalg.norm(p)) <= 1e-10
     assert not torch.equal(q, r) and float(torch.linalg.norm(p - r) / torch.linalg.norm(p)) <= 1e-6
+
+
+@pytest.mark.parametrize("eps", [1e-13, 4e-14])
+def test_a_restart_that_is_cut_off_takes_nothing_back(g, eps):
+    """A first run that ends within ten times the tolerance is the solution, whether or not there
+    are iterations left for the restart that would bring it closer."""
+    nth, nz, K = 1000, 250, 4
+    arrs = system(nth, nz, K, nth)
+    p = torch.zeros(K * nth * nz, dtype=torch.float64, device="cuda")
+
+    def run(max_iter):
+        return g.gmaf_solve_joint_noalloc(nth, nz, K, *arrs, p, g.solver_opts(eps=eps, max_iter=max_iter),
+                                          allow=(g.GMAF_OK, g.GMAF_NOT_CONVERGED))
+
+    st, hi, _ = run(100000)
+    assert st == 0
+    lo, most = 1, hi
+    while lo < hi:
+        mid = (lo + hi) // 2
+        lo, hi = (lo, mid) if run(mid)[0] == 0 else (mid + 1, hi)
+    st, it, first = run(lo)
+    assert st == 0 and it == lo < most and first <= 10.0 * eps
+    q = p.clone()
+    for more in (1, 2, 5, 20):
+        st, it, rel = run(lo + more)
+        assert st == 0 and (rel < first or torch.equal(p, q))
+    for more in range(1, 40):
+        assert run(lo - more)[0] == g.GMAF_NOT_CONVERGED
