@@ -52,9 +52,33 @@ static __global__ void __launch_bounds__(kThreads) k_dbnd32(const float *__restr
     }
 }
 
-int launch_dbnd32(const float *D32, const float *aE32, const float *aN32, float *dbnd, int nth,
-                  int nz, int nslots, int num_sms, cudaStream_t s)
+// Whether the diagonal is the sum of the couplings on the rows between, as the assembly forms it:
+// both are rounded to FP32, which leaves 2^-23 of it between them.  A caller's matrix may have a term
+// of its own there, which a rebuilt diagonal would lose.
+static __global__ void __launch_bounds__(kThreads) k_own_diag(const float *__restrict__ D32,
+                                                              const float *__restrict__ aE32,
+                                                              const float *__restrict__ aN32, int nth, int nz,
+                                                              long long m, Scalars *sc)
 {
+    bool own = false;
+    for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; q < m;
+         q += (long long)gridDim.x * blockDim.x) {
+        const long long row = q / nth;
+        const int i = (int)(q - row * nth), j = (int)(row % nz);
+        if (j == 0 || j == nz - 1) continue;
+        const double d = D32[q];
+        const double sum = (double)aE32[q] + (double)aE32[i == 0 ? q + nth - 1 : q - 1] + (double)aN32[q] +
+                           (double)aN32[q - nth];
+        own = own || !(fabs(d - sum) <= 0x1p-21 * fabs(d));
+    }
+    if (own) sc->own_diag = 1;
+}
+
+int launch_dbnd32(const float *D32, const float *aE32, const float *aN32, float *dbnd, int nth,
+                  int nz, int nslots, int num_sms, Scalars *sc, cudaStream_t s)
+{
+    const long long m = (long long)nslots * nth * nz;
+    k_own_diag<<<stream_grid(m, num_sms), kThreads, 0, s>>>(D32, aE32, aN32, nth, nz, m, sc);
     const long long total = (long long)nslots * 2 * nth;
     k_dbnd32<<<stream_grid(total, num_sms), kThreads, 0, s>>>(D32, aE32, aN32, dbnd, nth, nz, nslots);
     return cuda_status(cudaGetLastError());

@@ -20,8 +20,9 @@ DrecKernel drec_phase_a();
 
 // The Dirichlet term of the first and last rows that the rebuilt diagonal needs:
 // dbnd[slot][0 or 1][i] = D32 - (((aE + aW) + aN) + aS) in FP32 at rows 0 and
-// n_z - 1 (the sum in the order the phase kernel forms it).
+// n_z - 1 (the sum in the order the phase kernel forms it).  Sets sc->own_diag if the diagonal of
+// another row is not that sum: then it has to be read.
 int launch_dbnd32(const float *D32, const float *aE32, const float *aN32, float *dbnd, int nth,
-                  int nz, int nslots, int num_sms, cudaStream_t s);
+                  int nz, int nslots, int num_sms, Scalars *sc, cudaStream_t s);
 
 }  // namespace gmaf

@@ -50,6 +50,7 @@ struct Scalars {
     double alpha_pp;        // alpha of the older of two pending p updates (pending == 2)
     unsigned int ticket[6];
     unsigned int task_ctr[2];   // next task of phase A / phase B
+    int own_diag;           // mixed precision: some diagonal is not the sum of its couplings (k_own_diag)
 };
 
 enum Ticket { kTicketA = 0, kTicketB = 1, kTicketInit = 2, kTicketResid = 3, kTicketMisc = 4 };
@@ -131,7 +132,7 @@ struct GraphCache {
 
 // Autotuner decision for one solve shape.
 struct TuneEntry {
-    int tsize, nth, nz, K, precond, vec_ok;
+    int tsize, nth, nz, K, precond, vec_ok;     // vec_ok: + 2 with the rebuilt diagonal
     int choice;
 };
 constexpr int kTuneEntries = 32;

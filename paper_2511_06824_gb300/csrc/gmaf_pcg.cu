@@ -496,7 +496,7 @@ static int setup_run(gmaf_ctx *ctx, PcgRun<T> &run, PcgDesc<T> *desc_slot)
     key.nz = h.nz;
     key.K = h.K;
     key.precond = h.precond;
-    key.vec_ok = vo ? 1 : 0;
+    key.vec_ok = (vo ? 1 : 0) + (run.drec_ready ? 2 : 0);    // (choice counts among these candidates)
     int found = -1;
     for (int q = 0; q < ctx->ntune; ++q) {
         const TuneEntry &e = ctx->tune[q];
@@ -1327,14 +1327,18 @@ int solve_joint_device(gmaf_ctx *ctx, int nth, int nz, int K, int nslots, const 
     ResRun<float> rr;
     res_setup<float>(ctx, rr, nth, nz, K, nth % 4 == 0, m, nslots, false,
                      (size_t)gs * (kThreads / 32) * sizeof(double));
+    if (rr.on && rr.pl.tm == 3) {
+        // that form rebuilds the diagonal, where the matrix lets it (one read of a flag: 20 us, before
+        // solves of tens of milliseconds)
+        GMAF_TRY(launch_dbnd32((const float *)ctx->buf[B_D32], (const float *)ctx->buf[B_AE32],
+                               (const float *)ctx->buf[B_AN32], (float *)ctx->buf[B_DBND32], nth, nz,
+                               nslots, ctx->num_sms, dsc_outer, s));
+        GMAF_TRY(read_scalars(ctx, dsc_outer, ho));
+        rr.on = !ho->own_diag;
+        rr.q.dbnd = (const float *)ctx->buf[B_DBND32];
+    }
     if (rr.on) {
         ResParams<float> &q = rr.q;
-        if (rr.pl.tm == 3) {
-            GMAF_TRY(launch_dbnd32((const float *)ctx->buf[B_D32], (const float *)ctx->buf[B_AE32],
-                                   (const float *)ctx->buf[B_AN32], (float *)ctx->buf[B_DBND32], nth, nz,
-                                   nslots, ctx->num_sms, s));
-            q.dbnd = (const float *)ctx->buf[B_DBND32];
-        }
         q.precond = kernel_precond(opts);
         q.max_iter = opts->max_iter;
         q.guard_limit = ctx->loop_guard;
@@ -1409,9 +1413,8 @@ int solve_joint_device(gmaf_ctx *ctx, int nth, int nz, int K, int nslots, const 
         // the boundary term of the diagonal for the phase A variant that rebuilds it
         GMAF_TRY(ensure(ctx, B_DBND32, (size_t)nslots * 2 * nth * sizeof(float)));
         GMAF_TRY(launch_dbnd32(h.D, h.aE, h.aN, (float *)ctx->buf[B_DBND32], nth, nz, nslots,
-                               ctx->num_sms, s));
+                               ctx->num_sms, dsc_outer, s));
         h.dbnd = (const float *)ctx->buf[B_DBND32];
-        run.drec_ready = true;
     }
     // The first outer residual and the inner right-hand side are formed before the
     // kernel set is chosen, so that the autotuner times iterations on real data.
@@ -1463,6 +1466,7 @@ int solve_joint_device(gmaf_ctx *ctx, int nth, int nz, int K, int nslots, const 
                                            N, dsc_outer);
         GMAF_CUDA(cudaGetLastError());
         if (!tuned) {
+            run.drec_ready = h.dbnd && !ho->own_diag;
             GMAF_TRY(setup_run<float>(ctx, run, (PcgDesc<float> *)(dbase + 1024)));
             rd.partials = h.partials;
             GMAF_CUDA(cudaMemcpyAsync(d_rdesc, &rd, sizeof(ResidDesc), cudaMemcpyHostToDevice, s));

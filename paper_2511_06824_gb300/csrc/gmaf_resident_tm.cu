@@ -5,7 +5,7 @@
 // u stays in shared memory, and the
 // coefficients and x are streamed from L2, one group of rows ahead of the one worked on.
 // The diagonal is rebuilt from the couplings, as in the phase A of gmaf_drec.cu, to save
-// its traffic.
+// its traffic; a matrix whose diagonal is another one is left to the phase kernels.
 //
 // On 9 conditions of 1024 x 512 cells an iteration takes 37 to 39 us (A 16.8, B 21.2: the
 // coefficients' and x's 175 MB from L2 at 4.5 TB/s, and two exchanges of 1.5 us), the

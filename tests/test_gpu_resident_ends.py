@@ -226,3 +226,33 @@ def test_a_restart_that_is_cut_off_takes_nothing_back(g, nth, nz, K, eps, criter
         assert criterion == 1 or rel < first[2] or torch.equal(p, first[4])
     for more in range(1, min(40, lo)):
         assert solve(g, nth, nz, K, arrs, max_iter=lo - more, **kw)[0] == g.GMAF_NOT_CONVERGED
+
+
+# (n_theta, n_z, resident for a diagonal that is the couplings' sum)
+@pytest.mark.parametrize("nth,nz,fits", [(700, 300, True), (1028, 290, False)])
+@pytest.mark.parametrize("where", ["everywhere", "one cell"])
+def test_a_diagonal_with_a_term_of_its_own(g, monkeypatch, nth, nz, fits, where):
+    """Forms that rebuild the diagonal from the couplings are for systems whose diagonal is their
+    sum: with anything added to it (here 2 %) the diagonal is read, and the solve converges to what
+    FP64 gives."""
+    K = 9
+    D, aE, aN, S = system(nth, nz, K, nth)
+    monkeypatch.setenv("GMAF_VARIANT", "10604322")
+    plain = solve(g, nth, nz, K, [D, aE, aN, S], precision=1)[3]
+    assert plain["kernel_variant"] == 10604322
+    monkeypatch.delenv("GMAF_VARIANT")
+    assert resident(solve(g, nth, nz, K, [D, aE, aN, S], precision=1)[3]) == fits
+    more = D.clone()
+    if where == "everywhere":
+        more *= 1.02
+    else:
+        more[(K - 1) * nth * nz + (nz // 2) * nth + 7] *= 1.02
+    arrs = [more, aE, aN, S]
+    kw = dict(max_iter=20000, allow=(g.GMAF_OK, g.GMAF_NOT_CONVERGED, g.GMAF_NONFINITE))
+    ref = solve(g, nth, nz, K, arrs, **kw)
+    for variant in (None, "10604322"):
+        if variant:
+            monkeypatch.setenv("GMAF_VARIANT", variant)
+        st, it, rel, info, p = solve(g, nth, nz, K, arrs, precision=1, **kw)
+        assert st == 0 and info["kernel_variant"] not in (10604322, 50004160)
+        assert rel_l2(p, ref[4]) <= 1e-6
