@@ -1622,7 +1622,7 @@ __device__ __noinline__ void res_setup(const ResParams<T> &q)
     ResRows<T, VEC, RR, CS>(q, res_shared<T>()).setup();
 }
 // The norm of r64 as k_resid64 adds it up: a run of the refinement then works on the numbers that
-// it would have with the phase kernels, bit for bit (the last bit of the norm is a bit of p, whose
+// it would have with the phase kernels, bit for bit on every grid tested (the last bit of the norm is a bit of p, whose
 // rounding is all that r64 is made of towards the end; with the norm as the blocks' exact sum a
 // Picard step's Jacobian on 512 x 256 cells moved by 1e-10 to 1e-9, so it does by 1e-12).  First the sums of that kernel's warps,
 // then, in every block, what its blocks and its last block add: 16 us a refinement on 256 x 128 x 9

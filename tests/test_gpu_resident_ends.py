@@ -256,3 +256,19 @@ def test_a_diagonal_with_a_term_of_its_own(g, monkeypatch, nth, nz, fits, where)
         st, it, rel, info, p = solve(g, nth, nz, K, arrs, precision=1, **kw)
         assert st == 0 and info["kernel_variant"] not in (10604322, 50004160)
         assert rel_l2(p, ref[4]) <= 1e-6
+
+
+@pytest.mark.parametrize("nth,nz,K", [(64, 32, 1), (96, 48, 9), (132, 45, 9), (256, 128, 9), (512, 256, 9), (640, 200, 9)])
+@pytest.mark.parametrize("iters", [1, 3, 30, 100000])
+def test_mixed_runs_are_those_of_the_phase_kernels(g, monkeypatch, nth, nz, K, iters):
+    """Resident runs of up to 8 rows and the phase kernels of four columns a lane take the same
+    FP32 operations in the same order, and the norm of the FP64 residual is added up in that
+    kernel's order.  The grid's other sums are added in another order, but agree once they are
+    rounded to FP32: the same solution, to the last bit."""
+    arrs = system(nth, nz, K, nth)
+    kw = dict(precision=1, eps=1e-13, max_iter=iters, allow=(g.GMAF_OK, g.GMAF_NOT_CONVERGED))
+    a = solve(g, nth, nz, K, arrs, **kw)
+    monkeypatch.setenv("GMAF_VARIANT", "604322")
+    b = solve(g, nth, nz, K, arrs, **kw)
+    assert resident(a[3]) and b[3]["kernel_variant"] == 604322
+    assert a[0] == b[0] and a[1] == b[1] and torch.equal(a[4], b[4])
