@@ -890,30 +890,18 @@ struct ResRows {
     using V = Vec<T, VEC>;
     static constexpr int S = kResThreads * VEC;     // private fields: [row][thread][VEC]
     static constexpr int NS = kResSegs;
-    static constexpr bool kMixed = sizeof(T) == 4;  // FP32 runs inside FP64 refinement
     static constexpr int FE = RR * S, FN = 2 * RR * S, FI = 3 * RR * S, FD = 4 * RR * S;
 
     const ResParams<T> &q;
     ResShared<T> &sh;
-    int nth, nz, TC, all, tid, lane, wid;
+    int nth, nz, TC, tid, lane, wid;
     int j0, run, cg, c, lr0, nr;                    // the block's first row; first local row and rows of the run
     bool act, top, hasS, hasN;                      // rows at all; the block's last rows; a block below, above
     bool segw, sege, atw, ate, last;                // edges of a segment, of the row; the run ends at row nz - 1
     size_t off, coff;                               // first cell in the fields, in the coefficient slots
-    // shared memory: private fields (u, coefficients, r), then rows and edges
-    T *P;                                           // u: P[rr * S]
-    T *HU, *HR, *HI;                                // [2][nth] u, r, omega/D on the halo rows
-    T *HE;                                          // [nth] aE on the north halo row
-    T *YR, *WR;                                     // [nrr][nth] y south of each run, [nrr - 1][nth] w north
-    // edges of a row's segments of 32 threads, [rows + 1][NS]: last y, last aE, first w (own,
-    // of the west and of the east segment); [rows + 1][2] y of column 0 and w of column nth - 1
-    T *EY, *EYl, *EWr, *EC;
+    // shared memory that setup() fills, laid out as res_iterate describes it
+    T *P, *HU, *HR, *HI, *HE, *YR, *EY;
     int er;
-    const T *pS, *pN, *pW, *pE;                     // u beyond the run's rows and the warp's columns
-    T *pX;
-    int stX;
-    // rows of a block's halo area: 0, 1 = first and last row of v; 2, 3 = of z
-    unsigned long long *halo;
 
     __device__ __forceinline__ ResRows(const ResParams<T> &q_, ResShared<T> &sh_) : q(q_), sh(sh_)
     {
@@ -921,7 +909,6 @@ struct ResRows {
         nth = q.nth;
         nz = q.nz;
         TC = q.threads;
-        all = TC + 32;
         // (volatile: formed anew where it is used, not kept in registers across refinements)
         asm volatile("mov.u32 %0, %%tid.x;\n" : "=r"(tid));
         lane = tid & 31;
@@ -946,44 +933,14 @@ struct ResRows {
         last = top && j1 == nz;
         off = (size_t)cond * (size_t)q.n + (size_t)(j0 + lr0) * nth + c;
         coff = (size_t)q.cslot[cond] * (size_t)q.n + (size_t)(j0 + lr0) * nth + c;
-        T *const sm = reinterpret_cast<T *>(g_res_smem);
-        P = sm + tid * VEC;
+        P = reinterpret_cast<T *>(g_res_smem) + tid * VEC;
         HU = reinterpret_cast<T *>(g_res_smem + q.o_rows);
         HR = HU + 2 * nth;
         HI = HR + 2 * nth;
         HE = HI + 2 * nth;
         YR = HE + nth;
-        WR = YR + q.nrr * nth;
-        T *const edge = reinterpret_cast<T *>(g_res_smem + q.o_edge);
         er = (q.rows + 1) * NS;
-        EY = edge + lr0 * NS + (cg >> 5);
-        EYl = edge + lr0 * NS + (atw ? (q.ncg - 1) >> 5 : (cg >> 5) - 1);
-        EWr = edge + 2 * er + lr0 * NS + (ate ? 0 : (cg >> 5) + 1);
-        EC = edge + 3 * er + 2 * lr0;
-        pS = run == 0 ? HU + c : P - q.P * VEC + (RR - 1) * S;
-        pN = top ? HU + nth + c : P + q.P * VEC;
-        pW = sm + (run * q.P + (atw ? q.ncg - 1 : cg - 1)) * VEC + VEC - 1;
-        pE = sm + (run * q.P + (ate ? 0 : cg + 1)) * VEC;
-        pX = q.o_x >= 0 ? reinterpret_cast<T *>(g_res_smem + q.o_x) + tid * VEC : q.p + off;
-        stX = q.o_x >= 0 ? S : nth;
-        halo = q.halo + (size_t)blockIdx.x * 4 * q.halo_row + c * ((int)sizeof(T) / 4);
-    }
-
-    __device__ __forceinline__ void get_E(int rr, T (&x)[VEC]) const
-    {
-        V::ldrw(CS ? P + FE + rr * S : q.aE + coff + (size_t)rr * nth, x);
-    }
-    __device__ __forceinline__ void get_N(int rr, T (&x)[VEC]) const
-    {
-        V::ldrw(CS ? P + FN + rr * S : q.aN + coff + (size_t)rr * nth, x);
-    }
-    __device__ __forceinline__ void get_I(int rr, T (&x)[VEC]) const
-    {
-        V::ldrw(CS ? P + FI + rr * S : q.invD + coff + (size_t)rr * nth, x);
-    }
-    __device__ __forceinline__ void get_D(int rr, T (&x)[VEC]) const
-    {
-        V::ldrw(CS ? P + FD + rr * S : q.D + coff + (size_t)rr * nth, x);
+        EY = reinterpret_cast<T *>(g_res_smem + q.o_edge) + lr0 * NS + (cg >> 5);
     }
 
     // The coefficients, and zeros for u and where no block lies beyond.
