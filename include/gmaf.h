@@ -129,7 +129,9 @@ typedef struct {
                                   problem shape by the autotuner on the first solve of
                                   that shape.  50000000 + 1000 VEC + 10 RR: the resident
                                   solve (one launch, RR rows a thread), taken wherever
-                                  the system fits on the SMs */
+                                  the system fits on the SMs; where that run gives way
+                                  (other work keeps its blocks from running together, sums
+                                  out of its range, no room in the budget) a phase kernel */
     int32_t tasks;             /* strip x row-block x condition tasks per PCG phase
                                   (resident solve: blocks)                              */
     int32_t iterations_sum;    /* PCG iterations summed over the conditions: n_cond x

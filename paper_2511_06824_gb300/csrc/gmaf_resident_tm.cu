@@ -7,9 +7,10 @@
 // The diagonal is rebuilt from the couplings, as in the phase A of gmaf_drec.cu, to save
 // its traffic; a matrix whose diagonal is another one is left to the phase kernels.
 //
-// On 9 conditions of 1024 x 512 cells an iteration takes 37 to 39 us (A 16.8, B 21.2: the
-// coefficients' and x's 175 MB from L2 at 4.5 TB/s, and two exchanges of 1.5 us), the
-// phase kernels take 68.3; on 9 of 700 x 300 it is 33.3 against 56.7.
+// On 9 conditions of 1024 x 512 cells an iteration takes 37 to 39 us (A 16.8, B 21.2), with two
+// exchanges of 1.5 us; the phase kernels take 68.3.  The coefficients and x are 175 MB of it from
+// L2, where 321 MB are counted: the rest is spills (96 registers a thread) and polling.  On 9 of
+// 700 x 300 it is 33.3 us against 56.7.
 #include "gmaf_resident.cuh"
 #include "gmaf_tmem.cuh"
 
