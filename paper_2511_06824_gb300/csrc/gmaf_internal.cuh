@@ -44,13 +44,12 @@ struct Scalars {
     double rnorm;           // mixed precision: norm of the FP64 outer residual
     int iter, first, done, converged, status, guard, zero_rhs;
     int pending;            // alpha u terms not yet added to p (0, 1 or 2)
-    int max_iter;
+    int own_diag;           // mixed precision: some diagonal is not the sum of its couplings (k_own_diag)
     int cont;               // mixed precision: the next initial pass continues the recurrence
     double cscale;          //   (reliable update) with the old direction rescaled by cscale
     double alpha_pp;        // alpha of the older of two pending p updates (pending == 2)
     unsigned int ticket[6];
     unsigned int task_ctr[2];   // next task of phase A / phase B
-    int own_diag;           // mixed precision: some diagonal is not the sum of its couplings (k_own_diag)
 };
 
 enum Ticket { kTicketA = 0, kTicketB = 1, kTicketInit = 2, kTicketResid = 3, kTicketMisc = 4 };
