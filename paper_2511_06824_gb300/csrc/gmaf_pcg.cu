@@ -1328,8 +1328,8 @@ int solve_joint_device(gmaf_ctx *ctx, int nth, int nz, int K, int nslots, const 
     res_setup<float>(ctx, rr, nth, nz, K, nth % 4 == 0, m, nslots, false,
                      (size_t)gs * (kThreads / 32) * sizeof(double));
     if (rr.on && rr.pl.tm == 3) {
-        // that form rebuilds the diagonal, where the matrix lets it (one read of a flag: 20 us, before
-        // solves of tens of milliseconds)
+        // that form rebuilds the diagonal, where the matrix lets it (a pass and a read of its flag
+        // before solves of tens of milliseconds)
         GMAF_TRY(launch_dbnd32((const float *)ctx->buf[B_D32], (const float *)ctx->buf[B_AE32],
                                (const float *)ctx->buf[B_AN32], (float *)ctx->buf[B_DBND32], nth, nz,
                                nslots, ctx->num_sms, dsc_outer, s));
