@@ -60,7 +60,7 @@ struct ResParams {
     int threads, P, ncg, nrr, rows, nseg;
     int precond, mode, zero_init, max_iter, guard_limit;
     int o_rows, o_edge, o_x, o_q, o_keep, keep;     // keep: rows of a run whose E stays on the SM
-    unsigned polls;                     // limit of a wait
+    unsigned polls;                     // limit of a wait (FP32: for a neighbour's row)
     unsigned epoch;                     // exchanges of this run are epoch + 1, epoch + 2, ...
     unsigned long long mask;            // groups that run
     unsigned long long optional;        // scaled: groups whose p is within the limit already: a restart
